@@ -152,10 +152,11 @@ int aem_loglik_f64(const aem_system *sys, const aem_models_f64 *models, const do
 
 /* Launch-shape autotuner of the FP32 forward kernel (aem_forward_f32,
  * aem_loglik_f32 and every sampler call that evaluates the forward model).
- * Shapes: 0 = 256 threads per CTA with 4 resident CTAs per SM (the default),
+ * Shapes: 0 = 256 threads per CTA with 4 resident CTAs per SM,
  * 1 = 128 x 8, 2 = 512 x 2, 3 = 256 x 3, 4 = 128 x 6 (the register budget per
  * thread follows from the pair), each with a fixed grid-stride order of
- * models; 5..9 = the same five with dynamic scheduling (a CTA claims its
+ * models (a recorded 0, the default, stands for "none chosen": launches take
+ * shape 2 for at most two models per SM and shape 1 above); 5..9 = the same five with dynamic scheduling (a CTA claims its
  * next model from a counter in stream-ordered scratch when it finishes one).  aem_autotune_forward times every shape that
  * fits on an SM on the caller's sample batch (one untimed launch, then
  * `repeats` launches timed with CUDA events on `stream`; synchronous), and

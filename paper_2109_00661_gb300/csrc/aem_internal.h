@@ -42,6 +42,9 @@ struct aem_system {
     int device = 0;
     // device tables: omega[F], lam[K], hw[K], T[G*F] in both precisions
     float *d_omega_f = nullptr, *d_lam_f = nullptr, *d_hw_f = nullptr, *d_T_f = nullptr;
+    // the FP32 forward kernel's length unit (a power of two, metres) and its
+    // abscissae in it
+    float len = 1.f, *d_lamu_f = nullptr;
     double *d_omega_d = nullptr, *d_lam_d = nullptr, *d_hw_d = nullptr, *d_T_d = nullptr;
     int num_sms = 0;
     // device status word: kernels record AEM_ERR_TIMEOUT here when a bounded

@@ -16,7 +16,8 @@
 //
 // Recursion used (quasi-static TE mode, exp(+i w t)):
 //   u_n = sqrt(lambda^2 + s_n), Re u_n > 0
-//   r   = (s_n - s_{n+1}) / (u_n + u_{n+1})^2       (= (u_n - u_{n+1})/(u_n + u_{n+1}))
+//   r   = (u_n - u_{n+1}) / (u_n + u_{n+1})  (as (s_n - s_{n+1}) / (u_n + u_{n+1})^2 in
+//         the FP64 kernel, from the roots' products in the FP32 one)
 //   R_n = (r + R_{n+1} E) / (1 + r R_{n+1} E),  E = exp(-2 u_{n+1} h_{n+1})
 // carried projectively as R = N / D so the Moebius step needs no division:
 //   N' = r D + N E,  D' = D + r N E.  |D| grows by at most 2x per layer.
@@ -361,56 +362,92 @@ int launch_forward(const aem_system *sys, const Models *models, typename Ops::R 
 // (add/sub/mul/fma .f32x2): one issue slot per operation on both abscissae.
 // The special functions (sqrt, rsqrt, rcp, ex2, sin, cos) stay scalar.
 //
-// The recursion is carried in w = sqrt(2) u, which folds the constants:
-//   r = (s_a - s_b) / (u_a + u_b)^2 = B / (w_a + w_b)^2,  B = 2 (s_a - s_b)
+// The recursion is carried in w = sqrt(2) u.  Principal root of
+// 2 (lambda^2 + s) with x = lambda^2 + Re s, y = Im s > 0 and m = |x + i y|:
+//   t = m + |x|, rr = rsqrt(t); (t rr, y rr) is (Re w, Im w) when x >= 0 and
+//   (Im w, Re w) otherwise.
+// The interface coefficient comes from the two roots and their moduli alone,
+//   r = (u_a - u_b) / (u_a + u_b) = (u_a - u_b) conj(u_a + u_b) / |u_a + u_b|^2
+//     = [(m_a - m_b) + i (Im w_a Re w_b - Re w_a Im w_b)]
+//       / [m_a + m_b + Re w_a Re w_b + Im w_a Im w_b]
+// (|w|^2 = 2 m), nine paired operations and one reciprocal per abscissa where
+// B / (w_a + w_b)^2 with B = 2 (s_a - s_b) takes fourteen and two more
+// shared-memory records per interface.  Only Im R_0 is wanted; the rounding of
+// m_a - m_b enters it multiplied by Im E of the layers above and is attenuated
+// with the layer's own signal, and Im r keeps its relative accuracy, so the
+// spectrum's error is lower than with the differenced s (FP32 emulation on 150
+// random and 100 alternating stacks, relative to sum |w_k| |R_0|: largest
+// 6.3e-7 against 1.4e-6, rms 4.0e-8 against 7.5e-8).
 //   E = exp(-2 u h) = exp2(e w.x) (cos(e ln2 w.y) + i sin(e ln2 w.y)),
 //   e = -sqrt(2) h log2(e).
-// Principal root of 2 (lambda^2 + s) with x = lambda^2 + Re s, y = Im s > 0:
-//   t = sqrt(x^2 + y^2) + |x|, rr = rsqrt(t); (t rr, y rr) is (Re w, Im w) when
-//   x >= 0 and (Im w, Re w) otherwise.
 // The Moebius step (N, D) <- (r D + N E, D + r N E) keeps R_0 = N / D.
+// Lengths are counted in the power of two next to the system's 2 h + a
+// (aem_system::len: lambda, s and h scaled by it exactly), so that |lambda^2 + s|^2
+// and the product of two reciprocals' arguments stay inside the FP32 range
+// whatever the geometry.
 using namespace f32x2;  // paired FP32 helpers and the hardware approximations (f32x2.h)
 
 constexpr double kLn2Pi = 1.83787706640934548356;  // ln(2 pi)
 
-// w for both abscissae; sxx = (Re s, Re s), yyy = (Im s ^2, ...), syy = (Im s, Im s)
-__device__ __forceinline__ C2x2 wroot2(u64 lam2, u64 sxx, u64 yyy, u64 syy) {
-    const u64 x = add2(lam2, sxx);
-    const u64 v = fma2(x, x, yyy);
+struct Root {  // w of one layer for both abscissae, and m = |w|^2 / 2
+    u64 re, im, m;
+};
+
+// rec = ((Re s, Re s), (Im s, Im s)).
+__device__ __forceinline__ Root root2(u64 lam2, ulonglong2 rec) {
+    const u64 x = add2(lam2, rec.x);
+    const u64 v = fma2(x, x, mul2(rec.y, rec.y));
     float v0, v1, x0, x1;
     up2(v, v0, v1);
     up2(x, x0, x1);
-    const float t0 = sqrt_approx(v0) + fabsf(x0), t1 = sqrt_approx(v1) + fabsf(x1);
+    const float m0 = sqrt_approx(v0), m1 = sqrt_approx(v1);
+    const float t0 = m0 + fabsf(x0), t1 = m1 + fabsf(x1);
     const u64 rr = pk2(rsqrt_approx(t0), rsqrt_approx(t1));
-    const u64 p = mul2(pk2(t0, t1), rr), o = mul2(syy, rr);
+    const u64 p = mul2(pk2(t0, t1), rr), o = mul2(rec.y, rr);
+    Root w;
+    w.m = pk2(m0, m1);
     float p0, p1, o0, o1;
     up2(p, p0, p1);
     up2(o, o0, o1);
-    C2x2 w;
     w.re = pk2(x0 >= 0.f ? p0 : o0, x1 >= 0.f ? p1 : o1);
     w.im = pk2(x0 >= 0.f ? o0 : p0, x1 >= 0.f ? o1 : p1);
     return w;
 }
 
-// r = B / (wa + wb)^2 = B (cre - 2 i pp), (wx - i wy) = conj(q) / |q|^2.
-// Bv = ((Bx, Bx), (By, By)), Cv = ((-2 Bx, -2 Bx), (2 By, 2 By)).
-__device__ __forceinline__ C2x2 rcoef2(ulonglong2 Bv, ulonglong2 Cv, C2x2 a, C2x2 b) {
-    const u64 qx = add2(a.re, b.re), qy = add2(a.im, b.im);
-    float q0, q1;
-    up2(fma2(qx, qx, mul2(qy, qy)), q0, q1);
-    const u64 ir = pk2(rcp_approx(q0), rcp_approx(q1));
-    const u64 wx = mul2(qx, ir), wy = mul2(qy, ir);
-    const u64 cre = mul2(sub2(wx, wy), add2(wx, wy));
-    const u64 pp = mul2(wx, wy);
+// 1 / d for both abscissae from one reciprocal: three multiplications in place
+// of the second special-function operation (the layer-step's busiest unit;
+// marginal layer 98.8 -> 96.7 SM-sub-partition cycles per 32 items).
+__device__ __forceinline__ u64 rcp2(u64 d) {
+    float d0, d1;
+    up2(d, d0, d1);
+    const float i = rcp_approx(d0 * d1);
+    return pk2(i * d1, i * d0);
+}
+
+// The interface coefficient between a (above) and b.
+__device__ __forceinline__ C2x2 rcoef2(const Root &a, const Root &b) {
+    const u64 den = fma2(a.im, b.im, fma2(a.re, b.re, add2(a.m, b.m)));
+    const u64 ir = rcp2(den);
     C2x2 r;
-    r.re = fma2(Bv.x, cre, mul2(Cv.y, pp));
-    r.im = fma2(Bv.y, cre, mul2(Cv.x, pp));
+    r.re = mul2(sub2(a.m, b.m), ir);
+    r.im = mul2(sub2(mul2(a.im, b.re), mul2(a.re, b.im)), ir);
+    return r;
+}
+
+// rcoef2 for the air above the top layer: w_air = sqrt(2) lambda is real,
+// m_air = lambda^2; nwair = -w_air.
+__device__ __forceinline__ C2x2 rcoef2_air(u64 lam2, u64 nwair, const Root &b) {
+    const u64 den = sub2(add2(lam2, b.m), mul2(nwair, b.re));
+    const u64 ir = rcp2(den);
+    C2x2 r;
+    r.re = mul2(sub2(lam2, b.m), ir);
+    r.im = mul2(mul2(nwair, b.im), ir);
     return r;
 }
 
 // he = ((e, e), (e ln2, e ln2)) of the layer below the interface.
 // E = exp(-2 u h) of both abscissae as (Re, Im) pairs.
-__device__ __forceinline__ void expm2(C2x2 wb, ulonglong2 he, u64 &Ex, u64 &Ey) {
+__device__ __forceinline__ void expm2(const Root &wb, ulonglong2 he, u64 &Ex, u64 &Ey) {
     float a0, a1;
     up2(mul2(he.x, wb.re), a0, a1);
     const u64 e = pk2(ex2_approx(a0), ex2_approx(a1));
@@ -430,7 +467,7 @@ __device__ __forceinline__ void expm2(C2x2 wb, ulonglong2 he, u64 &Ex, u64 &Ey) 
 #endif
 }
 
-__device__ __forceinline__ void mobius2(C2x2 &N, C2x2 &D, C2x2 r, C2x2 wb, ulonglong2 he) {
+__device__ __forceinline__ void mobius2(C2x2 &N, C2x2 &D, C2x2 r, const Root &wb, ulonglong2 he) {
     u64 Ex, Ey;
     expm2(wb, he, Ex, Ey);
     const u64 Px = sub2(mul2(N.re, Ex), mul2(N.im, Ey));
@@ -445,23 +482,8 @@ __device__ __forceinline__ void mobius2(C2x2 &N, C2x2 &D, C2x2 r, C2x2 wb, ulong
     D.im = Dy;
 }
 
-// rcoef2 for the air above the top layer: w_air = sqrt(2) lambda is real.
-__device__ __forceinline__ C2x2 rcoef2_air(ulonglong2 Bv, ulonglong2 Cv, u64 wair, C2x2 b) {
-    const u64 qx = add2(wair, b.re), qy = b.im;
-    float q0, q1;
-    up2(fma2(qx, qx, mul2(qy, qy)), q0, q1);
-    const u64 ir = pk2(rcp_approx(q0), rcp_approx(q1));
-    const u64 wx = mul2(qx, ir), wy = mul2(qy, ir);
-    const u64 cre = mul2(sub2(wx, wy), add2(wx, wy));
-    const u64 pp = mul2(wx, wy);
-    C2x2 r;
-    r.re = fma2(Bv.x, cre, mul2(Cv.y, pp));
-    r.im = fma2(Bv.y, cre, mul2(Cv.x, pp));
-    return r;
-}
-
 // The first Moebius step, where D = 1: (N, D) <- (r + N E, 1 + r N E).
-__device__ __forceinline__ void mobius2_d1(C2x2 &N, C2x2 &D, C2x2 r, C2x2 wb, ulonglong2 he) {
+__device__ __forceinline__ void mobius2_d1(C2x2 &N, C2x2 &D, C2x2 r, const Root &wb, ulonglong2 he) {
     u64 Ex, Ey;
     expm2(wb, he, Ex, Ey);
     const u64 Px = sub2(mul2(N.re, Ex), mul2(N.im, Ey));
@@ -472,61 +494,71 @@ __device__ __forceinline__ void mobius2_d1(C2x2 &N, C2x2 &D, C2x2 r, C2x2 wb, ul
     D.im = fma2(r.re, Py, mul2(r.im, Px));
 }
 
-// Per frequency, a block of LS + 1 records of three ulonglong2: record 0 the
-// air interface (B, C in entries 1 and 2), record n + 1 layer n ((Re s,
-// (Im s)^2) in entry 0) and the interface below it (B, C in entries 1 and 2).
-constexpr int kRecWords = 3;
+__device__ __forceinline__ ulonglong2 lds16(unsigned a) {
+    ulonglong2 v;
+    asm volatile("ld.shared.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "r"(a));
+    return v;
+}
 
-// Im R_0 for the two abscissae of one work item.  LT > 0: the layer count is
-// the compile-time LT and the layer loop is unrolled completely (the record
-// offsets become immediates); LT = 0: the runtime L.  R is the frequency's
-// record block, Y its (Im s) pairs.
+// Im R_0 for the two abscissae of one work item.  rec, he: shared-memory
+// addresses of the frequency's layer records and of the layers' exponents.
+// LT > 0: the layer count is the compile-time LT and the layer loop is
+// unrolled completely; LT = 0: the runtime L, two layers per iteration.
 template <int LT>
-__device__ __forceinline__ void im_r0_pair(u64 lam2, u64 wair, const ulonglong2 *__restrict__ R,
-                                           const u64 *__restrict__ Y, const ulonglong2 *__restrict__ HE, int L_rt,
-                                           float &out0, float &out1) {
+__device__ __forceinline__ void im_r0_pair(u64 lam2, u64 nwair, unsigned rec, unsigned he, int L_rt, float &out0,
+                                           float &out1) {
     const int L = LT > 0 ? LT : L_rt;
-    ulonglong2 a = R[kRecWords * L];
-    C2x2 wb = wroot2(lam2, a.x, a.y, Y[L - 1]);
+    unsigned rp = rec + 16u * (unsigned)(L - 1);
+    Root wb = root2(lam2, lds16(rp));
     if (L == 1) {
-        up2(rcoef2_air(R[1], R[2], wair, wb).im, out0, out1);
+        up2(rcoef2_air(lam2, nwair, wb).im, out0, out1);
         return;
     }
-    a = R[kRecWords * (L - 1)];
-    C2x2 wn = wroot2(lam2, a.x, a.y, Y[L - 2]);
-    C2x2 N = rcoef2(R[kRecWords * (L - 1) + 1], R[kRecWords * (L - 1) + 2], wn, wb);
-    C2x2 D;  // 1 until the first Moebius step
-    ulonglong2 he = HE[L - 2];
-    wb = wn;
-    auto step = [&](int n) {
-        a = R[kRecWords * (n + 1)];
-        wn = wroot2(lam2, a.x, a.y, Y[n]);
-        const C2x2 r = rcoef2(R[kRecWords * (n + 1) + 1], R[kRecWords * (n + 1) + 2], wn, wb);
-        if (n == L - 3)
-            mobius2_d1(N, D, r, wb, he);
-        else
-            mobius2(N, D, r, wb, he);
-        he = HE[n];
-        wb = wn;
-    };
-    if constexpr (LT > 0) {
-        // the empty asm keeps each step's shared-memory loads in its own step:
-        // hoisting the later layers' records ahead raised the register
-        // pressure of the unrolled recursion into spills (128 bytes at 64
-        // registers) and measured 4 % slower
+    rp -= 16;
+    Root wa = root2(lam2, lds16(rp));
+    C2x2 N = rcoef2(wa, wb), D;
+    if (L == 2) {
+        mobius2_d1(N, D, rcoef2_air(lam2, nwair, wa), wa, lds16(he));
+    } else if constexpr (LT > 2) {
 #pragma unroll
         for (int n = LT - 3; n >= 0; --n) {
-            step(n);
+            wb = root2(lam2, lds16(rec + 16 * n));
+            if (n == LT - 3)
+                mobius2_d1(N, D, rcoef2(wb, wa), wa, lds16(he + 16 * (n + 1)));
+            else
+                mobius2(N, D, rcoef2(wb, wa), wa, lds16(he + 16 * (n + 1)));
+            wa = wb;
+            // each step's shared-memory loads stay in their step (hoisting
+            // them ahead raises the register pressure into spills)
             asm volatile("" ::: "memory");
         }
+        mobius2(N, D, rcoef2_air(lam2, nwair, wa), wa, lds16(he));
     } else {
-#pragma unroll 2
-        for (int n = L - 3; n >= 0; --n) step(n);
+        unsigned hp = he + 16u * (unsigned)(L - 2);
+        rp -= 16;
+        wb = root2(lam2, lds16(rp));
+        mobius2_d1(N, D, rcoef2(wb, wa), wa, lds16(hp));
+        // wb is layer L - 3; the layers above it come in pairs, so that the
+        // roots swap roles without a copy
+        if (L & 1) {
+            wa = wb;
+        } else {
+            rp -= 16;
+            hp -= 16;
+            wa = root2(lam2, lds16(rp));
+            mobius2(N, D, rcoef2(wa, wb), wb, lds16(hp));
+        }
+#pragma unroll 1
+        while (rp != rec) {
+            wb = root2(lam2, lds16(rp - 16));
+            mobius2(N, D, rcoef2(wb, wa), wa, lds16(hp - 16));
+            wa = root2(lam2, lds16(rp - 32));
+            mobius2(N, D, rcoef2(wa, wb), wb, lds16(hp - 32));
+            rp -= 32;
+            hp -= 32;
+        }
+        mobius2(N, D, rcoef2_air(lam2, nwair, wa), wa, lds16(he));
     }
-    if (L == 2)
-        mobius2_d1(N, D, rcoef2_air(R[1], R[2], wair, wb), wb, he);
-    else
-        mobius2(N, D, rcoef2_air(R[1], R[2], wair, wb), wb, he);
     float n0, n1, d0, d1;
     up2(sub2(mul2(N.im, D.re), mul2(N.re, D.im)), n0, n1);
     up2(fma2(D.re, D.re, mul2(D.im, D.im)), d0, d1);
@@ -538,33 +570,30 @@ __device__ __forceinline__ void im_r0_pair(u64 lam2, u64 wair, const ulonglong2 
 // launch shape, so that the Hankel sums come out identical whatever the
 // shape, the scheduling or the row stride (lmax) of the models.
 constexpr int kValsWords = 6144;
-static_assert(kValsWords % 512 == 0, "rounds must end on a multiple of every launch shape's thread count");
+static_assert(kValsWords % 32 == 0, "rounds must end on a whole group");
 
-// Words (floats) of the forward kernel's value region: the value buffer, or
-// the prologue's stmp[F*LS] (float2) that shares it, whichever is larger.
-__host__ __device__ inline size_t value_words(int F, int LS) {
-    const size_t st = (size_t)2 * F * LS;
-    return st > (size_t)kValsWords ? st : (size_t)kValsWords;
+// Words of the buffer one system uses: all of it, or its single round's items.
+__host__ __device__ inline int vals_words(int F, int K2) {
+    const int n = (F * K2 + 31) & ~31;
+    return n < kValsWords ? n : kValsWords;
 }
 
-// Shared memory (dynamic), in order: REC[F*(LS+1)*kRecWords] (the record
-// blocks of im_r0_pair), KR[2*K2] (ulonglong2: per abscissa pair the
-// (lambda^2, sqrt(2) lambda) pairs, then the two Hankel weights), Y[F*LS]
-// (u64), the value region (value_words floats), imh[F], T[G*F], TH[F*LS]
-// (float: the depth cutoff's thresholds).  The
-// items (frequency major, F*K2 of them) are taken in rounds of kValsWords:
-// every item stores
-// its weighted pair value at its own index in the buffer; after the round
-// each frequency the round touched is summed by four consecutive lanes (lane
-// s adds the values at s + 4 i into four accumulators by i mod 4, then a
-// tree over the sixteen partial sums, two levels by shuffles) and added to
-// imh[f], rounds in order.  The order of every sum is fixed by the
-// item indices alone.  (The throughput system's 60 x 100 items take one
-// round.)  Before the item loop the value region holds the prologue's
-// stmp[F*LS] (float2).
-template <int NT, int MINB, bool DYN>
+// Shared memory (dynamic), in order: REC[F*LS] (ulonglong2: per frequency and
+// layer the (Re s, Re s) and (Im s, Im s) pairs), KR[2*K2] (ulonglong2: per
+// abscissa pair the (lambda^2, -sqrt(2) lambda) pairs, then the two Hankel
+// weights), vals[kValsWords], imh[F], T[G*F], TH[F*LS] (float: the depth
+// cutoff's thresholds), MS[F] (float: max_n(-Re s_n), the lambda^2 under which
+// some root has a negative real part).  The items (frequency major, F*K2 of
+// them) are taken in rounds of kValsWords: every item stores its weighted pair
+// value at its own index in the buffer; after the round each frequency the
+// round touched is summed by four consecutive lanes (lane s adds the values at
+// s + 4 i into four accumulators by i mod 4, then a tree over the sixteen
+// partial sums, two levels by shuffles) and added to imh[f], rounds in order.
+// The order of every sum is fixed by the item indices alone.  (The throughput
+// system's 60 x 100 items take one round.)
+template <int NT, int MINB, bool DYN, bool SPEC>
 __global__ void __launch_bounds__(NT, MINB) forward_f32_kernel(ModelsView<FP32Ops> mv, int F, int G, int K,
-                                                               int cc_form, int LS,
+                                                               int cc_form, int LS, float len,
                                                                const float *__restrict__ g_omega,
                                                                const float *__restrict__ g_lam,
                                                                const float *__restrict__ g_hw,
@@ -582,13 +611,11 @@ __global__ void __launch_bounds__(NT, MINB) forward_f32_kernel(ModelsView<FP32Op
     constexpr int NW = NT / 32;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int K2 = (K + 1) / 2;
-    const int RB1 = (LS + 1) * kRecWords;  // ulonglong2 per frequency block
     ulonglong2 *REC = reinterpret_cast<ulonglong2 *>(smem_raw);
-    ulonglong2 *KR = REC + (size_t)F * RB1;
-    u64 *Y = reinterpret_cast<u64 *>(KR + 2 * K2);
-    float *vals = reinterpret_cast<float *>(Y + (size_t)F * LS);
-    float2 *stmp = reinterpret_cast<float2 *>(vals);  // prologue only: the item loop overwrites it
-    float *imh = vals + value_words(F, LS);
+    ulonglong2 *KR = REC + (size_t)F * LS;
+    u64 *HW = reinterpret_cast<u64 *>(KR + K2);
+    float *vals = reinterpret_cast<float *>(HW + K2);
+    float *imh = vals + vals_words(F, K2);
     float *Ts = imh + F;
     float *TH = Ts + (size_t)G * F;  // depth-cutoff thresholds, [F][LS]
     __shared__ ulonglong2 HE[AEM_MAX_LAYERS];
@@ -603,11 +630,12 @@ __global__ void __launch_bounds__(NT, MINB) forward_f32_kernel(ModelsView<FP32Op
     for (int k = tid; k < K2; k += blockDim.x) {
         const int kb = k + K2 < K ? k + K2 : K - 1;
         const float la = g_lam[k], lb = g_lam[kb];
-        KR[2 * k] = make_ulonglong2(pk2(la * la, lb * lb),
-                                    pk2(1.41421356237309505f * la, 1.41421356237309505f * lb));
-        KR[2 * k + 1] = make_ulonglong2(pk2(g_hw[k], k + K2 < K ? g_hw[kb] : 0.f), 0ull);
+        KR[k] = make_ulonglong2(pk2(la * la, lb * lb),
+                                pk2(-1.41421356237309505f * la, -1.41421356237309505f * lb));
+        HW[k] = pk2(g_hw[k], k + K2 < K ? g_hw[kb] : 0.f);
     }
-    const float mu0 = (float)kMu0;
+    const unsigned rec_a = (unsigned)__cvta_generic_to_shared(REC), he_a = (unsigned)__cvta_generic_to_shared(HE);
+    const float mu0 = (float)kMu0 * len * len, ilen = 1.f / len;
     const int FK2 = F * K2;
     const bool wide = K2 >= 32;  // 32 consecutive items span two frequencies at most
 
@@ -625,7 +653,7 @@ __global__ void __launch_bounds__(NT, MINB) forward_f32_kernel(ModelsView<FP32Op
         if (tid < L) {
             const size_t o = (size_t)p * mv.lmax + tid;
             lsig[tid] = exp10f(mv.logsig[o]);
-            lh[tid] = exp10f(mv.logh[o]);
+            lh[tid] = exp10f(mv.logh[o]) * ilen;
             const float e = -1.41421356237309505f * 1.44269504088896341f * lh[tid];
             HE[tid] = make_ulonglong2(pk2(e, e), pk2(e * 0.69314718055994531f, e * 0.69314718055994531f));
             lm[tid] = mv.m[o];
@@ -673,45 +701,27 @@ __global__ void __launch_bounds__(NT, MINB) forward_f32_kernel(ModelsView<FP32Op
                 }
             }
             const float sx = -w * mu0 * si, sy = w * mu0 * sr;
-            REC[(size_t)f * RB1 + kRecWords * (n + 1)] = make_ulonglong2(pk2(sx, sx), pk2(sy * sy, sy * sy));
-            Y[(size_t)f * LS + n] = pk2(sy, sy);
-            stmp[(size_t)f * LS + n] = make_float2(sx, sy);
+            REC[(size_t)f * LS + n] = make_ulonglong2(pk2(sx, sx), pk2(sy, sy));
         }
         __syncthreads();
-        for (int i = tid; i < F * L; i += blockDim.x) {
-            const int f = i / L, n = i - f * L;
-            const float2 a = stmp[(size_t)f * LS + n];
-            if (n + 1 < L) {
-                const float2 b = stmp[(size_t)f * LS + n + 1];
-                const float bx = 2.f * (a.x - b.x), by = 2.f * (a.y - b.y);
-                ulonglong2 *r = REC + (size_t)f * RB1 + kRecWords * (n + 1);
-                r[1] = make_ulonglong2(pk2(bx, bx), pk2(by, by));
-                r[2] = make_ulonglong2(pk2(-2.f * bx, -2.f * bx), pk2(2.f * by, 2.f * by));
-            }
-            if (n == 0) {
-                const float bx = -2.f * a.x, by = -2.f * a.y;
-                ulonglong2 *r = REC + (size_t)f * RB1;
-                r[1] = make_ulonglong2(pk2(bx, bx), pk2(by, by));
-                r[2] = make_ulonglong2(pk2(-2.f * bx, -2.f * bx), pk2(2.f * by, 2.f * by));
-            }
-        }
         // the depth cutoff's thresholds (depth_cutoff.h), one frequency per thread
         const bool cut = att0 > 0.f && L > 1;
         if (cut)
-            for (int f = tid; f < F; f += blockDim.x)
-                depth_thresholds([&](int n) { return stmp[(size_t)f * LS + n]; }, lh, L, att0, TH + (size_t)f * LS);
+            for (int f = tid; f < F; f += blockDim.x) {
+                const float4 *rf = reinterpret_cast<const float4 *>(REC + (size_t)f * LS);
+                depth_thresholds([&](int n) { const float4 v = rf[n]; return make_float2(v.x, v.z); }, lh, L, att0,
+                                 TH + (size_t)f * LS);
+            }
         __syncthreads();
 
         // The item loop in rounds of kValsWords items.  A warp takes whole
         // groups of 32 consecutive items (one per lane), the same groups in
         // every launch shape: its groups of the round are g = g0 + warp + j NW,
-        // taken 32 at a time, one per lane.  Each lane finds its group's layer
-        // count: the largest any of its items needs, which within a frequency
-        // is that of its smallest lambda (the pair's first abscissa), so the
-        // group's first item and the first item of each later frequency it
-        // reaches.  The chunk is then taken bucket by bucket of layer count (a
-        // ballot per count), so every bucket runs the recursion specialised
-        // on its count.
+        // looked at 32 at a time, one per lane.  Each lane finds its group's
+        // layer count: the largest any of its items needs, which within a
+        // frequency is that of its smallest lambda (the pair's first abscissa),
+        // so the group's first item and the first item of each later frequency
+        // it reaches.
         for (int r0 = 0; r0 < FK2; r0 += kValsWords) {
             const int r1 = r0 + kValsWords < FK2 ? r0 + kValsWords : FK2;
             const int g0 = r0 >> 5, g1 = (r1 + 31) >> 5;
@@ -727,53 +737,70 @@ __global__ void __launch_bounds__(NT, MINB) forward_f32_kernel(ModelsView<FP32Op
                         lpl = 1;
                         for (int ff = f0; ff <= f1; ++ff) {
                             float l2, lb2;
-                            up2(KR[2 * (ff == f0 ? first - f0 * K2 : 0)].x, l2, lb2);
+                            up2(KR[ff == f0 ? first - f0 * K2 : 0].x, l2, lb2);
                             lpl = max(lpl, depth_layers(l2, TH + (size_t)ff * LS, L));
                         }
                     }
                     if (steps_out) nsteps += (unsigned int)lpl * (unsigned int)(last + 1 - first);
                 }
-                for (int v = __reduce_max_sync(kFull, lpl); v >= 1; --v) {
-                    unsigned int mask = __ballot_sync(kFull, lpl == v);
-                    auto run = [&](auto lt) {
-                        constexpr int LT = decltype(lt)::value;
-                        while (mask) {
-                            const int jl = __ffs(mask) - 1;
-                            mask &= mask - 1;
-                            const int pk = __shfl_sync(kFull, pkl, jl);
-                            const int item = 32 * (gc + jl * NW) + lane;
-                            if (item >= r1) continue;
-                            int f = pk >> 16, k = (pk & 0xffff) + lane;
-                            if (k >= K2) {  // into the next frequency; further ones only when K2 < 32
+                auto item_of = [&](int pk, int j, auto body) {
+                    const int item = 32 * (gc + j * NW) + lane;
+                    if (item >= r1) return;
+                    int f = (pk >> 16) & 0xff, k = (pk & 0xffff) + lane;
+                    if (k >= K2) {  // into the next frequency; further ones only when K2 < 32
+                        k -= K2;
+                        ++f;
+                        if (!wide)
+                            while (k >= K2) {
                                 k -= K2;
                                 ++f;
-                                if (!wide)
-                                    while (k >= K2) {
-                                        k -= K2;
-                                        ++f;
-                                    }
                             }
-                            const ulonglong2 lw = KR[2 * k];
-                            float v0, v1;
-                            im_r0_pair<LT>(lw.x, lw.y, REC + f * RB1, Y + f * LS, HE, v, v0, v1);
-                            float h0, h1;
-                            up2(KR[2 * k + 1].x, h0, h1);
-                            vals[item - r0] = fmaf(h0, v0, h1 * v1);
+                    }
+                    const ulonglong2 lw = KR[k];
+                    float v0, v1;
+                    body(lw, rec_a + (unsigned)(f * LS) * 16u, v0, v1);
+                    float h0, h1;
+                    up2(HW[k], h0, h1);
+                    vals[item - r0] = fmaf(h0, v0, h1 * v1);
+                };
+                if constexpr (SPEC) {
+                    // bucket by bucket of layer count (a ballot per count), so
+                    // every bucket runs the recursion unrolled for its count
+                    for (int v = __reduce_max_sync(kFull, lpl); v >= 1; --v) {
+                        const unsigned int all = __ballot_sync(kFull, lpl == v);
+                        if (!all) continue;
+                        auto run = [&](auto lt) {
+                            constexpr int LT = decltype(lt)::value;
+                            for (unsigned int mask = all; mask; mask &= mask - 1) {
+                                const int jl = __ffs(mask) - 1;
+                                const int pk = __shfl_sync(kFull, pkl, jl);
+                                item_of(pk, jl, [&](ulonglong2 lw, unsigned rec, float &v0, float &v1) {
+                                    im_r0_pair<LT>(lw.x, lw.y, rec, he_a, v, v0, v1);
+                                });
+                            }
+                        };
+                        switch (v) {
+                            case 1: run(std::integral_constant<int, 1>{}); break;
+                            case 2: run(std::integral_constant<int, 2>{}); break;
+                            case 3: run(std::integral_constant<int, 3>{}); break;
+                            case 4: run(std::integral_constant<int, 4>{}); break;
+                            case 5: run(std::integral_constant<int, 5>{}); break;
+                            case 6: run(std::integral_constant<int, 6>{}); break;
+                            case 7: run(std::integral_constant<int, 7>{}); break;
+                            case 8: run(std::integral_constant<int, 8>{}); break;
+                            case 9: run(std::integral_constant<int, 9>{}); break;
+                            case 10: run(std::integral_constant<int, 10>{}); break;
+                            default: run(std::integral_constant<int, 0>{}); break;
                         }
-                    };
-                    if (!mask) continue;
-                    switch (v) {
-                        case 1: run(std::integral_constant<int, 1>{}); break;
-                        case 2: run(std::integral_constant<int, 2>{}); break;
-                        case 3: run(std::integral_constant<int, 3>{}); break;
-                        case 4: run(std::integral_constant<int, 4>{}); break;
-                        case 5: run(std::integral_constant<int, 5>{}); break;
-                        case 6: run(std::integral_constant<int, 6>{}); break;
-                        case 7: run(std::integral_constant<int, 7>{}); break;
-                        case 8: run(std::integral_constant<int, 8>{}); break;
-                        case 9: run(std::integral_constant<int, 9>{}); break;
-                        case 10: run(std::integral_constant<int, 10>{}); break;
-                        default: run(std::integral_constant<int, 0>{}); break;
+                    }
+                } else {
+                    pkl |= lpl << 24;
+                    const int nj = min(32, (g1 - gc + NW - 1) / NW);
+                    for (int j = 0; j < nj; ++j) {
+                        const int pk = __shfl_sync(kFull, pkl, j);
+                        item_of(pk, j, [&](ulonglong2 lw, unsigned rec, float &v0, float &v1) {
+                            im_r0_pair<0>(lw.x, lw.y, rec, he_a, pk >> 24, v0, v1);
+                        });
                     }
                 }
             }
@@ -857,27 +884,41 @@ __global__ void __launch_bounds__(NT, MINB) forward_f32_kernel(ModelsView<FP32Op
 
 size_t smem_bytes_f32(int F, int G, int K, int LS) {
     const int K2 = (K + 1) / 2;
-    return sizeof(ulonglong2) * ((size_t)F * (LS + 1) * kRecWords + 2 * (size_t)K2) + sizeof(u64) * (size_t)F * LS +
-           sizeof(float) * (value_words(F, LS) + F + (size_t)G * F + (size_t)F * LS);
+    return sizeof(ulonglong2) * ((size_t)F * LS + K2) + sizeof(u64) * (size_t)K2 +
+           sizeof(float) * (vals_words(F, K2) + (size_t)F + (size_t)G * F + (size_t)F * LS);
 }
 
-// Launch shapes of forward_f32_kernel: (threads per CTA, resident CTAs per SM
-// the register budget must allow).  Index 0 is the default.
+// Launch shapes of forward_f32_kernel: threads per CTA, resident CTAs per SM
+// the register budget must allow, and whether the recursion is unrolled per
+// layer count.  A marginal layer costs a warp's 32 items about 96 cycles of an
+// SM sub-partition unrolled and 104 in the two-layer loop (register-port and
+// special-function rates together, whatever the shape), but the unrolled code
+// (about 55 steps) overflows the instruction cache when many small CTAs are
+// each at another layer count, while the small CTAs lose less at the barriers
+// between a model's phases.  2^17 random models of the 60-frequency,
+// 200-abscissa system: 9.13 ms unrolled at 256 x 3, 10.8 ms looped at 128 x 8;
+// 32,768 models of the 40-frequency, 120-abscissa one (up to 8 layers): 0.96
+// and 0.89 ms.  (10.34 and 1.07 ms before the interface coefficient of the
+// roots alone, all unrolled.)
 struct F32Shape {
     int nt, minb;
 };
-constexpr F32Shape kF32Shapes[] = {{256, 4}, {128, 8}, {512, 2}, {256, 3}, {128, 6}};
+#define AEM_SHAPES(X)                                                                        \
+    X(0, 256, 4, false) X(1, 128, 8, false) X(2, 512, 2, true) X(3, 256, 3, true) X(4, 128, 6, false)
+#define AEM_SHAPE(I, NT, MINB, SPEC) {NT, MINB},
+constexpr F32Shape kF32Shapes[] = {AEM_SHAPES(AEM_SHAPE)};
+#undef AEM_SHAPE
 // shapes kNumBase .. 2 kNumBase - 1 are the same with dynamic model scheduling
 constexpr int kNumBase = sizeof(kF32Shapes) / sizeof(kF32Shapes[0]);
 constexpr int kNumF32Shapes = 2 * kNumBase;
 
-template <int NT, int MINB, bool DYN>
+template <int NT, int MINB, bool DYN, bool SPEC>
 int launch_shape(const aem_system *sys, const ModelsView<FP32Ops> &mv, int LS, float *gates, float *imh,
                  const double *y_obs, int obs_per, const double *eps_an, double eps_mn, double *ll,
                  cudaStream_t stream, int *counter_ext, const int *active, unsigned long long *steps,
                  const int8_t *valid) {
     const SystemTables &h = sys->host;
-    auto kern = forward_f32_kernel<NT, MINB, DYN>;
+    auto kern = forward_f32_kernel<NT, MINB, DYN, SPEC>;
     const size_t smem = smem_bytes_f32(h.F, h.G, h.K, LS);
     // always: the static shared memory counts against the 48 KB default too
     AEM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -895,7 +936,7 @@ int launch_shape(const aem_system *sys, const ModelsView<FP32Ops> &mv, int LS, f
     if (own)  // stream-ordered: one counter per launch, so launches on other streams never share it
         AEM_CUDA_TRY(cudaMallocAsync((void **)&counter, sizeof(int), stream));
     if (DYN) AEM_CUDA_TRY(cudaMemsetAsync(counter, 0, sizeof(int), stream));
-    kern<<<(unsigned)grid, NT, smem, stream>>>(mv, h.F, h.G, h.K, h.cc_form, LS, sys->d_omega_f, sys->d_lam_f,
+    kern<<<(unsigned)grid, NT, smem, stream>>>(mv, h.F, h.G, h.K, h.cc_form, LS, sys->len, sys->d_omega_f, sys->d_lamu_f,
                                                sys->d_hw_f, sys->d_T_f, gates, imh, y_obs, obs_per, eps_an, eps_mn,
                                                ll, counter, active, sys->depth_att, steps, valid);
     const cudaError_t e = cudaGetLastError();
@@ -908,23 +949,16 @@ int launch_shape_index(int idx, const aem_system *sys, const ModelsView<FP32Ops>
                        float *imh, const double *y_obs, int obs_per, const double *eps_an, double eps_mn, double *ll,
                        cudaStream_t stream, int *counter_ext = nullptr, const int *active = nullptr,
                        unsigned long long *steps = nullptr, const int8_t *valid = nullptr) {
-#define AEM_SHAPE(I, NT, MINB, DYN) \
-    case I:                         \
-        return launch_shape<NT, MINB, DYN>(sys, mv, LS, gates, imh, y_obs, obs_per, eps_an, eps_mn, ll, stream, \
-                                           counter_ext, active, steps, valid);
+#define AEM_SHAPE(I, NT, MINB, SPEC)                                                                                 \
+    case I:                                                                                                        \
+        return launch_shape<NT, MINB, false, SPEC>(sys, mv, LS, gates, imh, y_obs, obs_per, eps_an, eps_mn, ll, stream, \
+                                             counter_ext, active, steps, valid);                                   \
+    case I + kNumBase:                                                                                             \
+        return launch_shape<NT, MINB, true, SPEC>(sys, mv, LS, gates, imh, y_obs, obs_per, eps_an, eps_mn, ll, stream,  \
+                                            counter_ext, active, steps, valid);
     switch (idx) {
-        AEM_SHAPE(1, 128, 8, false)
-        AEM_SHAPE(2, 512, 2, false)
-        AEM_SHAPE(3, 256, 3, false)
-        AEM_SHAPE(4, 128, 6, false)
-        AEM_SHAPE(5, 256, 4, true)
-        AEM_SHAPE(6, 128, 8, true)
-        AEM_SHAPE(7, 512, 2, true)
-        AEM_SHAPE(8, 256, 3, true)
-        AEM_SHAPE(9, 128, 6, true)
-        default:
-            return launch_shape<256, 4, false>(sys, mv, LS, gates, imh, y_obs, obs_per, eps_an, eps_mn, ll, stream,
-                                               counter_ext, active, steps, valid);
+        AEM_SHAPES(AEM_SHAPE)
+        default: return fail(AEM_ERR_INVALID_ARG, "forward kernel: launch shape");
     }
 #undef AEM_SHAPE
 }
@@ -945,7 +979,11 @@ int launch_forward_f32(const aem_system *sys, const Models *models, float *gates
     ModelsView<FP32Ops> mv{models->n_models, models->lmax, models->nlayers, models->logsig, models->logh,
                            models->m, models->logtau, models->c};
     const int LS = models->lmax;
-    return launch_shape_index(sys->f32_shape[LS], sys, mv, LS, gates, imh, y_obs, obs_per, eps_an, eps_mn, ll,
+    // No shape recorded: the smallest CTAs for batches that fill the chip;
+    // with at most two models per SM the largest, which finish a model soonest.
+    int shape = sys->f32_shape[LS];
+    if (shape == 0) shape = models->n_models <= 2 * sys->num_sms ? 2 : 1;
+    return launch_shape_index(shape, sys, mv, LS, gates, imh, y_obs, obs_per, eps_an, eps_mn, ll,
                               (cudaStream_t)stream, counter_ext, active, steps, valid);
 }
 

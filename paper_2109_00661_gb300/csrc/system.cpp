@@ -302,9 +302,14 @@ extern "C" int aem_system_create(const aem_system_desc *desc, aem_system **out) 
         return cuda_fail(e, "cudaDeviceGetAttribute");
     }
     const SystemTables &h = s->host;
+    const double len = std::exp2(std::floor(std::log2(2.0 * h.h + h.a)));
+    std::vector<double> lamu(h.lam);
+    for (double &l : lamu) l *= len;
+    s->len = (float)len;
     if ((rc = upload(&s->d_omega_f, h.omega)) || (rc = upload(&s->d_lam_f, h.lam)) || (rc = upload(&s->d_hw_f, h.hw)) ||
         (rc = upload(&s->d_T_f, h.T)) || (rc = upload(&s->d_omega_d, h.omega)) || (rc = upload(&s->d_lam_d, h.lam)) ||
-        (rc = upload(&s->d_hw_d, h.hw)) || (rc = upload(&s->d_T_d, h.T))) {
+        (rc = upload(&s->d_hw_d, h.hw)) || (rc = upload(&s->d_T_d, h.T)) ||
+        (rc = upload(&s->d_lamu_f, lamu))) {
         aem_system_destroy(s);
         return rc;
     }
@@ -321,7 +326,7 @@ extern "C" int aem_system_create(const aem_system_desc *desc, aem_system **out) 
 extern "C" int aem_system_destroy(aem_system *s) {
     if (!s) return AEM_OK;
     void *ptrs[] = {s->d_omega_f, s->d_lam_f, s->d_hw_f, s->d_T_f,
-                    s->d_omega_d, s->d_lam_d, s->d_hw_d, s->d_T_d, s->d_status};
+                    s->d_omega_d, s->d_lam_d, s->d_hw_d, s->d_T_d, s->d_lamu_f, s->d_status};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     delete s;
