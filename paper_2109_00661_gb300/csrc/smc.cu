@@ -32,7 +32,6 @@ namespace {
 constexpr int KS = AEM_SMC_SLOTS;  // interface slots per profile
 constexpr int kMoves = 6;
 constexpr int kGroupThreads = 1024;
-constexpr int kClusterThreads = 512;  // per CTA of the cluster-split reweight step
 constexpr unsigned kFullMask = 0xffffffffu;
 constexpr int kPurposeMove = 64, kPurposeValue = 65, kPurposeAccept = 66, kPurposeResample = 67;
 // Langevin: acceptance uniform, and normal j of the proposal from words
@@ -245,44 +244,108 @@ __global__ void merge_kernel(PState st, int P, int LMS, int8_t *nl, T *logsig, T
     nl[i] = (int8_t)L;
 }
 
+// Exclusive prefix sums over a CTA of kGroupThreads threads; returns this
+// thread's prefix.  tmp: 33 values of shared memory, free again on return.
+template <class T>
+__device__ inline T block_scan(T v, T *tmp) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    T x = v;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const T t = __shfl_up_sync(kFullMask, x, d);
+        if (lane >= d) x += t;
+    }
+    if (lane == 31) tmp[warp] = x;
+    __syncthreads();
+    if (warp == 0) {
+        T y = tmp[lane];
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const T t = __shfl_up_sync(kFullMask, y, d);
+            if (lane >= d) y += t;
+        }
+        tmp[lane + 1] = y;
+        if (lane == 0) tmp[0] = 0;
+    }
+    __syncthreads();
+    const T r = tmp[warp] + x - v;
+    __syncthreads();
+    return r;
+}
+
 // ------------------------------------------------ grouping by model (stable)
 // One CTA per sounding: counts N_k, offsets and the particle indices of each
-// model in increasing index order (warp per model, ballot scans).
-__global__ void __launch_bounds__(kGroupThreads) group_kernel(const int *kappa, const int *lam, int N, int lp1,
-                                                              int M, int *perm, int *off, int *counts) {
-    extern __shared__ unsigned char mid[];
-    __shared__ int s_cnt[AEM_SMC_MAX_MODELS];
-    __shared__ int s_off[AEM_SMC_MAX_MODELS + 1];
-    const int s = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-    const int base = s * N;
-    for (int j = tid; j < N; j += blockDim.x) mid[j] = (unsigned char)(kappa[base + j] * lp1 + lam[base + j]);
-    __syncthreads();
-    for (int k = warp; k < M; k += nw) {
-        int cnt = 0;
-        for (int b0 = 0; b0 < N; b0 += 32) {
-            int j = b0 + lane;
-            cnt += __popc(__ballot_sync(kFullMask, j < N && mid[j] == k));
-        }
-        if (lane == 0) s_cnt[k] = cnt;
-    }
-    __syncthreads();
-    if (tid == 0) {
-        s_off[0] = 0;
-        for (int k = 0; k < M; ++k) s_off[k + 1] = s_off[k] + s_cnt[k];
-    }
-    __syncthreads();
-    for (int k = warp; k < M; k += nw) {
-        int pos = s_off[k];
-        for (int b0 = 0; b0 < N; b0 += 32) {
-            int j = b0 + lane;
-            bool p = j < N && mid[j] == k;
-            unsigned bal = __ballot_sync(kFullMask, p);
-            if (p) perm[base + pos + __popc(bal & ((1u << lane) - 1u))] = base + j;
-            pos += __popc(bal);
+// model in increasing index order.  Each of the 32 warps counts the models of
+// its slice of the particles (lanes of one model found by a ballot per bit of
+// the id, each particle's rank within its warp and model kept), and a scan over
+// (model, warp) turns the counts into first positions: one pass over the
+// particles whatever the number of models (a warp per model read them M / 16
+// times over: 30 us at 16,384 particles and 100 models).  model: the particle's
+// id (the standalone entries) in place of kappa * lp1 + lam; an id outside
+// [0, M) takes no part, and its anc_out / w_out entry is set to -1 / 0.
+// Dynamic shared memory: rank [N] (uint16), ids [N] (uint8; 255 for none).
+size_t group_smem_bytes(int N) { return 3 * (size_t)N; }
+__global__ void __launch_bounds__(kGroupThreads) group_kernel(const int *kappa, const int *lam, const int *model, int N,
+                                                              int lp1, int M, int *perm, int *off, int *counts,
+                                                              int *anc_out, double *w_out) {
+    constexpr int NW = kGroupThreads / 32;
+    extern __shared__ unsigned short rank[];
+    unsigned char *ids = reinterpret_cast<unsigned char *>(rank + N);
+    __shared__ int first[AEM_SMC_MAX_MODELS * NW];
+    __shared__ int tmp[33];
+    const int s = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int base = s * N, per = (N + NW - 1) / NW, j0 = warp * per, j1 = min(N, j0 + per);
+    for (int i = tid; i < M * NW; i += kGroupThreads) first[i] = 0;
+#pragma unroll 4
+    for (int j = tid; j < N; j += kGroupThreads) {
+        const int id = model ? model[base + j] : kappa[base + j] * lp1 + lam[base + j];
+        const bool ok = id >= 0 && id < M;
+        ids[j] = (unsigned char)(ok ? id : 255);
+        if (!ok) {
+            if (anc_out) anc_out[base + j] = -1;
+            if (w_out) w_out[base + j] = 0.0;
         }
     }
-    for (int k = tid; k < M; k += blockDim.x) counts[s * M + k] = s_cnt[k];
-    for (int k = tid; k <= M; k += blockDim.x) off[s * (M + 1) + k] = s_off[k];
+    __syncthreads();
+    auto id_of = [&](int j) { return j < j1 && ids[j] != 255 ? (int)ids[j] : -1; };
+    static_assert(AEM_SMC_MAX_MODELS <= 128 && AEM_SMC_MAX_PARTICLES <= 65536, "ids and ranks");
+    const int bits = 32 - __clz(M - 1 > 0 ? M - 1 : 1);
+    for (int b = j0; b < j1; b += 32) {
+        const int j = b + lane, id = id_of(j);
+        unsigned same = __ballot_sync(kFullMask, id >= 0);
+        for (int q = 0; q < bits; ++q) {
+            const unsigned set = __ballot_sync(kFullMask, (id >> q) & 1);
+            same &= (id >> q) & 1 ? set : ~set;
+        }
+        if (id >= 0) {
+            const int have = first[id * NW + warp];
+            rank[j] = (unsigned short)(have + __popc(same & ((1u << lane) - 1u)));
+            __syncwarp(same);
+            if (lane == __ffs(same) - 1) first[id * NW + warp] = have + __popc(same);
+        }
+        __syncwarp();
+    }
+    __syncthreads();
+    // exclusive scan over (model, warp)
+    const int total = M * NW, ch = (total + kGroupThreads - 1) / kGroupThreads, i0 = tid * ch;
+    int sum = 0;
+    for (int i = i0; i < min(total, i0 + ch); ++i) sum += first[i];
+    int run = block_scan(sum, tmp);
+    for (int i = i0; i < min(total, i0 + ch); ++i) {
+        const int v = first[i];
+        first[i] = run;
+        if (i % NW == 0) off[s * (M + 1) + i / NW] = run;
+        run += v;
+        if (i == total - 1) off[s * (M + 1) + M] = run;
+    }
+    __syncthreads();
+    for (int k = tid; k < M; k += kGroupThreads) {
+        const int next = k + 1 < M ? first[(k + 1) * NW] : off[s * (M + 1) + M];
+        counts[s * M + k] = next - first[k * NW];
+    }
+    __syncthreads();
+    for (int j = j0 + lane; j < j1; j += 32)
+        if (ids[j] != 255) perm[base + first[ids[j] * NW + warp] + rank[j]] = base + j;
 }
 
 template <class T>
@@ -292,321 +355,456 @@ __device__ inline T warp_sum_t(T v) {
     return v;
 }
 
-__device__ inline double warp_max(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(kFullMask, v, o));
-    return v;
-}
-
 // -------------------------------------------------------------- reweight (a7)
-// One CTA per sounding.  With W uniform within each model after the last
-// resample, a_i = dgamma * ll_i, S1_k = sum e^{a_i - a_max}, S2_k = sum e^{2(a_i - a_max)},
-// ESS_k = S1^2 / S2 and TESS = sum_k ESS_k.  gamma_t by bisection on TESS = alpha N.
-// dense (dynamic shared memory of reweight_dense_bytes(N)): the sounding's
-// log-likelihoods are staged once in model-grouped order, and each evaluation
-// forms every particle's e^{a_i - a_max} once, one particle per thread, before
-// the per-model sums read them (the FP64 exponentials are the step's cost on
-// this part, and per-model lanes would leave most of them idle on small
-// models); the sums, and so every result, are the same as without it.
-constexpr int kDenseMaxParticles = 12000;
-size_t reweight_dense_bytes(int N) {
-    return N <= kDenseMaxParticles ? (size_t)N * (2 * sizeof(double) + 1) : 0;
-}
-__global__ void __launch_bounds__(kGroupThreads)
-    reweight_kernel(const double *ll, const int *perm, const int *off, const int *counts, int N, int M, double alpha,
-                    int iters, double *gamma, double *logz, double *Wg, double *dgamma_out, int *done_out,
-                    int *status = nullptr, int dense = 0) {
-    extern __shared__ __align__(16) unsigned char rw_smem[];
-    double *sv = reinterpret_cast<double *>(rw_smem);               // [N] ll at each grouped position
-    double *se = sv + N;                                             // [N] e^{a - a_max} of the evaluation
-    unsigned char *spm = reinterpret_cast<unsigned char *>(se + N);  // [N] model at each grouped position
-    __shared__ double s_max[AEM_SMC_MAX_MODELS], s_s1[AEM_SMC_MAX_MODELS], s_ess[AEM_SMC_MAX_MODELS];
-    __shared__ double s_tess;
-    const int s = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-    const int *o = off + s * (M + 1);
-    const int *cnt = counts + s * M;
-    const double g0 = gamma[s];
-    if (g0 >= 1.0) {
-        if (tid == 0) {
-            dgamma_out[s] = 0.0;
-            done_out[s] = 1;
-        }
-        return;
-    }
-    for (int k = warp; k < M; k += nw) {
-        double mx = -INFINITY;
-        for (int r = lane; r < cnt[k]; r += 32) mx = fmax(mx, ll[perm[s * N + o[k] + r]]);
-        mx = warp_max(mx);
-        if (lane == 0) s_max[k] = mx;
-    }
-    __syncthreads();
-    // no particle of the sounding with a finite log-likelihood: there is no
-    // weight to form; record AEM_ERR_NONFINITE, keep gamma and log Z, and
-    // leave uniform weights within each model so the resample stays defined
-    if (tid == 0) {
-        bool any = false;
-        for (int k = 0; k < M; ++k) any = any || s_max[k] > -INFINITY;
-        s_tess = any ? 1.0 : 0.0;
-    }
-    __syncthreads();
-    if (s_tess == 0.0) {
-        for (int k = warp; k < M; k += nw)
-            for (int r = lane; r < cnt[k]; r += 32) Wg[s * N + o[k] + r] = 1.0 / (double)cnt[k];
-        if (tid == 0) {
-            dgamma_out[s] = 0.0;
-            done_out[s] = 0;
-            if (status) atomicExch(status, (int)AEM_ERR_NONFINITE);
-        }
-        return;
-    }
-    if (dense) {
-        for (int k = warp; k < M; k += nw)
-            for (int r = lane; r < cnt[k]; r += 32) {
-                sv[o[k] + r] = ll[perm[s * N + o[k] + r]];
-                spm[o[k] + r] = (unsigned char)k;
-            }
-        __syncthreads();
-    }
-    auto evaluate = [&](double dg) {
-        if (dense) {
-            for (int q = tid; q < o[M]; q += blockDim.x) {
-                const double v = sv[q];
-                se[q] = (v == -INFINITY) ? 0.0 : exp(dg * (v - s_max[spm[q]]));
-            }
-            __syncthreads();
-        }
-        for (int k = warp; k < M; k += nw) {
-            double s1 = 0.0, s2 = 0.0;
-            const double mk = s_max[k];
-            for (int r = lane; r < cnt[k]; r += 32) {
-                double e;
-                if (dense) {
-                    e = se[o[k] + r];
-                } else {
-                    const double v = ll[perm[s * N + o[k] + r]];
-                    e = (v == -INFINITY) ? 0.0 : exp(dg * (v - mk));
-                }
-                s1 += e;
-                s2 += e * e;
-            }
-            s1 = warp_sum_t(s1);
-            s2 = warp_sum_t(s2);
-            if (lane == 0) {
-                s_s1[k] = s1;
-                s_ess[k] = (cnt[k] > 0 && s2 > 0.0) ? s1 * s1 / s2 : 0.0;
-            }
-        }
-        __syncthreads();
-        if (warp == 0) {
-            double t = 0.0;
-            for (int k = lane; k < M; k += 32) t += s_ess[k];
-            t = warp_sum_t(t);
-            if (lane == 0) s_tess = t;
-        }
-        __syncthreads();
-        return s_tess;
-    };
-    const double target = alpha * (double)o[M];  // N, less any particle the grouping left out
-    double hi = 1.0 - g0, dg;
-    int done;
-    if (evaluate(hi) >= target) {
-        dg = hi;
-        done = 1;
-    } else {
-        double lo = 0.0;
-        for (int it = 0; it < iters; ++it) {
-            double mid = 0.5 * (lo + hi);
-            if (evaluate(mid) >= target)
-                lo = mid;
-            else
-                hi = mid;
-        }
-        // lo = 0: no probed step kept TESS >= alpha N (more than (1 - alpha) N
-        // particles with ll = -inf drop out at any positive step); take the
-        // smallest probed step and record AEM_ERR_NO_BRACKET
-        if (lo == 0.0 && status && tid == 0) atomicExch(status, (int)AEM_ERR_NO_BRACKET);
-        dg = lo > 0.0 ? lo : hi;
-        done = 0;
-        evaluate(dg);
-    }
-    for (int k = warp; k < M; k += nw) {
-        const int n = cnt[k];
-        if (n == 0) continue;
-        const double mk = s_max[k], s1 = s_s1[k];
-        for (int r = lane; r < n; r += 32) {
-            // the last evaluation was at dg: its e^{a - a_max} are in se
-            double e;
-            if (dense) {
-                e = se[o[k] + r];
-            } else {
-                const double v = ll[perm[s * N + o[k] + r]];
-                e = (v == -INFINITY) ? 0.0 : exp(dg * (v - mk));
-            }
-            Wg[s * N + o[k] + r] = e / s1;
-        }
-        if (lane == 0) logz[s * M + k] += dg * mk + log(s1) - log((double)n);
-    }
-    if (tid == 0) {
-        gamma[s] = done ? 1.0 : g0 + dg;
-        dgamma_out[s] = dg;
-        done_out[s] = done;
-    }
+// With W uniform within each model after the last resample,
+// a_i = dgamma * ll_i, S1_k = sum e^{a_i - a_max}, S2_k = sum e^{2(a_i - a_max)},
+// ESS_k = S1^2 / S2 and TESS = sum_k ESS_k; gamma_t by bisection on TESS = alpha N
+// (`iters` halvings of (0, 1 - gamma_{t-1}]).
+//
+// FP64 is the whole cost (an SM retires about 1.65 FP64 operations a clock: a
+// warp's exponential takes some 340 cycles, one addition 19), so few
+// evaluations are made in it.  TESS decreases in dgamma, so a halving needs
+// FP64 only where TESS is close to alpha N: each probe is evaluated in FP32
+// first (error about 3e-6 of TESS) and decided there while it is further than
+// kScreen from the target; at the first probe that is not, the crossing itself
+// is found by Newton's method on the FP64 TESS with the FP32 slope (kept inside
+// the bracket) in about three evaluations, and the remaining halvings compare
+// their midpoint with it.  Where that does not settle, the remaining probes are
+// evaluated in FP64 one by one.  One more FP64 evaluation at the step taken
+// gives the weights and log Z.
+//
+// A cluster of C CTAs works on one sounding (C = 1: a plain CTA).  CTA r stages
+// the r-th of C equal slices of the model-grouped positions, in FP32 into every
+// CTA of the cluster: each screens all particles by itself.  Of an FP64
+// evaluation CTA r takes its own slice, 32 positions per warp and pass whatever
+// their models (the exponentials stay dense), and after one cluster barrier
+// every CTA adds the C partial sums of each model in rank order through
+// distributed shared memory, so all CTAs take the same decisions.  The partials
+// are double-buffered: evaluation e writes buffer e mod 2, and the barrier of
+// evaluation e + 1 is passed only after every CTA has read evaluation e's.
+// 9,600 particles in 20 models, alpha 0.5: 3.9 ms with every probe in FP64 on
+// one SM, 116 us now (16 FP32 probes of 2.6 us, three FP64 ones of 13.7 us).
+constexpr double kScreen = 1e-4;    // of alpha N
+constexpr double kSettled = 1e-10;  // relative step after which the next one is below 2^-49 (slope to 1e-5)
+constexpr int kNewton = 8;
+constexpr int kMaxCluster = 8;
+
+// Dynamic shared memory: v64 [slice] (ll - max of its model, then the
+// exponentials), b1, b2 [blocks + models] (a 32-position block's share of a
+// model's sums: blocks and models both advance along the positions, so block
+// i's part of model k has entry i + k to itself), v32 [N], md [slice] (uint8,
+// the positions' models).
+__host__ __device__ inline int reweight_slice(int N, int C) { return N / C + 1; }
+size_t reweight_smem_bytes(int N, int C) {
+    const size_t n = (size_t)reweight_slice(N, C);
+    return sizeof(double) * (n + 2 * ((n + 31) / 32 + AEM_SMC_MAX_MODELS)) + sizeof(float) * (size_t)N + n;
 }
 
-// The same reweight step split over a thread-block cluster of C CTAs per
-// sounding, for samplers with few soundings and many particles (one CTA per
-// sounding would leave most SMs idle while its FP64 sums run 60 bisection
-// passes).  CTA r of the cluster takes the r-th of C equal slices of the
-// sounding's model-grouped particle positions; every evaluation forms, per
-// model, the partial sums S1, S2 (and once the maximum) over its slice, then
-// after one cluster barrier every CTA adds the C partials of each model in
-// rank order through distributed shared memory, so all CTAs evaluate TESS
-// identically and take the same bisection decisions.  The partials are
-// double-buffered: evaluation e writes buffer e mod 2, and the barrier of
-// evaluation e + 1 is passed only after every CTA has read evaluation e's.
-__global__ void __launch_bounds__(kClusterThreads)
-    reweight_cluster_kernel(const double *ll, const int *perm, const int *off, const int *counts, int N, int M,
-                            double alpha, int iters, double *gamma, double *logz, double *Wg, double *dgamma_out,
-                            int *done_out, int *status) {
+struct RwArgs {
+    const double *ll;
+    const int *perm, *off, *counts;
+    int N, M;
+    double alpha;
+    int iters;
+    const double *gamma_in;  // [S], or null: gamma0
+    double gamma0;
+    double *gamma_out;  // [S] or null
+    double *logz;       // [S][M], added to (logz_add) or set
+    int logz_add;
+    double *Wg;     // grouped weights, or null
+    double *W_out;  // weights by particle, or null
+    double *dgamma_out;
+    int *done_out, *status;
+};
+
+__global__ void __launch_bounds__(kGroupThreads) reweight_kernel(const RwArgs a) {
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
-    __shared__ double p_s1[2][AEM_SMC_MAX_MODELS], p_s2[2][AEM_SMC_MAX_MODELS], p_max[AEM_SMC_MAX_MODELS];
-    __shared__ double s_max[AEM_SMC_MAX_MODELS], s_s1[AEM_SMC_MAX_MODELS], s_ess[AEM_SMC_MAX_MODELS];
-    __shared__ double s_tess;
+    constexpr int NW = kGroupThreads / 32;
+    extern __shared__ __align__(16) unsigned char rw_smem[];
+    // a warp's share of a model's FP32 sums, warp w's part of model k at w + k
+    __shared__ float f1[NW + AEM_SMC_MAX_MODELS], f2[NW + AEM_SMC_MAX_MODELS], f3[NW + AEM_SMC_MAX_MODELS],
+        f4[NW + AEM_SMC_MAX_MODELS];
+    __shared__ double p_s1[2][AEM_SMC_MAX_MODELS], p_s2[2][AEM_SMC_MAX_MODELS], s_max[AEM_SMC_MAX_MODELS],
+        s_s1[AEM_SMC_MAX_MODELS], s_red[4];
+    __shared__ long long p_key[AEM_SMC_MAX_MODELS];
+    __shared__ float s_fred[2][4], s_g;
+    __shared__ double s_x;
+    __shared__ int so[AEM_SMC_MAX_MODELS + 1], s_any, s_op;
     const int C = (int)cl.num_blocks(), rank = (int)cl.block_rank();
-    const int s = blockIdx.x / C, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5;
-    const int *o = off + s * (M + 1);
-    const int *cnt = counts + s * M;
-    const double g0 = gamma[s];
+    const int s = blockIdx.x / C, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int N = a.N, M = a.M;
+    const double g0 = a.gamma_in ? a.gamma_in[s] : a.gamma0;
     if (g0 >= 1.0) {  // the same for every CTA of the cluster: none reaches a barrier
         if (tid == 0 && rank == 0) {
-            dgamma_out[s] = 0.0;
-            done_out[s] = 1;
+            a.dgamma_out[s] = 0.0;
+            a.done_out[s] = 1;
         }
         return;
     }
-    const int total = o[M];
+    const int *perm = a.perm + (size_t)s * N;
+    for (int k = tid; k <= M; k += kGroupThreads) so[k] = a.off[s * (M + 1) + k];
+    constexpr long long kLowest = -0x7fffffffffffffffll - 1;
+    for (int k = tid; k < M; k += kGroupThreads) p_key[k] = kLowest;
+    if (tid == 0) s_any = 0;
+    __syncthreads();
+    const int total = so[M];
     const int lo_pos = (int)((long long)total * rank / C), hi_pos = (int)((long long)total * (rank + 1) / C);
-    // positions of model k inside this CTA's slice
-    auto span = [&](int k, int &a, int &b) {
-        a = o[k] > lo_pos ? o[k] : lo_pos;
-        b = o[k + 1] < hi_pos ? o[k + 1] : hi_pos;
+    const int own = hi_pos - lo_pos, sl = reweight_slice(N, C), blocks = (own + 31) >> 5;
+    double *v64 = reinterpret_cast<double *>(rw_smem);
+    double *b1 = v64 + sl, *b2 = b1 + (sl + 31) / 32 + AEM_SMC_MAX_MODELS;
+    float *v32 = reinterpret_cast<float *>(b2 + (sl + 31) / 32 + AEM_SMC_MAX_MODELS);
+    unsigned char *md = reinterpret_cast<unsigned char *>(v32 + N);
+    auto first_model = [&](int q) {  // of position q: the last k with so[k] <= q
+        int k = 0, b = M;
+        while (b - k > 1) {
+            const int m = (k + b) >> 1;
+            if (so[m] <= q)
+                k = m;
+            else
+                b = m;
+        }
+        return k;
     };
-    for (int k = warp; k < M; k += nw) {
-        int a, b;
-        span(k, a, b);
-        double mx = -INFINITY;
-        for (int q = a + lane; q < b; q += 32) mx = fmax(mx, ll[perm[s * N + q]]);
-        mx = warp_max(mx);
-        if (lane == 0) p_max[k] = mx;
+    // per-model maxima: this slice's by integer comparison (the doubles' bits in
+    // an order-preserving form), then the cluster's
+    for (int i = tid; i < own; i += kGroupThreads) {
+        const double v = a.ll[perm[lo_pos + i]];
+        const int k = first_model(lo_pos + i);
+        v64[i] = v;
+        md[i] = (unsigned char)k;
+        const long long b = __double_as_longlong(v);
+        atomicMax(&p_key[k], b ^ ((b >> 63) & 0x7fffffffffffffffll));
     }
-    cl.sync();
-    for (int k = tid; k < M; k += blockDim.x) {
-        double mx = -INFINITY;
-        for (int q = 0; q < C; ++q) mx = fmax(mx, *cl.map_shared_rank(&p_max[k], q));
+    __syncthreads();
+    if (C > 1) cl.sync();
+    for (int k = tid; k < M; k += kGroupThreads) {
+        long long key = p_key[k];
+        for (int q = 0; q < C; ++q) {
+            const long long o = *cl.map_shared_rank(&p_key[k], q);
+            key = o > key ? o : key;
+        }
+        const double mx = key == kLowest ? -INFINITY
+                                         : __longlong_as_double(key ^ ((key >> 63) & 0x7fffffffffffffffll));
         s_max[k] = mx;
+        if (mx > -INFINITY) s_any = 1;
     }
     __syncthreads();
-    if (tid == 0) {
-        bool any = false;
-        for (int k = 0; k < M; ++k) any = any || s_max[k] > -INFINITY;
-        s_tess = any ? 1.0 : 0.0;
-    }
-    __syncthreads();
-    if (s_tess == 0.0) {  // no finite log-likelihood in the sounding (see reweight_kernel)
-        for (int k = warp; k < M; k += nw) {
-            int a, b;
-            span(k, a, b);
-            for (int q = a + lane; q < b; q += 32) Wg[s * N + q] = 1.0 / (double)cnt[k];
+    if (!s_any) {
+        // no particle of the sounding with a finite log-likelihood: there is no
+        // weight to form; record AEM_ERR_NONFINITE, keep gamma and log Z, and
+        // leave uniform weights within each model so the resample stays defined
+        for (int i = tid; i < own; i += kGroupThreads) {
+            const int k = md[i];
+            const double w = 1.0 / (double)(so[k + 1] - so[k]);
+            if (a.Wg) a.Wg[(size_t)s * N + lo_pos + i] = w;
+            if (a.W_out) a.W_out[perm[lo_pos + i]] = w;
         }
-        if (tid == 0 && rank == 0) {
-            dgamma_out[s] = 0.0;
-            done_out[s] = 0;
-            if (status) atomicExch(status, (int)AEM_ERR_NONFINITE);
+        if (rank == 0) {
+            if (!a.logz_add)
+                for (int k = tid; k < M; k += kGroupThreads) a.logz[(size_t)s * M + k] = 0.0;
+            if (tid == 0) {
+                a.dgamma_out[s] = 0.0;
+                a.done_out[s] = 0;
+                if (a.status) atomicExch(a.status, (int)AEM_ERR_NONFINITE);
+            }
         }
-        cl.sync();  // no CTA leaves while another may still read its p_max
+        if (C > 1) cl.sync();  // no CTA leaves while another may still read its p_key
         return;
     }
-    int buf = 0;
-    auto evaluate = [&](double dg) {
-        for (int k = warp; k < M; k += nw) {
-            int a, b;
-            span(k, a, b);
-            double s1 = 0.0, s2 = 0.0;
-            const double mk = s_max[k];
-            for (int q = a + lane; q < b; q += 32) {
-                const double v = ll[perm[s * N + q]];
-                const double e = (v == -INFINITY) ? 0.0 : exp(dg * (v - mk));
+    for (int i = tid; i < own; i += kGroupThreads) {
+        const double v = v64[i], d = v == -INFINITY ? -INFINITY : v - s_max[md[i]];
+        v64[i] = d;
+        const float f = fmaxf((float)d, -3e38f);  // finite: a product with a zero exponential stays zero
+        for (int q = 0; q < C; ++q) *cl.map_shared_rank(&v32[lo_pos + i], q) = f;
+    }
+    if (C > 1)
+        cl.sync();
+    else
+        __syncthreads();
+    const int w0 = (int)((long long)total * warp / NW), w1 = (int)((long long)total * (warp + 1) / NW);
+    const int k_first = first_model(w0);
+    const int nw = (M + 31) >> 5;  // warps with a thread per model
+    // TESS and its slope in FP32 into s_fred, over all particles: each warp an
+    // equal share of the positions
+    auto screen = [&](float g) {
+        for (int k = k_first; k < M && so[k] < w1; ++k) {
+            const int qa = max(so[k], w0), qb = min(so[k + 1], w1);
+            if (qa >= qb) continue;
+            float s1 = 0.f, s2 = 0.f, d1 = 0.f, d2 = 0.f;
+            for (int q = qa + lane; q < qb; q += 32) {
+                const float v = v32[q];
+                float e;
+                asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(g * v));
+                const float ve = v * e;
                 s1 += e;
-                s2 += e * e;
+                s2 = fmaf(e, e, s2);
+                d1 += ve;
+                d2 = fmaf(ve, e, d2);
             }
             s1 = warp_sum_t(s1);
             s2 = warp_sum_t(s2);
+            d1 = warp_sum_t(d1);
+            d2 = warp_sum_t(d2);
             if (lane == 0) {
-                p_s1[buf][k] = s1;
-                p_s2[buf][k] = s2;
+                f1[warp + k] = s1;
+                f2[warp + k] = s2;
+                f3[warp + k] = d1;
+                f4[warp + k] = d2;
             }
         }
-        cl.sync();
-        for (int k = tid; k < M; k += blockDim.x) {
-            double s1 = 0.0, s2 = 0.0;
-            for (int q = 0; q < C; ++q) {
-                s1 += *cl.map_shared_rank(&p_s1[buf][k], q);
-                s2 += *cl.map_shared_rank(&p_s2[buf][k], q);
+        __syncthreads();
+        if (warp < nw) {
+            float ess = 0.f, de = 0.f;
+            if (tid < M && so[tid] < so[tid + 1]) {
+                float s1 = 0.f, s2 = 0.f, d1 = 0.f, d2 = 0.f;
+                const int qa = so[tid], qb = so[tid + 1];
+                int w = (int)((long long)qa * NW / total);
+                while (w > 0 && (int)((long long)total * w / NW) > qa) --w;
+                for (; w < NW; ++w) {
+                    const int x0 = (int)((long long)total * w / NW), x1 = (int)((long long)total * (w + 1) / NW);
+                    if (x0 >= qb) break;
+                    if (max(x0, qa) < min(x1, qb)) {
+                        s1 += f1[w + tid];
+                        s2 += f2[w + tid];
+                        d1 += f3[w + tid];
+                        d2 += f4[w + tid];
+                    }
+                }
+                if (s2 > 0.f) {
+                    ess = s1 * s1 / s2;
+                    // d (S1^2 / S2) with dS1 = sum v e, dS2 = 2 sum v e^2
+                    de = 2.f * s1 / s2 * (d1 - s1 / s2 * d2);
+                }
             }
-            s_s1[k] = s1;
-            s_ess[k] = (cnt[k] > 0 && s2 > 0.0) ? s1 * s1 / s2 : 0.0;
+            ess = warp_sum_t(ess);
+            de = warp_sum_t(de);
+            if (lane == 0) {
+                s_fred[0][warp] = ess;
+                s_fred[1][warp] = de;
+            }
         }
         __syncthreads();
-        if (warp == 0) {
-            double t = 0.0;
-            for (int k = lane; k < M; k += 32) t += s_ess[k];
-            t = warp_sum_t(t);
-            if (lane == 0) s_tess = t;
-        }
-        __syncthreads();
-        buf ^= 1;
-        return s_tess;
     };
-    const double target = alpha * (double)total;
-    double hi = 1.0 - g0, dg;
-    int done;
-    if (evaluate(hi) >= target) {
-        dg = hi;
-        done = 1;
-    } else {
-        double lo = 0.0;
-        for (int it = 0; it < iters; ++it) {
+    int buf = 0;
+    // TESS in FP64 into s_red; final: the exponentials replace v64 and each model's S1 is
+    // left in s_s1
+    auto evaluate = [&](double dg, bool final) {
+        for (int i = warp; i < blocks; i += NW) {
+            const int q = 32 * i + lane;
+            double e = 0.0;
+            int k = -1;
+            if (q < own) {
+                const double v = v64[q];
+                k = md[q];
+                e = v == -INFINITY ? 0.0 : exp(dg * v);
+                if (final) v64[q] = e;
+            }
+            const double e2 = e * e;
+            const int ka = md[32 * i], kb = md[min(32 * i + 31, own - 1)];
+            for (int kk = ka; kk <= kb; ++kk) {
+                // both sums in one butterfly: the lower half of the warp takes
+                // S1, the upper S2
+                const double x1 = k == kk ? e : 0.0, x2 = k == kk ? e2 : 0.0;
+                const double give = lane < 16 ? x2 : x1, keep = lane < 16 ? x1 : x2;
+                double x = keep + __shfl_xor_sync(kFullMask, give, 16);
+#pragma unroll
+                for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(kFullMask, x, o);
+                if (lane == 0) b1[i + kk] = x;
+                if (lane == 16) b2[i + kk] = x;
+            }
+        }
+        __syncthreads();
+        double s1 = 0.0, s2 = 0.0;
+        if (tid < M) {
+            const int qa = max(so[tid], lo_pos) - lo_pos, qb = min(so[tid + 1], hi_pos) - lo_pos;
+            for (int i = qa >> 5; 32 * i < qb; ++i) {
+                s1 += b1[i + tid];
+                s2 += b2[i + tid];
+            }
+        }
+        if (C > 1) {
+            if (tid < M) {
+                p_s1[buf][tid] = s1;
+                p_s2[buf][tid] = s2;
+            }
+            cl.sync();
+            if (tid < M) {
+                double r1[kMaxCluster], r2[kMaxCluster];
+#pragma unroll
+                for (int q = 0; q < kMaxCluster; ++q) {  // every load before the first sum
+                    r1[q] = q < C ? *cl.map_shared_rank(&p_s1[buf][tid], q) : 0.0;
+                    r2[q] = q < C ? *cl.map_shared_rank(&p_s2[buf][tid], q) : 0.0;
+                }
+                s1 = s2 = 0.0;
+#pragma unroll
+                for (int q = 0; q < kMaxCluster; ++q) {
+                    s1 += r1[q];
+                    s2 += r2[q];
+                }
+            }
+            buf ^= 1;
+        }
+        if (warp < nw) {
+            double ess = 0.0;
+            if (tid < M) {
+                if (final) s_s1[tid] = s1;
+                if (s2 > 0.0) ess = s1 * s1 / s2;
+            }
+            ess = warp_sum_t(ess);
+            if (lane == 0) s_red[warp] = ess;
+        }
+        __syncthreads();
+    };
+    // The halvings are driven by warp 0 alone (FP64 control code run by every
+    // warp would cost 19 cycles per operation and warp): it asks the CTA for the
+    // FP32 or FP64 TESS at a point, or for the last evaluation.
+    enum { kOpScreen, kOpEvaluate, kOpFinal };
+    const double target = a.alpha * (double)total;  // N, less any particle the grouping left out
+    double hi = 1.0 - g0, lo = 0.0, x = hi, xa = 0.0, xb = 0.0, cross = 0.0;
+    int it = -1, how = 0, newton = -1, done = 0;  // it = -1: the probe at 1 - gamma
+    // how: 0 FP32 decides, 1 the crossing, 2 FP64 decides
+    auto ask_screen = [&](double at) {
+        const double g = at * 1.4426950408889634;
+        x = at;
+        if (lane == 0) {
+            s_g = (float)g;
+            s_x = at;
+            s_op = g > 1e-30 ? kOpScreen : kOpEvaluate;  // below, FP32 cannot tell a particle from one at -inf
+        }
+    };
+    auto ask = [&](int op, double at) {
+        x = at;
+        if (lane == 0) {
+            s_x = at;
+            s_op = op;
+        }
+    };
+    // the next request after the probe of halving `it` was decided
+    auto next = [&](bool keep) {
+        if (it < 0) {
+            if (keep) {
+                done = 1;
+                ask(kOpFinal, hi);
+                return;
+            }
+        } else if (keep) {
+            lo = x;
+        } else {
+            hi = x;
+        }
+        ++it;
+        for (; how == 1 && it < a.iters; ++it) {
             const double mid = 0.5 * (lo + hi);
-            if (evaluate(mid) >= target)
+            if (mid <= cross)
                 lo = mid;
             else
                 hi = mid;
         }
-        if (lo == 0.0 && status && tid == 0 && rank == 0) atomicExch(status, (int)AEM_ERR_NO_BRACKET);
-        dg = lo > 0.0 ? lo : hi;
-        done = 0;
-        evaluate(dg);
-    }
-    for (int k = warp; k < M; k += nw) {
-        int a, b;
-        span(k, a, b);
-        const double mk = s_max[k], s1 = s_s1[k];
-        for (int q = a + lane; q < b; q += 32) {
-            const double v = ll[perm[s * N + q]];
-            Wg[s * N + q] = (v == -INFINITY) ? 0.0 : exp(dg * (v - mk)) / s1;
+        if (it >= a.iters) {
+            // lo = 0: no probed step kept TESS >= alpha N (more than (1 - alpha) N
+            // particles with ll = -inf drop out at any positive step); take the
+            // smallest probed step and record AEM_ERR_NO_BRACKET
+            if (lo == 0.0 && a.status && lane == 0 && rank == 0) atomicExch(a.status, (int)AEM_ERR_NO_BRACKET);
+            ask(kOpFinal, lo > 0.0 ? lo : hi);
+            return;
         }
+        const double mid = 0.5 * (lo + hi);
+        if (how == 0)
+            ask_screen(mid);
+        else
+            ask(kOpEvaluate, mid);
+    };
+    if (warp == 0) ask_screen(hi);
+    __syncthreads();
+    float slope = 0.f;
+    for (;;) {
+        const int op = s_op;
+        if (op == kOpScreen)
+            screen(s_g);
+        else
+            evaluate(s_x, op == kOpFinal);
+        if (op == kOpFinal) break;
+        if (warp == 0) {
+            if (op == kOpScreen) {
+                float t = 0.f;
+                slope = 0.f;
+                for (int w = 0; w < nw; ++w) {
+                    t += s_fred[0][w];
+                    slope += s_fred[1][w];
+                }
+                const double off = (double)t - target;
+                if (fabs(off) > kScreen * target) {
+                    next(off >= 0.0);
+                } else {
+                    double y = x;
+                    if (it >= 0) {
+                        newton = 0;
+                        xa = lo;
+                        xb = hi;
+                        y = x - off / (double)slope;  // FP32's own step first
+                        if (!(y > xa && y < xb)) y = x;
+                    }
+                    ask(kOpEvaluate, y);
+                }
+            } else {
+                double t = 0.0;
+                for (int w = 0; w < nw; ++w) t += s_red[w];
+                if (newton < 0) {
+                    if (it >= 0) how = 2;
+                    next(t >= target);
+                } else {
+                    // Newton's method for the crossing, started at this halving's midpoint
+                    if (t >= target)
+                        xa = x;
+                    else
+                        xb = x;
+                    double y = x - (t - target) / (double)slope;
+                    const bool in = y > xa && y < xb;  // false for NaN
+                    const bool settled = in && fabs(y - x) <= kSettled * x;
+                    if (!settled && ++newton < kNewton) {
+                        ask(kOpEvaluate, in ? y : 0.5 * (xa + xb));
+                    } else {
+                        newton = -1;
+                        const double mid = 0.5 * (lo + hi);
+                        if (settled) {
+                            how = 1;
+                            cross = y;
+                            x = mid;
+                            next(mid <= cross);
+                        } else {
+                            how = 2;
+                            ask(kOpEvaluate, mid);
+                        }
+                    }
+                }
+            }
+        }
+        __syncthreads();
+    }
+    const double dg = s_x;
+    for (int i = tid; i < own; i += kGroupThreads) {
+        const int k = md[i];
+        const double w = s_max[k] == -INFINITY ? 0.0 : v64[i] / s_s1[k];
+        if (a.Wg) a.Wg[(size_t)s * N + lo_pos + i] = w;
+        if (a.W_out) a.W_out[perm[lo_pos + i]] = w;
     }
     if (rank == 0) {
-        for (int k = tid; k < M; k += blockDim.x)
-            if (cnt[k] > 0) logz[s * M + k] += dg * s_max[k] + log(s_s1[k]) - log((double)cnt[k]);
-        if (tid == 0) {
-            gamma[s] = done ? 1.0 : g0 + dg;
-            dgamma_out[s] = dg;
-            done_out[s] = done;
+        for (int k = tid; k < M; k += kGroupThreads) {
+            const int n = so[k + 1] - so[k];
+            const double z = n > 0 ? dg * s_max[k] + log(s_s1[k]) - log((double)n) : 0.0;
+            if (a.logz_add)
+                a.logz[(size_t)s * M + k] += z;
+            else
+                a.logz[(size_t)s * M + k] = z;
+        }
+        if (tid == 0) {  // warp 0: `done` is the driver's
+            if (a.gamma_out) a.gamma_out[s] = done ? 1.0 : g0 + dg;
+            a.dgamma_out[s] = dg;
+            a.done_out[s] = done;
         }
     }
-    cl.sync();  // every CTA's partials stay readable until all have finished
+    if (C > 1) cl.sync();  // every CTA's partials stay readable until all have finished
 }
 
 // Non-finite log-likelihoods (NaN, or +inf, which no Gaussian likelihood can
@@ -652,22 +850,45 @@ __global__ void odds_kernel(const int *counts, int S, int M, int lp1, int N, dou
 }
 
 // ------------------------------------------------------------- resample (a8)
-// One CTA per sounding, warp per model.  q_r = round(W_r 2^40), C = prefix
-// sums with the last entry forced to 2^40; output slot j takes the smallest r
-// with C_r > floor((j 2^40 + u40_k) / N_k).
+// One CTA per sounding.  q_r = round(W_r 2^40), C = prefix sums with the last
+// entry forced to 2^40; output slot j takes the smallest r with
+// C_r > floor((j 2^40 + u40_k) / N_k).  In integers that is j 2^40 + u40_k <
+// N_k C_r, so r's slots are [cnt(C_{r-1}), cnt(C_r)) with cnt(C) =
+// ceil((N_k C - u40_k) / 2^40): one block scan of the q_r over all models'
+// positions (exact: 100 models' sums fit 47 bits; a model's own prefix is the
+// difference to its first one), the slot where each r begins marked in shared
+// memory, and a running maximum over the slots in place of a binary search of
+// C in global memory per slot (9,600 particles in 20 models: 24 us; one model
+// of 16,384 took 14 dependent reads of C for each of its 512 slots per lane).
+// Dynamic shared memory: q [N] (u64), mark [N] (int).
+// round(w 2^40) to nearest even from w's bits, 0 <= w < 2^22 (any other value
+// gives some in-range integer): integer work only, as a warp's FP64 product and
+// conversion cost 38 cycles.
+__device__ inline unsigned long long cdf_quantum(double w) {
+    const unsigned long long bits = (unsigned long long)__double_as_longlong(w);
+    const int e = (int)((bits >> 52) & 0x7ff);
+    if (e == 0) return 0ull;  // zero, or too small to count
+    const unsigned long long m = (bits & 0xfffffffffffffull) | 0x10000000000000ull;
+    const int right = 1075 - kCdfBits - e;  // m 2^(e - 1075) 2^40 = m >> right
+    if (right <= 0) return right > -11 ? m << -right : 0ull;
+    if (right > 54) return 0ull;
+    const unsigned long long q = m >> right, rest = m - (q << right), half = 1ull << (right - 1);
+    return q + ((rest > half || (rest == half && (q & 1ull))) ? 1ull : 0ull);
+}
+
+size_t resample_smem_bytes(int N) { return (sizeof(unsigned long long) + sizeof(int)) * (size_t)N; }
 __global__ void __launch_bounds__(kGroupThreads)
-    resample_kernel(const double *Wg, const int *perm, const int *off, const int *counts, int N, int M,
+    resample_kernel(const double *Wg, const double *W, const int *perm, const int *off, int N, int M,
                     const unsigned long long *u40_in, unsigned long long seed, int stage, const int *stage_dev,
-                    unsigned long long *C,
                     int *anc) {
-    const int s = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int *o = off + s * (M + 1);
-    const int *cnt = counts + s * M;
+    extern __shared__ unsigned long long sq[];
+    int *mark = reinterpret_cast<int *>(sq + N);
+    __shared__ unsigned long long s_u40[AEM_SMC_MAX_MODELS], s_first[AEM_SMC_MAX_MODELS], tmp64[33];
+    __shared__ int so[AEM_SMC_MAX_MODELS + 1], tmp32[33];
+    const int s = blockIdx.x, tid = threadIdx.x;
     const unsigned long long one = 1ull << kCdfBits;
-    for (int k = warp; k < M; k += nw) {
-        const int n = cnt[k];
-        if (n == 0) continue;
-        const int b = s * N + o[k];
+    for (int k = tid; k <= M; k += kGroupThreads) so[k] = off[s * (M + 1) + k];
+    for (int k = tid; k < M; k += kGroupThreads) {
         unsigned long long u40;
         if (u40_in) {
             u40 = u40_in[s * M + k];
@@ -677,34 +898,80 @@ __global__ void __launch_bounds__(kGroupThreads)
                         (uint32_t)(stage_dev ? *stage_dev : stage), 0u);
             u40 = (((unsigned long long)w[0] << 8) | (unsigned long long)(w[1] >> 24)) & (one - 1ull);
         }
-        unsigned long long carry = 0;
-        for (int r0 = 0; r0 < n; r0 += 32) {
-            int r = r0 + lane;
-            unsigned long long q = r < n ? (unsigned long long)__double2ll_rn(Wg[b + r] * (double)one) : 0ull;
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                unsigned long long t = __shfl_up_sync(kFullMask, q, d);
-                if (lane >= d) q += t;
-            }
-            if (r < n) C[b + r] = carry + q;
-            carry += __shfl_sync(kFullMask, q, 31);
-        }
-        __syncwarp();
-        if (lane == 0) C[b + n - 1] = one;
-        __syncwarp();
-        for (int j = lane; j < n; j += 32) {
-            unsigned long long thr = ((unsigned long long)j * one + u40) / (unsigned long long)n;
-            int lo = 0, hi = n - 1;
-            while (lo < hi) {
-                int mid = (lo + hi) >> 1;
-                if (C[b + mid] > thr)
-                    hi = mid;
-                else
-                    lo = mid + 1;
-            }
-            anc[perm[b + j]] = perm[b + lo];
+        s_u40[k] = u40;
+    }
+    __syncthreads();
+    const int total = so[M], ch = (total + kGroupThreads - 1) / kGroupThreads;
+    const int a = min(total, tid * ch), b = min(total, a + ch);
+    const int *pm = perm + (size_t)s * N;
+#pragma unroll 4
+    for (int r = tid; r < total; r += kGroupThreads)
+        sq[r] = cdf_quantum(W ? W[pm[r]] : Wg[(size_t)s * N + r]);
+    __syncthreads();
+    unsigned long long sum = 0;
+    for (int r = a; r < b; ++r) sum += sq[r];
+    const unsigned long long before = block_scan(sum, tmp64);
+    int k0 = 0;  // the model of position a: the last one that begins at or before it
+    for (int hi = M; hi - k0 > 1;) {
+        const int m = (k0 + hi) >> 1;
+        if (so[m] <= a)
+            k0 = m;
+        else
+            hi = m;
+    }
+    // each model's prefix at its first position, and its first slot's default
+    {
+        unsigned long long run = before;
+        int k = k0;
+        for (int r = a; r < b; ++r) {
+            while (so[k + 1] <= r) ++k;
+            if (r == so[k]) s_first[k] = run;
+            mark[r] = r == so[k] ? r : -1;
+            run += sq[r];
         }
     }
+    __syncthreads();
+    {
+        unsigned long long run = before;
+        int k = k0;
+        for (int r = a; r < b; ++r) {
+            while (so[k + 1] <= r) ++k;
+            const unsigned long long n = (unsigned long long)(so[k + 1] - so[k]), u = s_u40[k];
+            auto cnt = [&](unsigned long long C) {
+                const unsigned long long t = n * C;
+                const unsigned long long c = t > u ? (t - u + one - 1ull) >> kCdfBits : 0ull;
+                return (int)(c < n ? c : n);
+            };
+            const int c0 = cnt(run - s_first[k]);  // 0 at the model's first position
+            run += sq[r];
+            const int c1 = r + 1 == so[k + 1] ? (int)n : cnt(run - s_first[k]);
+            if (c1 > c0) mark[so[k] + c0] = r;
+        }
+    }
+    __syncthreads();
+    // running maximum over the slots (the marks grow within a model, and every
+    // model's first slot has one)
+    int top = -1;
+    for (int j = a; j < b; ++j) top = max(top, mark[j]);
+    const int lane = tid & 31, warp = tid >> 5;
+    int x = top;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int t = __shfl_up_sync(kFullMask, x, d);
+        if (lane >= d) x = max(x, t);
+    }
+    if (lane == 31) tmp32[warp + 1] = x;
+    int prev = __shfl_up_sync(kFullMask, x, 1);
+    if (lane == 0) prev = -1;
+    __syncthreads();
+    for (int w = 1; w <= warp; ++w) prev = max(prev, tmp32[w]);
+    for (int j = a; j < b; ++j) {
+        prev = max(prev, mark[j]);
+        mark[j] = prev;
+    }
+    __syncthreads();
+#pragma unroll 4
+    for (int j = tid; j < total; j += kGroupThreads) anc[pm[j]] = pm[mark[j]];
 }
 
 __global__ void gather_kernel(PState dst, PState src, const int *anc, int P) {
@@ -1744,35 +2011,6 @@ __global__ void philox_kernel(const uint32_t *ctr, uint32_t k0, uint32_t k1, uin
     for (int q = 0; q < 4; ++q) out[4 * i + q] = c[q];
 }
 
-// Model ids from a plain int array (the standalone reweight / resample entry
-// points take the model of each particle directly).
-// Model ids of the standalone a7 / a8 entries.  An id outside [0, n_models)
-// takes no part: it is given a group key no model has (255 > AEM_SMC_MAX_MODELS),
-// and its ancestor (resample) or weight (reweight) output is set to -1 / 0.
-__global__ void split_model_kernel(const int *model, int n, int n_models, int *kappa, int *lam, int *anc_out,
-                                   double *w_out) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int id = model[i];
-    const bool ok = id >= 0 && id < n_models;
-    kappa[i] = ok ? id : 255;
-    lam[i] = 0;
-    if (!ok && anc_out) anc_out[i] = -1;
-    if (!ok && w_out) w_out[i] = 0.0;
-}
-
-// perm lists the grouped particles only (off[M] of them, fewer than n when
-// some ids were out of range)
-__global__ void scatter_kernel(const double *Wg, const int *perm, const int *off, int M, double *W) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < off[M]) W[perm[i]] = Wg[i];
-}
-
-__global__ void gather_weights_kernel(const double *W, const int *perm, const int *off, int M, double *Wg) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < off[M]) Wg[i] = W[perm[i]];
-}
-
 inline unsigned blocks_for(long long n, int t) { return (unsigned)((n + t - 1) / t); }
 
 }  // namespace
@@ -1782,6 +2020,43 @@ inline unsigned blocks_for(long long n, int t) { return (unsigned)((n + t - 1) /
 // Host side
 // ========================================================================
 using namespace aem;
+
+namespace {
+// The dynamic shared memory the reweight and resample kernels may ask for
+// (the largest sounding's, so that no caller lowers it under another).
+int stage_kernel_attributes() {
+    AEM_CUDA_TRY(cudaFuncSetAttribute(reweight_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)reweight_smem_bytes(AEM_SMC_MAX_PARTICLES, 1)));
+    AEM_CUDA_TRY(cudaFuncSetAttribute(group_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)group_smem_bytes(AEM_SMC_MAX_PARTICLES)));
+    AEM_CUDA_TRY(cudaFuncSetAttribute(resample_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)resample_smem_bytes(AEM_SMC_MAX_PARTICLES)));
+    return AEM_OK;
+}
+
+// The reweight step of S soundings of N particles: one CTA per sounding, or,
+// when the soundings are few and large (N >= 1024), a cluster of up to eight
+// CTAs each as long as the clusters fit the SMs together.
+int launch_reweight(const RwArgs &a, int S, int num_sms, cudaStream_t stream) {
+    int C = 1;
+    if (a.N >= 1024)
+        while (C < kMaxCluster && (long long)S * C * 2 <= num_sms) C *= 2;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(S * C), 1, 1);
+    cfg.blockDim = dim3(kGroupThreads, 1, 1);
+    cfg.dynamicSmemBytes = reweight_smem_bytes(a.N, C);
+    cfg.stream = stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)C;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = C > 1 ? 1 : 0;
+    AEM_CUDA_TRY(cudaLaunchKernelEx(&cfg, reweight_kernel, a));
+    return AEM_OK;
+}
+}  // namespace
 
 struct smc_state {
     const aem_system *sys = nullptr;
@@ -1796,7 +2071,6 @@ struct smc_state {
     int *anc = nullptr, *perm = nullptr, *off = nullptr, *counts = nullptr, *acc = nullptr, *nprop = nullptr,
         *done = nullptr;
     double *Wg = nullptr, *gamma = nullptr, *logz = nullptr, *dgamma = nullptr;
-    unsigned long long *C = nullptr;
     int8_t *m_nl = nullptr;
     float *m_logsig = nullptr, *m_logh = nullptr, *m_m = nullptr, *m_logtau = nullptr, *m_c = nullptr;
     double *y = nullptr, *eps_an = nullptr;
@@ -2031,7 +2305,7 @@ extern "C" int smc_create(const aem_system *sys, const smc_desc *desc, const dou
         (rc = dalloc(st, &st->nprop, (size_t)st->S * kMoves)) || (rc = dalloc(st, &st->done, (size_t)st->S)) ||
         (rc = dalloc(st, &st->Wg, P)) || (rc = dalloc(st, &st->gamma, (size_t)st->S)) ||
         (rc = dalloc(st, &st->logz, (size_t)st->S * st->M)) || (rc = dalloc(st, &st->dgamma, (size_t)st->S)) ||
-        (rc = dalloc(st, &st->C, P)) || (rc = dalloc(st, &st->m_nl, P)) ||
+        (rc = dalloc(st, &st->m_nl, P)) ||
         (rc = dalloc(st, &st->m_logsig, P * st->LMS)) || (rc = dalloc(st, &st->m_logh, P * st->LMS)) ||
         (rc = dalloc(st, &st->m_m, P * st->LMS)) || (rc = dalloc(st, &st->m_logtau, P * st->LMS)) ||
         (rc = dalloc(st, &st->m_c, P * st->LMS)) || (rc = dalloc(st, &st->y, (size_t)st->S * G)) ||
@@ -2090,15 +2364,10 @@ extern "C" int smc_create(const aem_system *sys, const smc_desc *desc, const dou
         smc_destroy(st);
         return cuda_fail(e, "smc_create: upload data");
     }
-    // the reweight step's staging of the sounding's log-likelihoods: set now,
-    // not during a stream capture of the stage loop
-    const size_t rw_smem = reweight_dense_bytes(st->N);
-    if (rw_smem > 48 * 1024) {
-        e = cudaFuncSetAttribute(reweight_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rw_smem);
-        if (e != cudaSuccess) {
-            smc_destroy(st);
-            return cuda_fail(e, "smc_create: reweight shared memory");
-        }
+    // set now, not during a stream capture of the stage loop
+    if ((rc = stage_kernel_attributes())) {
+        smc_destroy(st);
+        return rc;
     }
     *out = st;
     return AEM_OK;
@@ -2156,45 +2425,25 @@ static int take_status(smc_state *st) {
                        : "reweight: a sounding has no particle with a finite log-likelihood");
 }
 
-// The reweight step of every sounding: one CTA per sounding, or, when the
-// soundings are few (the cluster of C CTAs per sounding still fits the SMs,
-// C <= 8) and large (N >= 1024), the cluster-split form.
 static int launch_reweight(smc_state *st, cudaStream_t stream) {
-    int C = 1;
-    if (st->N >= 1024)
-        while (C < 8 && (long long)st->S * C * 2 <= st->sys->num_sms) C *= 2;
-    if (C == 1) {
-        const size_t smem = reweight_dense_bytes(st->N);
-        reweight_kernel<<<st->S, kGroupThreads, smem, stream>>>(st->cur.ll, st->perm, st->off, st->counts, st->N,
-                                                                st->M, st->d.alpha, st->d.bisect_iters, st->gamma,
-                                                                st->logz, st->Wg, st->dgamma, st->done, st->d_status,
-                                                                smem > 0);
-        AEM_CUDA_TRY(cudaGetLastError());
-        return AEM_OK;
-    }
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)(st->S * C), 1, 1);
-    cfg.blockDim = dim3(kClusterThreads, 1, 1);
-    cfg.dynamicSmemBytes = 0;
-    cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)C;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    AEM_CUDA_TRY(cudaLaunchKernelEx(&cfg, reweight_cluster_kernel, (const double *)st->cur.ll, (const int *)st->perm,
-                                    (const int *)st->off, (const int *)st->counts, st->N, st->M, st->d.alpha,
-                                    st->d.bisect_iters, st->gamma, st->logz, st->Wg, st->dgamma, st->done,
-                                    st->d_status));
+    const RwArgs a{st->cur.ll, st->perm,  st->off,  st->counts, st->N,   st->M,   st->d.alpha, st->d.bisect_iters,
+                   st->gamma,  0.0,       st->gamma, st->logz,  1,       st->Wg,  nullptr,     st->dgamma,
+                   st->done,   st->d_status};
+    return launch_reweight(a, st->S, st->sys->num_sms, stream);
+}
+
+static int launch_resample(smc_state *st, int stage, const int *stage_dev, cudaStream_t stream) {
+    resample_kernel<<<st->S, kGroupThreads, resample_smem_bytes(st->N), stream>>>(st->Wg, nullptr, st->perm, st->off, st->N,
+                                                                           st->M, nullptr, st->d.seed, stage,
+                                                                           stage_dev, st->anc);
+    AEM_CUDA_TRY(cudaGetLastError());
     return AEM_OK;
 }
 
 static int launch_group(smc_state *st) {
-    group_kernel<<<st->S, kGroupThreads, st->N, st->stream>>>(st->cur.kappa, st->cur.lam, st->N,
-                                                              st->d.lambda_max + 1, st->M, st->perm, st->off,
-                                                              st->counts);
+    group_kernel<<<st->S, kGroupThreads, group_smem_bytes(st->N), st->stream>>>(st->cur.kappa, st->cur.lam, nullptr, st->N,
+                                                          st->d.lambda_max + 1, st->M, st->perm, st->off, st->counts,
+                                                          nullptr, nullptr);
     AEM_CUDA_TRY(cudaGetLastError());
     return AEM_OK;
 }
@@ -2214,10 +2463,8 @@ extern "C" int smc_reweight(smc_state *st, double *gamma_out) {
 
 extern "C" int smc_resample(smc_state *st) {
     if (!st) return fail(AEM_ERR_INVALID_ARG, "smc_resample: NULL state");
-    resample_kernel<<<st->S, kGroupThreads, 0, st->stream>>>(st->Wg, st->perm, st->off, st->counts, st->N, st->M,
-                                                             nullptr, st->d.seed, st->stage, nullptr, st->C,
-                                                             st->anc);
-    AEM_CUDA_TRY(cudaGetLastError());
+    int rc = launch_resample(st, st->stage, nullptr, st->stream);
+    if (rc) return rc;
     gather_kernel<<<blocks_for(st->P, 256), 256, 0, st->stream>>>(st->alt, st->cur, st->anc, st->P);
     AEM_CUDA_TRY(cudaGetLastError());
     PState t = st->cur;
@@ -2424,9 +2671,7 @@ static int enqueue_graph_stage(smc_state *st, int R, int stop_stage, cudaGraphCo
     int rc = launch_group(st);
     if (rc) return rc;
     if ((rc = launch_reweight(st, s))) return rc;
-    resample_kernel<<<st->S, kGroupThreads, 0, s>>>(st->Wg, st->perm, st->off, st->counts, st->N, st->M, nullptr,
-                                                    st->d.seed, 0, st->d_stage, st->C, st->anc);
-    AEM_CUDA_TRY(cudaGetLastError());
+    if ((rc = launch_resample(st, 0, st->d_stage, s))) return rc;
     gather_kernel<<<blocks_for(st->P, 256), 256, 0, s>>>(st->alt, st->cur, st->anc, st->P);
     AEM_CUDA_TRY(cudaGetLastError());
     copy_state_kernel<<<blocks_for(st->P, 256), 256, 0, s>>>(st->cur, st->alt, st->P);
@@ -2926,9 +3171,8 @@ extern "C" size_t aem_smc_workspace_bytes(int n, int n_models) {
 
 namespace {
 struct Workspace {
-    int *kappa, *lam, *perm, *off, *counts, *done;
-    double *Wg, *gamma;
-    unsigned long long *C;
+    double *Wg;
+    int *perm, *off, *counts;
 };
 
 Workspace carve(void *base, int n, int M) {
@@ -2938,21 +3182,11 @@ Workspace carve(void *base, int n, int M) {
     Workspace w;
     w.Wg = (double *)(p + o);
     o = align(o + sizeof(double) * n);
-    w.C = (unsigned long long *)(p + o);
-    o = align(o + sizeof(unsigned long long) * n);
-    w.gamma = (double *)(p + o);
-    o = align(o + sizeof(double));
-    w.kappa = (int *)(p + o);
-    o = align(o + sizeof(int) * n);
-    w.lam = (int *)(p + o);
-    o = align(o + sizeof(int) * n);
     w.perm = (int *)(p + o);
     o = align(o + sizeof(int) * n);
     w.off = (int *)(p + o);
     o = align(o + sizeof(int) * (M + 1));
     w.counts = (int *)(p + o);
-    o = align(o + sizeof(int) * M);
-    w.done = (int *)(p + o);
     return w;
 }
 
@@ -2975,18 +3209,16 @@ extern "C" int aem_reweight(const double *ll, const int *model, int n, int n_mod
         return fail(AEM_ERR_INVALID_ARG, "aem_reweight: NULL pointer or value out of range");
     cudaStream_t s = (cudaStream_t)stream;
     Workspace w = carve(work, n, n_models);
-    split_model_kernel<<<blocks_for(n, 256), 256, 0, s>>>(model, n, n_models, w.kappa, w.lam, nullptr, W);
-    group_kernel<<<1, kGroupThreads, n, s>>>(w.kappa, w.lam, n, 1, n_models, w.perm, w.off, w.counts);
-    AEM_CUDA_TRY(cudaMemcpyAsync(w.gamma, &gamma_prev, sizeof(double), cudaMemcpyHostToDevice, s));
-    AEM_CUDA_TRY(cudaMemsetAsync(logz_inc, 0, sizeof(double) * n_models, s));
-    const size_t smem = reweight_dense_bytes(n);
-    if (smem > 48 * 1024)
-        AEM_CUDA_TRY(cudaFuncSetAttribute(reweight_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    reweight_kernel<<<1, kGroupThreads, smem, s>>>(ll, w.perm, w.off, w.counts, n, n_models, alpha, bisect_iters,
-                                                   w.gamma, logz_inc, w.Wg, dgamma, reached_one, nullptr, smem > 0);
-    scatter_kernel<<<blocks_for(n, 256), 256, 0, s>>>(w.Wg, w.perm, w.off, n_models, W);
+    if ((rc = stage_kernel_attributes())) return rc;
+    int dev = 0, num_sms = 0;
+    AEM_CUDA_TRY(cudaGetDevice(&dev));
+    AEM_CUDA_TRY(cudaDeviceGetAttribute(&num_sms, cudaDevAttrMultiProcessorCount, dev));
+    group_kernel<<<1, kGroupThreads, group_smem_bytes(n), s>>>(nullptr, nullptr, model, n, 1, n_models, w.perm, w.off, w.counts, nullptr,
+                                             W);
     AEM_CUDA_TRY(cudaGetLastError());
-    return AEM_OK;
+    const RwArgs a{ll,      w.perm,  w.off,    w.counts, n, n_models, alpha, bisect_iters, nullptr,
+                   gamma_prev, nullptr, logz_inc, 0,     nullptr, W,  dgamma, reached_one, nullptr};
+    return launch_reweight(a, 1, num_sms, s);
 }
 
 extern "C" int aem_resample_systematic(const double *W, const int *model, int n, int n_models,
@@ -2997,11 +3229,12 @@ extern "C" int aem_resample_systematic(const double *W, const int *model, int n,
     if (!W || !model || !u40 || !ancestor) return fail(AEM_ERR_INVALID_ARG, "aem_resample_systematic: NULL pointer");
     cudaStream_t s = (cudaStream_t)stream;
     Workspace w = carve(work, n, n_models);
-    split_model_kernel<<<blocks_for(n, 256), 256, 0, s>>>(model, n, n_models, w.kappa, w.lam, ancestor, nullptr);
-    group_kernel<<<1, kGroupThreads, n, s>>>(w.kappa, w.lam, n, 1, n_models, w.perm, w.off, w.counts);
-    gather_weights_kernel<<<blocks_for(n, 256), 256, 0, s>>>(W, w.perm, w.off, n_models, w.Wg);
-    resample_kernel<<<1, kGroupThreads, 0, s>>>(w.Wg, w.perm, w.off, w.counts, n, n_models, u40, 0ull, 0, nullptr,
-                                                w.C, ancestor);
+    if ((rc = stage_kernel_attributes())) return rc;
+    group_kernel<<<1, kGroupThreads, group_smem_bytes(n), s>>>(nullptr, nullptr, model, n, 1, n_models, w.perm, w.off, w.counts, ancestor,
+                                             nullptr);
+    AEM_CUDA_TRY(cudaGetLastError());
+    resample_kernel<<<1, kGroupThreads, resample_smem_bytes(n), s>>>(nullptr, W, w.perm, w.off, n, n_models, u40, 0ull, 0,
+                                                              nullptr, ancestor);
     AEM_CUDA_TRY(cudaGetLastError());
     return AEM_OK;
 }
