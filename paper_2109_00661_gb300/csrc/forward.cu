@@ -1,14 +1,14 @@
 // Batched forward model and Gaussian log-likelihood on sm_103a.
 //
-// One CTA works on one model at a time (grid-stride over models).  For that
-// model it stages, in shared memory, s_n(w_f) = i w_f mu0 sigma_n(w_f) for every
-// frequency node and merged layer (Cole-Cole, Section 2), then its threads
-// sweep the flattened (frequency, Hankel abscissa) index space.  Each item runs
-// the bottom-up TE reflection recursion over the layers (the hot loop: F*K*L
-// layer-steps per model) and weights Im R_0 by the folded Hankel weight; the
-// sums over the abscissae of a frequency are taken in a fixed order (per-warp
-// rows in the FP64 kernel, a per-item value buffer in the FP32 kernel, which
-// also drops the layers under its depth cutoff, depth_cutoff.h).  The
+// One CTA (FP32; grid-stride over models) or cluster of CTAs (FP64; by
+// frequency) works on one model at a time.  For that model it stages, in shared
+// memory, s_n(w_f) = i w_f mu0 sigma_n(w_f) for every frequency node and merged
+// layer (Cole-Cole, Section 2), then its threads sweep the flattened (frequency,
+// Hankel abscissa) index space.  Each item runs the bottom-up TE reflection
+// recursion over the layers (the hot loop: F*K*L layer-steps per model) and
+// weights Im R_0 by the folded Hankel weight; the sums over the abscissae of a
+// frequency are taken in a fixed order from a per-item value buffer.  The FP32
+// kernel also drops the layers under its depth cutoff (depth_cutoff.h).  The
 // epilogue applies the G x F step-off transform and, for
 // the likelihood entry points, the Gaussian log-likelihood of Section 2.3.2
 // (FP32 terms with an FP64 sum in the FP32 kernel, FP64 throughout in the
@@ -16,11 +16,11 @@
 //
 // Recursion used (quasi-static TE mode, exp(+i w t)):
 //   u_n = sqrt(lambda^2 + s_n), Re u_n > 0
-//   r   = (u_n - u_{n+1}) / (u_n + u_{n+1})  (as (s_n - s_{n+1}) / (u_n + u_{n+1})^2 in
-//         the FP64 kernel, from the roots' products in the FP32 one)
+//   r   = (u_n - u_{n+1}) / (u_n + u_{n+1})
 //   R_n = (r + R_{n+1} E) / (1 + r R_{n+1} E),  E = exp(-2 u_{n+1} h_{n+1})
 // carried projectively as R = N / D so the Moebius step needs no division:
 //   N' = r D + N E,  D' = D + r N E.  |D| grows by at most 2x per layer.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -33,109 +33,7 @@
 namespace aem {
 namespace {
 
-constexpr int kThreads = 256;
 constexpr unsigned kFull = 0xffffffffu;
-
-template <class R>
-struct C2 {
-    R x, y;
-};
-
-template <class R>
-__device__ __forceinline__ C2<R> cmul(C2<R> a, C2<R> b) {
-    return {a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x};
-}
-
-// ---- precision-specific primitives ------------------------------------
-struct FP32Ops {
-    using R = float;  // the FP32 path has its own kernel (forward_f32_kernel below)
-};
-
-struct FP64Ops {
-    using R = double;
-    static __device__ __forceinline__ double rsq(double v) { return rsqrt(v); }
-    static __device__ __forceinline__ double sq(double v) { return sqrt(v); }
-    static __device__ __forceinline__ double rcp(double v) { return 1.0 / v; }
-    static __device__ __forceinline__ void expsincos(double re, double im, double *e, double *s, double *c) {
-        *e = exp(re);
-        sincos(im, s, c);
-    }
-};
-
-// Principal square root of (x, y) with y >= 0 (Im s_n >= 0 for a passive
-// medium): q = sqrt((|w| + |x|)/2); the other component is y / (2 q).
-template <class Ops>
-__device__ __forceinline__ C2<typename Ops::R> csqrt_upper(typename Ops::R x, typename Ops::R y) {
-    using R = typename Ops::R;
-    R mod = Ops::sq(x * x + y * y);
-    R t = R(0.5) * (mod + fabs(x));
-    R rq = Ops::rsq(t);
-    R q = t * rq;
-    R o = R(0.5) * y * rq;
-    C2<R> u;
-    u.x = (x >= R(0)) ? q : o;
-    u.y = (x >= R(0)) ? o : q;
-    return u;
-}
-
-// Im R_0 for one (lambda, frequency) pair; s points at this frequency's L
-// layer values, thick at the L-1 finite thicknesses.
-template <class Ops>
-__device__ __forceinline__ typename Ops::R im_r0(typename Ops::R lam, typename Ops::R lam2,
-                                                 const C2<typename Ops::R> *__restrict__ s,
-                                                 const typename Ops::R *__restrict__ thick, int L) {
-    using R = typename Ops::R;
-    C2<R> sb = s[L - 1];
-    C2<R> ub = csqrt_upper<Ops>(lam2 + sb.x, sb.y);
-    C2<R> N = {R(0), R(0)}, D = {R(1), R(0)};
-    bool first = true;
-    for (int n = L - 2; n >= -1; --n) {
-        C2<R> sn, un;
-        if (n >= 0) {
-            sn = s[n];
-            un = csqrt_upper<Ops>(lam2 + sn.x, sn.y);
-        } else {
-            sn = {R(0), R(0)};
-            un = {lam, R(0)};
-        }
-        // r = (s_n - s_below) / (u_n + u_below)^2
-        C2<R> q = {un.x + ub.x, un.y + ub.y};
-        R q2 = q.x * q.x + q.y * q.y;
-        R iq2 = Ops::rcp(q2);
-        R iq4 = iq2 * iq2;
-        C2<R> qq = {q.x * q.x - q.y * q.y, R(-2) * q.x * q.y};  // conj(q^2)
-        C2<R> A = {sn.x - sb.x, sn.y - sb.y};
-        C2<R> r = cmul(A, qq);
-        r.x *= iq4;
-        r.y *= iq4;
-        if (first) {
-            N = r;
-            first = false;
-        } else {
-            // E = exp(-2 u_below h_below)
-            R hb = thick[n + 1];
-            R e, sn_, cs_;
-            Ops::expsincos(R(-2) * ub.x * hb, R(-2) * ub.y * hb, &e, &sn_, &cs_);
-            C2<R> E = {e * cs_, e * sn_};
-            C2<R> P = cmul(N, E);
-            C2<R> rD = cmul(r, D);
-            C2<R> rP = cmul(r, P);
-            N = {rD.x + P.x, rD.y + P.y};
-            D = {D.x + rP.x, D.y + rP.y};
-        }
-        sb = sn;
-        ub = un;
-    }
-    R dd = D.x * D.x + D.y * D.y;
-    return (N.y * D.x - N.x * D.y) * Ops::rcp(dd);
-}
-
-template <class R>
-__device__ __forceinline__ R pow10r(R v);
-template <>
-__device__ __forceinline__ double pow10r<double>(double v) { return exp10(v); }
-
-__device__ __forceinline__ void sincospi_r(double v, double *s, double *c) { sincospi(v, s, c); }
 
 template <class R>
 __device__ __forceinline__ R warp_sum(R v) {
@@ -144,189 +42,327 @@ __device__ __forceinline__ R warp_sum(R v) {
     return v;
 }
 
-template <class Ops>
+template <class R>
 struct ModelsView {
-    using R = typename Ops::R;
     int n, lmax;
     const int8_t *nlayers;
     const R *logsig, *logh, *m, *logtau, *c;
 };
 
-constexpr int kWarps = kThreads / 32;
+// ===================================================================== FP64
+// The plain double-precision form.  This part retires about 1.65 FP64
+// operations a clock per SM (1/78 of FP32), so the kernel's time is its count
+// of FP64 operations, and everything else is free: roots and reciprocals take
+// the hardware's 20-bit estimates and one third-order step, the exponential and
+// the sine and cosine a table in shared memory and a short polynomial, signs,
+// exponents and table indices integer instructions.  About 70 FP64 operations
+// per layer-step (154 with the library's sqrt, rsqrt, division, exp and
+// sincos): 1,024 models of 1..10 layers, 60 frequencies, 200 abscissae, 20.0
+// -> 9.06 ms, at the rate the FP64 pipe allows (71 operations of 19.4 cycles a
+// warp: 9.2 ms).
+//
+// The recursion is the FP32 kernel's (w = sqrt(2) u, the interface coefficient
+// from the roots and their moduli).
+namespace f64 {
 
-// Shared memory layout (dynamic): s_tab[F * LMAX] complex, thick[LMAX],
-// imh[F], T[G * F], lam[K], lam2[K], hw[K], imh_w[kWarps * F].
-// Each warp owns one row of imh_w, so the Hankel sums are formed in a fixed
-// order (no atomics) and the result does not depend on scheduling.
-template <class Ops>
-__global__ void __launch_bounds__(kThreads) forward_kernel(ModelsView<Ops> mv, int F, int G, int K, int cc_form,
-                                                           const typename Ops::R *__restrict__ g_omega,
-                                                           const typename Ops::R *__restrict__ g_lam,
-                                                           const typename Ops::R *__restrict__ g_hw,
-                                                           const typename Ops::R *__restrict__ g_T,
-                                                           typename Ops::R *__restrict__ gates_out,
-                                                           typename Ops::R *__restrict__ imh_out,
-                                                           const double *__restrict__ y_obs, int obs_per,
-                                                           const double *__restrict__ eps_an, double eps_mn,
-                                                           double *__restrict__ ll_out,
-                                                           const int *__restrict__ active,
-                                                           const int8_t *__restrict__ valid) {
-    using R = typename Ops::R;
-    if (active && *active == 0) return;  // a gated launch the caller switched off on the device
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int LM = AEM_MAX_LAYERS;
-    C2<R> *s_tab = reinterpret_cast<C2<R> *>(smem_raw);
-    R *thick = reinterpret_cast<R *>(s_tab + (size_t)F * LM);
-    R *imh = thick + LM;
-    R *Ts = imh + F;
-    R *lam_s = Ts + (size_t)G * F;
-    R *lam2_s = lam_s + K;
-    R *hw_s = lam2_s + K;
-    R *imh_w = hw_s + K;
-    __shared__ R lsig[AEM_MAX_LAYERS], lm[AEM_MAX_LAYERS], ltau[AEM_MAX_LAYERS], lc[AEM_MAX_LAYERS];
-    __shared__ double ll_part[kThreads / 32];
+// 1 / sqrt(v) and 1 / v, v > 0 normal: y (1 + e (1/2 + 3/8 e)), e = 1 - v y^2,
+// and y (1 + e + e^2), e = 1 - v y, leave 5/16 e^3 and e^3 of e < 2^-18.
+__device__ __forceinline__ double rsq(double v) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(v));
+    const double e = fma(-(v * y), y, 1.0);
+    return fma(fma(e, 0.375, 0.5), e * y, y);
+}
+__device__ __forceinline__ double rcp(double v) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(v));
+    const double e = fma(-v, y, 1.0);
+    return fma(fma(e, e, e), y, y);
+}
 
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int i = tid; i < G * F; i += blockDim.x) Ts[i] = g_T[i];
-    for (int k = tid; k < K; k += blockDim.x) {
-        R l = g_lam[k];
-        lam_s[k] = l;
-        lam2_s[k] = l * l;
-        hw_s[k] = g_hw[k];
+// Tables of the complex exponential (Tang 1989's scheme): 2^(j/64), and sine
+// and cosine of j pi / 32.
+struct Tables {
+    double ex[64];
+    double2 sc[64];
+};
+__device__ inline void fill(Tables *t) {
+    for (int j = threadIdx.x; j < 64; j += blockDim.x) {
+        t->ex[j] = exp2(j * 0.015625);
+        sincospi(j * 0.03125, &t->sc[j].x, &t->sc[j].y);
     }
-    const R mu0 = R(kMu0);
-    const int FK = F * K;
+}
 
-    for (int p = blockIdx.x; p < mv.n; p += gridDim.x) {
-        if (valid && !valid[p]) continue;  // a proposal the caller will not use (CTA-uniform)
-        const int L = mv.nlayers[p];
-        __syncthreads();  // previous model's epilogue is done with imh / s_tab
-        if (tid < L) {
-            size_t o = (size_t)p * mv.lmax + tid;
-            lsig[tid] = pow10r<R>(mv.logsig[o]);
-            thick[tid] = pow10r<R>(mv.logh[o]);
-            lm[tid] = mv.m[o];
-            ltau[tid] = pow10r<R>(mv.logtau[o]);
-            lc[tid] = mv.c[o];
+constexpr double kShift = 6755399441055744.0;  // 1.5 * 2^52: the low word of x + kShift is round(x)
+
+// exp(x) for x <= 0 (0 below -700): x = k ln2 / 64 + r, |r| < 0.0055, and
+// e^r - 1 to r^5 (the next term is 4e-17).
+__device__ __forceinline__ double exp_neg(double x, const Tables *t) {
+    const double n = fma(x, 92.332482616893657, kShift);  // 64 / ln 2
+    const int k = __double2loint(n);
+    const double kd = n - kShift;
+    // ln2 / 64, its leading 32 bits and the rest
+    double r = fma(kd, -1.08304246932675596326e-02, x);
+    r = fma(kd, -2.98158582698529370e-12, r);
+    const double r2 = r * r;
+    double q = fma(r, 1.0 / 120.0, 1.0 / 24.0);
+    q = fma(q, r, 1.0 / 6.0);
+    q = fma(q, r, 0.5);
+    const double T = t->ex[k & 63];
+    const double e = fma(fma(r2, q, r), T, T);
+    // -inf <= x <= -700, from the high word's range
+    const bool gone = (unsigned)__double2hiint(x) - 0xc085e000u <= 0xfff00000u - 0xc085e000u;
+    const unsigned hi = (unsigned)__double2hiint(e) + ((unsigned)(k >> 6) << 20);
+    return gone ? 0.0 : __hiloint2double((int)hi, __double2loint(e));
+}
+
+// sine and cosine of x = k pi / 32 + r, |r| < 0.0491: r's to r^7 and r^8, then
+// the table's angle by the addition theorems.
+__device__ __forceinline__ void sincos_tab(double x, const Tables *t, double *s, double *c) {
+    const double n = fma(x, 10.185916357881302, kShift);  // 32 / pi
+    const int k = __double2loint(n);
+    const double kd = n - kShift;
+    // pi / 32 as two doubles; the first product is exact in the fused step
+    double r = fma(kd, -0.098174770424681035, x);
+    r = fma(kd, -3.8270212473354788e-18, r);
+    const double r2 = r * r;
+    double p = fma(r2, -1.0 / 5040.0, 1.0 / 120.0);
+    p = fma(p, r2, -1.0 / 6.0);
+    const double sr = fma(p * r2, r, r);
+    double q = fma(r2, 1.0 / 40320.0, -1.0 / 720.0);
+    q = fma(q, r2, 1.0 / 24.0);
+    q = fma(q, r2, -0.5);
+    const double cr = q * r2;  // cos r - 1
+    const double2 a = t->sc[k & 63];
+    *s = fma(a.y, sr, fma(a.x, cr, a.x));
+    *c = fma(-a.x, sr, fma(a.y, cr, a.y));
+}
+
+struct Root {  // w = sqrt(2 (x + i y)), m = |w|^2 / 2
+    double re, im, m;
+};
+struct Rec {  // per frequency and layer
+    double sx, sy, sy2;
+};
+
+__device__ __forceinline__ Root root(double lam2, const Rec &s) {
+    const double x = lam2 + s.sx;
+    const double v = fma(x, x, s.sy2);
+    Root w;
+    w.m = v * rsq(v);
+    const double t = w.m + fabs(x), rr = rsq(t), p = t * rr, o = s.sy * rr;
+    const bool pos = __double2hiint(x) >= 0;
+    w.re = pos ? p : o;
+    w.im = pos ? o : p;
+    return w;
+}
+
+struct C {
+    double x, y;
+};
+
+// (u_a - u_b) / (u_a + u_b)
+__device__ __forceinline__ C coef(const Root &a, const Root &b) {
+    const double i = rcp(fma(a.im, b.im, fma(a.re, b.re, a.m + b.m)));
+    return {(a.m - b.m) * i, fma(a.im, b.re, -(a.re * b.im)) * i};
+}
+
+// Im R_0 of one (lambda, frequency); rec: the frequency's layers, ha: -sqrt(2) h.
+__device__ __forceinline__ double im_r0(double lam2, double wair, const Rec *__restrict__ rec,
+                                        const double *__restrict__ ha, int L, const Tables *t) {
+    Root b = root(lam2, rec[L - 1]);
+    C N = {0.0, 0.0}, D = {1.0, 0.0};
+#pragma unroll 1
+    for (int n = L - 2; n >= -1; --n) {
+        Root a;
+        if (n >= 0)
+            a = root(lam2, rec[n]);
+        else
+            a = {wair, 0.0, lam2};
+        const C r = coef(a, b);
+        if (n == L - 2) {
+            N = r;
+        } else {
+            const double h = ha[n + 1], ph = h * b.im;
+            const double e = exp_neg(h * b.re, t);
+            double sn, cs;
+            if ((__double2hiint(ph) & 0x7fffffff) < 0x41900000)  // |phase| < 2^26
+                sincos_tab(ph, t, &sn, &cs);
+            else
+                sincos(ph, &sn, &cs);
+            const C E = {e * cs, e * sn};
+            const C P = {fma(N.x, E.x, -(N.y * E.y)), fma(N.x, E.y, N.y * E.x)};
+            const C N1 = {fma(r.x, D.x, fma(-r.y, D.y, P.x)), fma(r.x, D.y, fma(r.y, D.x, P.y))};
+            D = {fma(r.x, P.x, fma(-r.y, P.y, D.x)), fma(r.x, P.y, fma(r.y, P.x, D.y))};
+            N = N1;
         }
-        for (int i = tid; i < kWarps * F; i += blockDim.x) imh_w[i] = R(0);
+        b = a;
+    }
+    return fma(N.y, D.x, -(N.x * D.y)) * rcp(fma(D.x, D.x, D.y * D.y));
+}
+
+}  // namespace f64
+
+constexpr int kThreads64 = 256;
+constexpr int kChunk64 = 8;  // frequencies whose items share the value buffer
+
+// Shared memory (dynamic): vals [kChunk64 * K], lam2 [K], wair [K], hw [K],
+// rec [kChunk64 * lmax], imh [F].
+size_t smem_bytes_f64(int F, int K, int lmax) {
+    return sizeof(double) * ((size_t)kChunk64 * K + 3 * (size_t)K + F) + sizeof(f64::Rec) * (size_t)kChunk64 * lmax;
+}
+
+// A cluster of C CTAs per model, CTA r over the r-th of C equal ranges of the
+// frequencies, a chunk at a time: layer records, items (one per thread and
+// pass, into the value buffer), one fixed-order sum per frequency.  Rank 0
+// collects the spectrum through distributed shared memory and forms gates and
+// likelihood.
+__global__ void __launch_bounds__(kThreads64) forward_f64_kernel(ModelsView<double> mv, int F, int G, int K,
+                                                               int cc_form, const double *__restrict__ g_omega,
+                                                               const double *__restrict__ g_lam,
+                                                               const double *__restrict__ g_hw,
+                                                               const double *__restrict__ g_T,
+                                                               double *__restrict__ gates_out,
+                                                               double *__restrict__ imh_out,
+                                                               const double *__restrict__ y_obs, int obs_per,
+                                                               const double *__restrict__ eps_an, double eps_mn,
+                                                               double *__restrict__ ll_out,
+                                                               const int *__restrict__ active,
+                                                               const int8_t *__restrict__ valid) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    const int C = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+    const int p = blockIdx.x / C;
+    if (active && *active == 0) return;  // a gated launch the caller switched off on the device
+    if (valid && !valid[p]) return;      // a proposal the caller will not use (the whole cluster)
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    double *vals = reinterpret_cast<double *>(smem_raw);
+    double *lam2 = vals + (size_t)kChunk64 * K, *wair = lam2 + K, *hw = wair + K, *imh = hw + K;
+    f64::Rec *rec = reinterpret_cast<f64::Rec *>(imh + F);
+    __shared__ f64::Tables tab;
+    __shared__ double lsig[AEM_MAX_LAYERS], lm[AEM_MAX_LAYERS], ltau[AEM_MAX_LAYERS], lc[AEM_MAX_LAYERS],
+        ha[AEM_MAX_LAYERS];
+    __shared__ double ll_part[2];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int L = mv.nlayers[p];
+    f64::fill(&tab);
+    for (int k = tid; k < K; k += kThreads64) {
+        const double l = g_lam[k];
+        lam2[k] = l * l;
+        wair[k] = 1.4142135623730951 * l;
+        hw[k] = g_hw[k];
+    }
+    if (tid < L) {
+        const size_t o = (size_t)p * mv.lmax + tid;
+        lsig[tid] = exp10(mv.logsig[o]);
+        ha[tid] = -1.4142135623730951 * exp10(mv.logh[o]);
+        lm[tid] = mv.m[o];
+        ltau[tid] = exp10(mv.logtau[o]);
+        lc[tid] = mv.c[o];
+    }
+    const int f0 = F * rank / C, f1 = F * (rank + 1) / C;
+    for (int fc = f0; fc < f1; fc += kChunk64) {
+        const int nf = min(kChunk64, f1 - fc);
         __syncthreads();
-        // Cole-Cole per (frequency, layer): x = (w tau)^c e^{i pi c / 2}
-        for (int i = tid; i < F * L; i += blockDim.x) {
-            int f = i / L, n = i - f * L;
-            R w = g_omega[f];
-            R sig = lsig[n], mm = lm[n];
-            R sr = sig, si = R(0);
-            if (mm != R(0)) {
-                R cc = lc[n];
-                R mag = exp(cc * log(w * ltau[n]));
-                R sp, cp;
-                sincospi_r(R(0.5) * cc, &sp, &cp);
-                R xr = R(1) + mag * cp, xi = mag * sp;  // 1 + x
-                R den = xr * xr + xi * xi;
+        // Cole-Cole per (frequency, layer): x = (w tau)^c e^{i pi c / 2}, s = i w mu0 sigma
+        for (int i = tid; i < nf * L; i += kThreads64) {
+            const int f = i / L, n = i - f * L;
+            const double w = g_omega[fc + f];
+            const double sig = lsig[n], mm = lm[n];
+            double sr = sig, si = 0.0;
+            if (mm != 0.0) {
+                const double cc = lc[n];
+                const double mag = exp(cc * log(w * ltau[n]));
+                double sp, cp;
+                sincospi(0.5 * cc, &sp, &cp);
+                const double xr = 1.0 + mag * cp, xi = mag * sp;  // 1 + x
+                const double den = xr * xr + xi * xi;
                 // every form is written without cancellation (see the FP32 kernel)
                 if (cc_form == AEM_CC_PAPER) {
                     // sigma_inf ((1 - m) + x) / (1 + x)
-                    sr = sig * (((R(1) - mm) + mag * cp) * xr + xi * xi) / den;
+                    sr = sig * (((1.0 - mm) + mag * cp) * xr + xi * xi) / den;
                     si = sig * (mm * xi / den);
                 } else if (cc_form == AEM_CC_LITERAL) {
                     // sigma_0 (1 + (1 - m) x) / (1 + x)
-                    R br = R(1) + (R(1) - mm) * mag * cp, bi = (R(1) - mm) * mag * sp;
+                    const double br = 1.0 + (1.0 - mm) * mag * cp, bi = (1.0 - mm) * mag * sp;
                     sr = sig * (br * xr + bi * xi) / den;
                     si = -sig * (mm * xi / den);
                 } else {
                     // sigma_0 (1 + x) / (1 + (1 - m) x)
-                    R br = R(1) + (R(1) - mm) * mag * cp, bi = (R(1) - mm) * mag * sp;
-                    R bd = br * br + bi * bi;
+                    const double br = 1.0 + (1.0 - mm) * mag * cp, bi = (1.0 - mm) * mag * sp;
+                    const double bd = br * br + bi * bi;
                     sr = sig * (xr * br + xi * bi) / bd;
                     si = sig * (mm * xi / bd);
                 }
             }
-            // s = i w mu0 sigma
-            s_tab[(size_t)f * LM + n] = {-w * mu0 * si, w * mu0 * sr};
+            const double sx = -w * kMu0 * si, sy = w * kMu0 * sr;
+            rec[f * L + n] = {sx, sy, sy * sy};
         }
         __syncthreads();
-
-        // Hot loop over (frequency, abscissa) items.
-        int f = tid / K, k = tid - (tid / K) * K;
-        for (int base = 0; base < FK; base += blockDim.x) {
-            const int item = base + tid;
-            R val = R(0);
-            int fl = -1;
-            if (item < FK) {
-                fl = f;
-                val = hw_s[k] * im_r0<Ops>(lam_s[k], lam2_s[k], s_tab + (size_t)f * LM, thick, L);
-            }
-            // segmented warp reduction over lanes that share a frequency
-            unsigned pending = __ballot_sync(kFull, fl >= 0);
-            while (pending) {
-                int leader = __ffs(pending) - 1;
-                int fsel = __shfl_sync(kFull, fl, leader);
-                R part = warp_sum<R>(fl == fsel ? val : R(0));
-                if (lane == leader) imh_w[warp * F + fsel] += part;
-                pending &= ~__ballot_sync(kFull, fl == fsel);
-            }
-            k += blockDim.x;
+        int f = tid / K, k = tid - f * K;
+        for (int item = tid; item < nf * K; item += kThreads64) {
+            vals[item] = hw[k] * f64::im_r0(lam2[k], wair[k], rec + f * L, ha, L, &tab);
+            k += kThreads64;
             while (k >= K) {
                 k -= K;
                 ++f;
             }
         }
         __syncthreads();
-        for (int j = tid; j < F; j += blockDim.x) {
-            R acc = R(0);
-#pragma unroll
-            for (int w = 0; w < kWarps; ++w) acc += imh_w[w * F + j];
-            imh[j] = acc;
+        // a warp per frequency: lanes stride its values, then a shuffle tree
+        for (int j = warp; j < nf; j += kThreads64 / 32) {
+            double acc = 0.0;
+            for (int q = lane; q < K; q += 32) acc += vals[j * K + q];
+            acc = warp_sum<double>(acc);
+            if (lane == 0) imh[fc + j] = acc;
+        }
+    }
+    if (C > 1) {
+        cl.sync();
+        if (rank == 0)
+            for (int j = f1 + tid; j < F; j += kThreads64) {
+                int r = (int)((long long)j * C / F);
+                while (r + 1 < C && F * (r + 1) / C <= j) ++r;
+                while (F * r / C > j) --r;
+                imh[j] = *cl.map_shared_rank(&imh[j], r);
+            }
+        cl.sync();  // rank 0 has read the others' spectra
+        if (rank != 0) return;
+    }
+    __syncthreads();
+    if (imh_out)
+        for (int j = tid; j < F; j += kThreads64) imh_out[(size_t)p * F + j] = imh[j];
+    double term = 0.0;
+    if (tid < G && (gates_out || ll_out)) {
+        double acc = 0.0;
+        for (int j = 0; j < F; ++j) acc += g_T[(size_t)tid * F + j] * imh[j];
+        if (gates_out) gates_out[(size_t)p * G + tid] = acc;
+        if (ll_out) {
+            const double ea = eps_an[tid];
+            const double v = ea * ea + (eps_mn * acc) * (eps_mn * acc);
+            // models [s*obs_per, (s+1)*obs_per) share sounding s's data
+            const double *yo = y_obs + (obs_per > 0 ? (size_t)(p / obs_per) * G : 0);
+            const double rr = yo[tid] - acc;
+            term = rr * rr / v + log(2.0 * kPi * v);
+        }
+    }
+    if (ll_out) {
+        if (warp * 32 < G) {
+            const double t = warp_sum<double>(term);
+            if (lane == 0) ll_part[warp] = t;
         }
         __syncthreads();
-
-        // Epilogue: gates, optional Im H, optional log-likelihood.
-        double term = 0.0;
-        if (tid < G) {
-            R acc = R(0);
-            for (int j = 0; j < F; ++j) acc += Ts[tid * F + j] * imh[j];
-            if (gates_out) gates_out[(size_t)p * G + tid] = acc;
-            if (ll_out) {
-                double yh = (double)acc;
-                double ea = eps_an[tid];
-                double v = ea * ea + (eps_mn * yh) * (eps_mn * yh);
-                // models [s*obs_per, (s+1)*obs_per) share sounding s's data
-                const double *yo = y_obs + (obs_per > 0 ? (size_t)(p / obs_per) * G : 0);
-                double rr = yo[tid] - yh;
-                term = rr * rr / v + log(2.0 * kPi * v);
-            }
-        }
-        if (imh_out)
-            for (int j = tid; j < F; j += blockDim.x) imh_out[(size_t)p * F + j] = imh[j];
-        if (ll_out) {
-            if (warp * 32 < G) {
-                double t = warp_sum<double>(term);
-                if (lane == 0) ll_part[warp] = t;
-            }
-            __syncthreads();
-            if (tid == 0) {
-                double acc = 0.0;
-                for (int w = 0; w * 32 < G; ++w) acc += ll_part[w];
-                ll_out[p] = -0.5 * acc;
-            }
+        if (tid == 0) {
+            double acc = 0.0;
+            for (int w = 0; w * 32 < G; ++w) acc += ll_part[w];
+            ll_out[p] = -0.5 * acc;
         }
     }
 }
 
-template <class Ops>
-size_t smem_bytes(int F, int G, int K) {
-    using R = typename Ops::R;
-    return sizeof(C2<R>) * (size_t)F * AEM_MAX_LAYERS +
-           sizeof(R) * (AEM_MAX_LAYERS + F + (size_t)G * F + 3 * (size_t)K + (size_t)kWarps * F);
-}
-
-template <class Ops, class Models>
-int launch_forward(const aem_system *sys, const Models *models, typename Ops::R *gates, typename Ops::R *imh,
-                   const double *y_obs, int obs_per, const double *eps_an, double eps_mn, double *ll, void *stream,
-                   const typename Ops::R *omega, const typename Ops::R *lam, const typename Ops::R *hw,
-                   const typename Ops::R *T, const char *name, const int *active = nullptr,
-                   const int8_t *valid = nullptr) {
+int launch_forward_f64(const aem_system *sys, const aem_models_f64 *models, double *gates, double *imh,
+                       const double *y_obs, int obs_per, const double *eps_an, double eps_mn, double *ll, void *stream,
+                       const char *name, const int *active = nullptr, const int8_t *valid = nullptr) {
     if (!sys || !models) return fail(AEM_ERR_INVALID_ARG, std::string(name) + ": NULL system or models");
     if (models->n_models < 0 || models->lmax < 1 || models->lmax > AEM_MAX_LAYERS)
         return fail(AEM_ERR_INVALID_ARG, std::string(name) + ": n_models < 0 or lmax outside 1..AEM_MAX_LAYERS");
@@ -336,24 +372,37 @@ int launch_forward(const aem_system *sys, const Models *models, typename Ops::R 
         return fail(AEM_ERR_INVALID_ARG, std::string(name) + ": NULL model array");
     if (ll && (!y_obs || !eps_an)) return fail(AEM_ERR_INVALID_ARG, std::string(name) + ": NULL y_obs or eps_an");
     const SystemTables &h = sys->host;
-    ModelsView<Ops> mv{models->n_models, models->lmax, models->nlayers, models->logsig, models->logh,
-                       models->m, models->logtau, models->c};
-    size_t smem = smem_bytes<Ops>(h.F, h.G, h.K);
-    auto kern = forward_kernel<Ops>;
-    // always: the static shared memory counts against the 48 KB default too
-    AEM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    int per_sm = 0;
-    AEM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, smem));
-    if (per_sm < 1) per_sm = 1;
-    long long grid = (long long)sys->num_sms * per_sm;
-    if (grid > models->n_models) grid = models->n_models;
-    kern<<<(unsigned)grid, kThreads, smem, (cudaStream_t)stream>>>(mv, h.F, h.G, h.K, h.cc_form, omega, lam, hw, T,
-                                                                   gates, imh, y_obs, obs_per, eps_an, eps_mn, ll,
-                                                                   active, valid);
-    AEM_CUDA_TRY(cudaGetLastError());
+    const ModelsView<double> mv{models->n_models, models->lmax, models->nlayers, models->logsig, models->logh,
+                                models->m, models->logtau, models->c};
+    const size_t smem = smem_bytes_f64(h.F, h.K, models->lmax);
+    // the largest any system needs, so that no caller lowers it under another
+    AEM_CUDA_TRY(cudaFuncSetAttribute(forward_f64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)smem_bytes_f64(AEM_MAX_FREQ, AEM_MAX_HANKEL, AEM_MAX_LAYERS)));
+    // Models are split over clusters of up to eight CTAs until there are 16 CTAs
+    // per SM to balance the last wave with (every CTA keeps at least two
+    // frequencies).
+    int C = 1;
+    while (C < 8 && (long long)models->n_models * C < 16LL * sys->num_sms && h.F >= 4 * C) C *= 2;
+    if ((long long)models->n_models * C > 0x7fffffffLL)
+        return fail(AEM_ERR_INVALID_ARG, std::string(name) + ": too many models");
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(models->n_models * C), 1, 1);
+    cfg.blockDim = dim3(kThreads64, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = (cudaStream_t)stream;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)C;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = C > 1 ? 1 : 0;
+    AEM_CUDA_TRY(cudaLaunchKernelEx(&cfg, forward_f64_kernel, mv, h.F, h.G, h.K, h.cc_form,
+                                    (const double *)sys->d_omega_d, (const double *)sys->d_lam_d,
+                                    (const double *)sys->d_hw_d, (const double *)sys->d_T_d, gates, imh, y_obs, obs_per,
+                                    eps_an, eps_mn, ll, active, valid));
     return AEM_OK;
 }
-
 
 // ===================================================================== FP32
 // FP32 hot path.  Each thread carries TWO Hankel abscissae of the same
@@ -592,7 +641,7 @@ __host__ __device__ inline int vals_words(int F, int K2) {
 // The order of every sum is fixed by the item indices alone.  (The throughput
 // system's 60 x 100 items take one round.)
 template <int NT, int MINB, bool DYN, bool SPEC>
-__global__ void __launch_bounds__(NT, MINB) forward_f32_kernel(ModelsView<FP32Ops> mv, int F, int G, int K,
+__global__ void __launch_bounds__(NT, MINB) forward_f32_kernel(ModelsView<float> mv, int F, int G, int K,
                                                                int cc_form, int LS, float len,
                                                                const float *__restrict__ g_omega,
                                                                const float *__restrict__ g_lam,
@@ -913,7 +962,7 @@ constexpr int kNumBase = sizeof(kF32Shapes) / sizeof(kF32Shapes[0]);
 constexpr int kNumF32Shapes = 2 * kNumBase;
 
 template <int NT, int MINB, bool DYN, bool SPEC>
-int launch_shape(const aem_system *sys, const ModelsView<FP32Ops> &mv, int LS, float *gates, float *imh,
+int launch_shape(const aem_system *sys, const ModelsView<float> &mv, int LS, float *gates, float *imh,
                  const double *y_obs, int obs_per, const double *eps_an, double eps_mn, double *ll,
                  cudaStream_t stream, int *counter_ext, const int *active, unsigned long long *steps,
                  const int8_t *valid) {
@@ -945,7 +994,7 @@ int launch_shape(const aem_system *sys, const ModelsView<FP32Ops> &mv, int LS, f
     return AEM_OK;
 }
 
-int launch_shape_index(int idx, const aem_system *sys, const ModelsView<FP32Ops> &mv, int LS, float *gates,
+int launch_shape_index(int idx, const aem_system *sys, const ModelsView<float> &mv, int LS, float *gates,
                        float *imh, const double *y_obs, int obs_per, const double *eps_an, double eps_mn, double *ll,
                        cudaStream_t stream, int *counter_ext = nullptr, const int *active = nullptr,
                        unsigned long long *steps = nullptr, const int8_t *valid = nullptr) {
@@ -976,7 +1025,7 @@ int launch_forward_f32(const aem_system *sys, const Models *models, float *gates
     if (!models->nlayers || !models->logsig || !models->logh || !models->m || !models->logtau || !models->c)
         return fail(AEM_ERR_INVALID_ARG, std::string(name) + ": NULL model array");
     if (ll && (!y_obs || !eps_an)) return fail(AEM_ERR_INVALID_ARG, std::string(name) + ": NULL y_obs or eps_an");
-    ModelsView<FP32Ops> mv{models->n_models, models->lmax, models->nlayers, models->logsig, models->logh,
+    ModelsView<float> mv{models->n_models, models->lmax, models->nlayers, models->logsig, models->logh,
                            models->m, models->logtau, models->c};
     const int LS = models->lmax;
     // No shape recorded: the smallest CTAs for batches that fill the chip;
@@ -994,10 +1043,8 @@ namespace aem {
 int loglik_f64_soundings(const aem_system *sys, const aem_models_f64 *models, const double *y_obs,
                          int models_per_sounding, const double *eps_an, double eps_mn, double *ll,
                          cudaStream_t stream, const int *active, const int8_t *valid) {
-    return launch_forward<FP64Ops>(sys, models, (double *)nullptr, (double *)nullptr, y_obs, models_per_sounding,
-                                   eps_an, eps_mn, ll, (void *)stream, sys ? sys->d_omega_d : nullptr,
-                                   sys ? sys->d_lam_d : nullptr, sys ? sys->d_hw_d : nullptr,
-                                   sys ? sys->d_T_d : nullptr, "loglik (SMC, FP64)", active, valid);
+    return launch_forward_f64(sys, models, nullptr, nullptr, y_obs, models_per_sounding, eps_an, eps_mn, ll,
+                              (void *)stream, "loglik (SMC, FP64)", active, valid);
 }
 int loglik_f32_soundings(const aem_system *sys, const aem_models_f32 *models, const double *y_obs,
                          int models_per_sounding, const double *eps_an, double eps_mn, double *ll,
@@ -1023,9 +1070,7 @@ extern "C" int aem_forward_f32_count(const aem_system *sys, const aem_models_f32
 
 extern "C" int aem_forward_f64(const aem_system *sys, const aem_models_f64 *models, double *gates, double *imh,
                                void *stream) {
-    return launch_forward<FP64Ops>(sys, models, gates, imh, nullptr, 0, nullptr, 0.0, nullptr, stream,
-                                   sys ? sys->d_omega_d : nullptr, sys ? sys->d_lam_d : nullptr,
-                                   sys ? sys->d_hw_d : nullptr, sys ? sys->d_T_d : nullptr, "aem_forward_f64");
+    return launch_forward_f64(sys, models, gates, imh, nullptr, 0, nullptr, 0.0, nullptr, stream, "aem_forward_f64");
 }
 
 extern "C" int aem_loglik_f32(const aem_system *sys, const aem_models_f32 *models, const double *y_obs,
@@ -1037,9 +1082,7 @@ extern "C" int aem_loglik_f32(const aem_system *sys, const aem_models_f32 *model
 extern "C" int aem_loglik_f64(const aem_system *sys, const aem_models_f64 *models, const double *y_obs,
                               const double *eps_an, double eps_mn, double *ll, double *gates, void *stream) {
     if (!ll && models && models->n_models > 0) return fail(AEM_ERR_INVALID_ARG, "aem_loglik_f64: ll is NULL");
-    return launch_forward<FP64Ops>(sys, models, gates, nullptr, y_obs, 0, eps_an, eps_mn, ll, stream,
-                                   sys ? sys->d_omega_d : nullptr, sys ? sys->d_lam_d : nullptr,
-                                   sys ? sys->d_hw_d : nullptr, sys ? sys->d_T_d : nullptr, "aem_loglik_f64");
+    return launch_forward_f64(sys, models, gates, nullptr, y_obs, 0, eps_an, eps_mn, ll, stream, "aem_loglik_f64");
 }
 
 namespace aem {
@@ -1070,7 +1113,7 @@ extern "C" int aem_autotune_forward(aem_system *sys, const aem_models_f32 *sampl
         return fail(AEM_ERR_INVALID_ARG, "aem_autotune_forward: NULL model array");
     cudaStream_t s = (cudaStream_t)stream;
     const int LS = sample->lmax;
-    ModelsView<FP32Ops> mv{sample->n_models, sample->lmax, sample->nlayers, sample->logsig, sample->logh,
+    ModelsView<float> mv{sample->n_models, sample->lmax, sample->nlayers, sample->logsig, sample->logh,
                            sample->m, sample->logtau, sample->c};
     float *gates = nullptr;
     AEM_CUDA_TRY(cudaMallocAsync((void **)&gates, sizeof(float) * (size_t)sample->n_models * sys->host.G, s));
