@@ -29,17 +29,25 @@ GATES_BF16_SPLIT = 2
 F32_SHAPES = 10  # AEM_F32_SHAPES: launch shapes of the FP32 forward kernel
 
 
+_have_cuda = False
+
+
 def _torch():
+    # a device found once stays: asking again costs microseconds per call
+    global _have_cuda
     import torch
-    if not torch.cuda.is_available():
-        raise AEMError("paper_2109_00661_gb300 needs a CUDA device; there is no CPU path")
+    if not _have_cuda:
+        if not torch.cuda.is_available():
+            raise AEMError("paper_2109_00661_gb300 needs a CUDA device; there is no CPU path")
+        _have_cuda = True
     return torch
 
 
 def _stream_ptr(stream):
+    if stream is not None:
+        return ctypes.c_void_p(stream.cuda_stream)
     torch = _torch()
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return ctypes.c_void_p(s.cuda_stream)
+    return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
 
 
 def _dptr(t):
@@ -66,6 +74,22 @@ class System:
         self.F, self.G, self.K = int(n_freq), len(self._times), int(n_hankel)
         self.loop_radius, self.height, self.current, self.cc_form = loop_radius, height, current, cc_form
         self.times = self._times.copy()
+        self._eps = {}
+
+    def _eps_vector(self, eps_an, dev):
+        """The additive noise floor of every gate, eps_an, as a device vector.
+        Built once per value (at most 16 of them) and kept with the system: a
+        fill per call costs 10 us of host time, copying a host scalar waits for
+        the stream.  The values are on the device before another stream can
+        read them, and close() drains the device before they go."""
+        torch = _torch()
+        e = self._eps.get((eps_an, dev))
+        if e is None:
+            e = torch.full((self.G,), eps_an, dtype=torch.float64, device=dev)
+            if len(self._eps) < 16 and not torch.cuda.is_current_stream_capturing():
+                torch.cuda.current_stream(dev).synchronize()
+                self._eps[(eps_an, dev)] = e
+        return e
 
     @property
     def handle(self):
@@ -106,8 +130,9 @@ class System:
 
     def close(self):
         if getattr(self, "_h", None) is not None and self._h.value:
-            _lib.load().aem_system_destroy(self._h)
+            _lib.load().aem_system_destroy(self._h)  # cudaFree: waits for the device
             self._h = ctypes.c_void_p()
+            self._eps.clear()
 
     def __del__(self):
         try:
@@ -185,7 +210,10 @@ def forward_layer_steps(system, models, stream=None):
 def _obs(y_obs, eps_an, system, dev):
     torch = _torch()
     y = torch.as_tensor(y_obs, dtype=torch.float64, device=dev).contiguous()
-    e = torch.as_tensor(eps_an, dtype=torch.float64, device=dev).expand(system.G).contiguous()
+    if isinstance(eps_an, (int, float)):
+        e = system._eps_vector(float(eps_an), dev)
+    else:
+        e = torch.as_tensor(eps_an, dtype=torch.float64, device=dev).expand(system.G).contiguous()
     return y, e
 
 
@@ -247,8 +275,7 @@ def _loglik(fn, models, dtype, y_obs, eps_an, eps_mn, system, want_gates, stream
     ms = _models_struct(models, dtype)
     P = ms.n_models
     dev = models["logsig"].device
-    y_obs = torch.as_tensor(y_obs, dtype=torch.float64, device=dev).contiguous()
-    eps_an = torch.as_tensor(eps_an, dtype=torch.float64, device=dev).expand(system.G).contiguous()
+    y_obs, eps_an = _obs(y_obs, eps_an, system, dev)
     ll = torch.empty(P, dtype=torch.float64, device=dev)
     gates = torch.empty((P, system.G), dtype=dtype, device=dev) if want_gates else None
     check(fn(system.handle, ctypes.byref(ms), _dptr(y_obs), _dptr(eps_an), float(eps_mn), _dptr(ll), _dptr(gates),
@@ -275,8 +302,7 @@ def loglik_grad_f32(system, models, y_obs, eps_an, eps_mn, stream=None):
     ms = _models_struct(models, torch.float32)
     P, lmax = ms.n_models, ms.lmax
     dev = models["logsig"].device
-    y_obs = torch.as_tensor(y_obs, dtype=torch.float64, device=dev).contiguous()
-    eps_an = torch.as_tensor(eps_an, dtype=torch.float64, device=dev).expand(system.G).contiguous()
+    y_obs, eps_an = _obs(y_obs, eps_an, system, dev)
     ll = torch.empty(P, dtype=torch.float64, device=dev)
     grad = torch.empty((P, lmax, 5), dtype=torch.float32, device=dev)
     check(_lib.load().aem_loglik_grad_f32(system.handle, ctypes.byref(ms), _dptr(y_obs), _dptr(eps_an),

@@ -3,6 +3,7 @@
 
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <string>
 #include <vector>
 
@@ -22,6 +23,31 @@ int cuda_fail(cudaError_t err, const char *what);
         cudaError_t _e = (expr);                                  \
         if (_e != cudaSuccess) return ::aem::cuda_fail(_e, #expr); \
     } while (0)
+
+// How many CTAs of a kernel fit an SM with that much dynamic shared memory:
+// asked of the runtime once and kept in *slot (0: not asked yet), with the
+// kernel's dynamic shared memory limit raised to all that its static share
+// leaves (the same value whoever asks, so no caller lowers it under another)
+// and the SM's unified storage given to shared memory.  Setting both and asking
+// on every launch cost 6 us.
+template <class Kernel>
+int resident_ctas(std::atomic<int> *slot, Kernel kern, int threads, size_t smem, int device, int *out) {
+    int n = slot->load(std::memory_order_relaxed);
+    if (n == 0) {
+        cudaFuncAttributes fa{};
+        int optin = 0;
+        AEM_CUDA_TRY(cudaFuncGetAttributes(&fa, kern));
+        AEM_CUDA_TRY(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device));
+        AEM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          optin - (int)fa.sharedSizeBytes));
+        AEM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                          (int)cudaSharedmemCarveoutMaxShared));
+        AEM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, threads, smem));
+        if (n > 0) slot->store(n, std::memory_order_relaxed);
+    }
+    *out = n;
+    return AEM_OK;
+}
 
 // Host-side tables (double) and their device copies (float and double).
 struct SystemTables {
@@ -57,6 +83,11 @@ struct aem_system {
     // launch shape of the FP32 forward kernel per lmax (index into its shape
     // table, 0 = default), set by aem_autotune_forward / aem_forward_shape
     int f32_shape[AEM_MAX_LAYERS + 1] = {};
+    // CTAs per SM of each kernel, asked once (resident_ctas): the FP32 forward
+    // shapes and the adjoint per lmax, the tensor-core transform per mode
+    mutable std::atomic<int> fwd_ctas[AEM_F32_SHAPES][AEM_MAX_LAYERS + 1] = {};
+    mutable std::atomic<int> grad_ctas[AEM_MAX_LAYERS + 1] = {};
+    mutable std::atomic<int> tc_ctas[3] = {};
     // the FP32 forward kernel's depth cutoff (aem_system_set_depth_cutoff):
     // attenuation exponent, 0 = the whole stack always
     float depth_att = 20.f;

@@ -961,7 +961,7 @@ constexpr F32Shape kF32Shapes[] = {AEM_SHAPES(AEM_SHAPE)};
 constexpr int kNumBase = sizeof(kF32Shapes) / sizeof(kF32Shapes[0]);
 constexpr int kNumF32Shapes = 2 * kNumBase;
 
-template <int NT, int MINB, bool DYN, bool SPEC>
+template <int IDX, int NT, int MINB, bool DYN, bool SPEC>
 int launch_shape(const aem_system *sys, const ModelsView<float> &mv, int LS, float *gates, float *imh,
                  const double *y_obs, int obs_per, const double *eps_an, double eps_mn, double *ll,
                  cudaStream_t stream, int *counter_ext, const int *active, unsigned long long *steps,
@@ -969,14 +969,8 @@ int launch_shape(const aem_system *sys, const ModelsView<float> &mv, int LS, flo
     const SystemTables &h = sys->host;
     auto kern = forward_f32_kernel<NT, MINB, DYN, SPEC>;
     const size_t smem = smem_bytes_f32(h.F, h.G, h.K, LS);
-    // always: the static shared memory counts against the 48 KB default too
-    AEM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    // the kernel reads its tables from shared memory only: give the SM's
-    // unified L1/shared storage to shared memory so more CTAs stay resident
-    AEM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                      (int)cudaSharedmemCarveoutMaxShared));
     int per_sm = 0;
-    AEM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NT, smem));
+    if (const int rc = resident_ctas(&sys->fwd_ctas[IDX][LS], kern, NT, smem, sys->device, &per_sm)) return rc;
     if (per_sm < 1) return fail(AEM_ERR_UNSUPPORTED, "forward kernel: launch shape does not fit on an SM");
     long long grid = (long long)sys->num_sms * per_sm;
     if (grid > mv.n) grid = mv.n;
@@ -1000,10 +994,10 @@ int launch_shape_index(int idx, const aem_system *sys, const ModelsView<float> &
                        unsigned long long *steps = nullptr, const int8_t *valid = nullptr) {
 #define AEM_SHAPE(I, NT, MINB, SPEC)                                                                                 \
     case I:                                                                                                        \
-        return launch_shape<NT, MINB, false, SPEC>(sys, mv, LS, gates, imh, y_obs, obs_per, eps_an, eps_mn, ll, stream, \
+        return launch_shape<I, NT, MINB, false, SPEC>(sys, mv, LS, gates, imh, y_obs, obs_per, eps_an, eps_mn, ll, stream, \
                                              counter_ext, active, steps, valid);                                   \
     case I + kNumBase:                                                                                             \
-        return launch_shape<NT, MINB, true, SPEC>(sys, mv, LS, gates, imh, y_obs, obs_per, eps_an, eps_mn, ll, stream,  \
+        return launch_shape<I + kNumBase, NT, MINB, true, SPEC>(sys, mv, LS, gates, imh, y_obs, obs_per, eps_an, eps_mn, ll, stream,  \
                                             counter_ext, active, steps, valid);
     switch (idx) {
         AEM_SHAPES(AEM_SHAPE)

@@ -525,6 +525,35 @@ __global__ void gates_fp32_kernel(TcArgs a) {
 
 inline int round_up(int x, int m) { return (x + m - 1) / m * m; }
 
+// CTAs per SM of the tensor-core transform.  The occupancy query has reported
+// one CTA per SM for the TF32 tile where two fit (the profiler's shared-memory
+// limit says two); take the count the SM's shared memory, registers and tensor
+// memory allow when it is larger.
+template <class Kernel>
+int tc_resident(const aem_system *sys, int mode, Kernel kern, size_t smem, int ncols, int *out) {
+    int per_sm = sys->tc_ctas[mode].load(std::memory_order_relaxed);
+    if (per_sm == 0) {
+        std::atomic<int> asked{0};
+        if (const int rc = resident_ctas(&asked, kern, kThreads, smem, sys->device, &per_sm)) return rc;
+        if (per_sm > 0) {
+            int smem_sm = 0, reserved = 0;
+            AEM_CUDA_TRY(cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, sys->device));
+            AEM_CUDA_TRY(cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, sys->device));
+            cudaFuncAttributes fa{};
+            AEM_CUDA_TRY(cudaFuncGetAttributes(&fa, kern));
+            int by_smem = smem_sm / (int)(smem + (size_t)reserved);
+            const int by_regs = fa.numRegs > 0 ? 65536 / (fa.numRegs * kThreads) : 1;
+            const int by_tmem = 512 / ncols;
+            if (by_smem > by_regs) by_smem = by_regs;
+            if (by_smem > by_tmem) by_smem = by_tmem;
+            if (by_smem > per_sm) per_sm = by_smem;
+            sys->tc_ctas[mode].store(per_sm, std::memory_order_relaxed);
+        }
+    }
+    *out = per_sm;
+    return AEM_OK;
+}
+
 }  // namespace
 
 int gates_from_spectrum(const aem_system *sys, const float *imh, int P, int mode, const double *y_obs,
@@ -549,30 +578,9 @@ int gates_from_spectrum(const aem_system *sys, const float *imh, int P, int mode
     const size_t smem = (size_t)2 * (kTM + a.N) * a.KP * ES + 1024 + sizeof(float2) * 2 * AEM_MAX_GATES +
                         sizeof(float) * AEM_MAX_GATES + sizeof(float2) * kTM + 64;
     auto kern = tf32 ? gates_tc_kernel<0> : gates_tc_kernel<1>;
-    AEM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    // all of the SM's unified storage to shared memory, so that several CTAs
-    // (two for the TF32 split's 84 KB, five for the BF16 split's 43 KB) stay resident
-    AEM_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                      (int)cudaSharedmemCarveoutMaxShared));
     int per_sm = 0;
-    AEM_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, smem));
+    if (const int rc = tc_resident(sys, mode, kern, smem, a.ncols, &per_sm)) return rc;
     if (per_sm < 1) return fail(AEM_ERR_UNSUPPORTED, "aem_gates_from_spectrum: tile does not fit in shared memory");
-    // the occupancy query has reported one CTA per SM for the TF32 tile where
-    // two fit (the profiler's shared-memory limit says two); take the count
-    // the SM's shared memory, registers and tensor memory allow when it is larger
-    {
-        int smem_sm = 0, reserved = 0;
-        AEM_CUDA_TRY(cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, sys->device));
-        AEM_CUDA_TRY(cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, sys->device));
-        cudaFuncAttributes fa{};
-        AEM_CUDA_TRY(cudaFuncGetAttributes(&fa, kern));
-        int by_smem = smem_sm / (int)(smem + (size_t)reserved);
-        const int by_regs = fa.numRegs > 0 ? 65536 / (fa.numRegs * kThreads) : 1;
-        const int by_tmem = 512 / a.ncols;
-        if (by_smem > by_regs) by_smem = by_regs;
-        if (by_smem > by_tmem) by_smem = by_tmem;
-        if (by_smem > per_sm) per_sm = by_smem;
-    }
     const int ntiles = (P + kTM - 1) / kTM;
     int grid = sys->num_sms * per_sm;
     if (grid > ntiles) grid = ntiles;
