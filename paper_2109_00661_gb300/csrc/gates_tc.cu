@@ -37,6 +37,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <type_traits>
 
 #include "aem_internal.h"
 
@@ -161,6 +162,15 @@ struct Split<0> {
         const float r = x - __uint_as_float(hi);
         asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(lo) : "f"(r));
     }
+    // The same for finite x in integers: round to 11 bits, ties away, by adding
+    // half of the 13 dropped ones (the conversion takes some four instructions).
+    // The tensor core ignores an operand's low 13 bits, so lo needs no mask.  A
+    // NaN's bits would carry out of the format: the caller converts those above.
+    __device__ static void run_finite(float x, uint32_t &hi, uint32_t &lo) {
+        hi = (__float_as_uint(x) + 0x1000u) & 0xffffe000u;
+        lo = __float_as_uint(x - __uint_as_float(hi)) + 0x1000u;
+    }
+    static constexpr float kFinite = 1.7e38f;  // half of the largest, so that hi stays finite
 };
 template <>
 struct Split<1> {
@@ -172,6 +182,8 @@ struct Split<1> {
         hi = __bfloat16_as_ushort(h);
         lo = __bfloat16_as_ushort(l);
     }
+    __device__ static void run_finite(float x, uint16_t &hi, uint16_t &lo) { run(x, hi, lo); }
+    static constexpr float kFinite = 1.7e38f;
 };
 
 struct TcArgs {
@@ -185,29 +197,66 @@ struct TcArgs {
     float *gates;  // [P][G] or null
     double *ll;    // [P] or null
     int *status;
+    float gh, gl;    // G ln 2 pi as a float pair
     uint32_t spins;  // iteration limit of the completion wait
     int skip_mma;    // diagnostics: issue nothing for the first tile (the wait then runs out)
 };
 
-// The likelihood terms of one model's gates (Section 2.3.2), FP32 terms
-// with the TwoSum-carried sum: for gate g, yh the prediction, (yhi, ylo) the
-// float pair of the datum and ea2 = eps_an^2,
-//   r = (yhi - yh) + ylo,  v = ea2 + (eps_mn yh)^2,  t = r^2 / v + ln v,
-// and ll = -1/2 (sum t + G ln 2 pi) formed in FP64 once per model.
+// The likelihood terms of one model's gates (Section 2.3.2): for gate g, yh
+// the prediction, (yhi, ylo) the float pair of the datum and ea2 = eps_an^2,
+//   r = (yhi - yh) + ylo,  v = ea2 + (eps_mn yh)^2,
+// and ll = -1/2 (sum r^2 / v + sum ln v + G ln 2 pi), formed in FP64 once per
+// model.  The quotients are FP32, rounded once (a reciprocal and one residual
+// step), their sum an unevaluated FP32 pair (TwoSum).  The logarithms need none
+// per gate: v = m 2^e, the m in [1, 2) multiply up (a factor 2^-24 each) and the
+// e add up exactly, and sum ln v = ln2 sum e + ln prod m (a single-precision
+// ln v near -45 rounds by 2e-6, the product's factor by 6e-8).  No branch per
+// gate, so that the gates overlap: a library division and logarithm each made
+// the epilogue a chain of some 2,500 cycles per tile.  A quotient or variance
+// outside the range this is exact in marks the model, and the caller forms its
+// terms again with `exact` (the library's functions).
 struct LlAcc {
-    float s = 0.f, e = 0.f;
-    __device__ __forceinline__ void add(float yh, float2 y, float ea2, float em) {
-        const float r = (y.x - yh) + y.y;
-        const float q = em * yh;
-        const float v = fmaf(q, q, ea2);
-        const float t = __fdiv_rn(r * r, v) + logf(v);
+    float s = 0.f, e = 0.f, prod = 1.f;
+    int ex = 0;
+    bool odd = false;
+    __device__ __forceinline__ void plus(float t) {
         float s1, e1;
         two_sum(s, t, s1, e1);
         s = s1;
         e += e1;
     }
-    __device__ __forceinline__ double ll(int G) const {
-        return -0.5 * (((double)s + (double)e) + (double)G * kLn2Pi);
+    template <bool EXACT>
+    __device__ __forceinline__ void add(float yh, float2 y, float ea2, float em) {
+        const float r = (y.x - yh) + y.y;
+        const float q = em * yh;
+        const float v = fmaf(q, q, ea2);
+        const float r2 = r * r;
+        if constexpr (EXACT) {
+            plus(__fdiv_rn(r2, v) + logf(v));
+        } else {
+            const unsigned bits = __float_as_uint(v);
+            float i;
+            asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(i) : "f"(v));
+            float t = r2 * i;
+            t = fmaf(fmaf(-t, v, r2), i, t);
+            plus(t);
+            ex += (int)(bits >> 23) - 127;
+            prod *= __uint_as_float((bits & 0x7fffffu) | 0x3f800000u);
+            // v in [2^-100, 2^100], t < 2^100, and r^2 zero or large enough for the residual
+            odd |= bits - (27u << 23) > (200u << 23) || !(t < 1.2e30f) || (r2 < 1e-30f && r2 != 0.f);
+        }
+    }
+    // after at most 64 gates (prod < 2^64); gh + gl = G ln 2 pi.  The terms meet
+    // in the FP32 pair, each sum exact (an FP64 operation costs a warp 19 cycles
+    // of the SM), ex ln2 as an exact product and its small rest.
+    __device__ __forceinline__ double ll(float gh, float gl) {
+        plus(logf(prod));
+        plus((float)ex * 0.693359375f);
+        plus((float)ex * -2.12194440e-4f);
+        plus(gh);
+        const float hi = s + (e + gl);  // renormalised, so that the doubles' sum is exact
+        const float lo = (s - hi) + (e + gl);
+        return (double)(-0.5f * hi) + (double)(-0.5f * lo);
     }
 };
 
@@ -245,10 +294,11 @@ __device__ __forceinline__ void stage_chunk(const float *__restrict__ src, int F
 // c = tid + j kThreads (j < JC = kTM NKC / kThreads), each chunk KC / 4 float4
 // loads; a tile needs JC KC / 4 <= kPF of them per thread (F <= 64 for both
 // splits) and F a multiple of 4 (16-byte rows).  The next tile's loads are
-// issued before the current tile's MMA wait and epilogue, so their latency
-// overlaps both.  Chunk j's core-matrix index is (tid >> 3) + 32 j: its
-// quotient and remainder by NKC (row group, core-matrix column) advance by
-// those of 32 with one carry per chunk, from one division per thread.
+// issued before the current tile's epilogue, so their latency overlaps it.
+// Chunk j is core-matrix row r7 + 8 q, column kc, with (q, kc) the quotient and
+// remainder of (tid >> 3) + 32 j by NKC: the same for every tile, so each
+// chunk's element offset and shared-memory offset are kept, not formed again
+// (their arithmetic was a quarter of the kernel's instructions).
 constexpr int kPF = 8;
 
 template <int KIND>
@@ -257,73 +307,144 @@ struct TilePrefetch {
     static constexpr int Q = KC / 4;                 // float4 loads per chunk
     static constexpr int JMAX = kPF / Q;             // chunks per thread
     float4 v[kPF];
-    int nkc;   // NKC
-    int pack;  // divmod(tid >> 3, NKC) and divmod(32, NKC), a byte each (all below 64 when the prefetch applies)
+    int at[JMAX];  // element offset in the tile << 8 of the chunk | its parts inside the row; negative: no chunk
+    int to[JMAX];  // shared-memory offset
 
-    __device__ __forceinline__ void init(int NKC, int tid) {
-        nkc = NKC;
-        const int q0 = (tid >> 3) / NKC, dq = 32 / NKC;
-        pack = q0 | (((tid >> 3) - q0 * NKC) << 8) | (dq << 16) | ((32 - dq * NKC) << 24);
+    __device__ __forceinline__ void init(int NKC, int F, uint32_t sbo, int tid) {
+        const int jc = NKC * kTM / kThreads, r7 = tid & 7;
+#pragma unroll
+        for (int j = 0; j < JMAX; ++j) {
+            const int i = (tid >> 3) + 32 * j, q = i / NKC, kc = i - q * NKC;
+            const int parts = min(Q, max(0, (F - kc * KC + 3) / 4));
+            at[j] = j < jc ? ((((r7 + 8 * q) * F + kc * KC) << 8) | parts) : -1;
+            to[j] = q * (int)sbo + kc * 128 + r7 * 16;
+        }
     }
 
     __device__ __forceinline__ void load(const float *__restrict__ imh, int P, int F, size_t row0) {
-        const int jc = nkc * kTM / kThreads, r7 = threadIdx.x & 7;
-        const int dq = (pack >> 16) & 0xff, dc = pack >> 24;
-        int q = pack & 0xff, kc = (pack >> 8) & 0xff;
+        const float *src = imh + row0 * F;
+        const int end = P - (int)row0 >= kTM ? kTM * F : (P - (int)row0) * F;  // elements of this tile
 #pragma unroll
         for (int j = 0; j < JMAX; ++j) {
-            const size_t m = row0 + (size_t)(r7 + 8 * q);
+            const int o = at[j] >> 8, parts = at[j] & 0xff;
 #pragma unroll
-            for (int part = 0; part < Q; ++part) {
-                const int k0 = kc * KC + part * 4;
-                v[j * Q + part] = (j < jc && m < (size_t)P && k0 < F)
-                                      ? __ldg(reinterpret_cast<const float4 *>(imh + m * F + k0))
-                                      : make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int p = 0; p < Q; ++p)
+                v[j * Q + p] = at[j] >= 0 && o < end && p < parts
+                                   ? __ldg(reinterpret_cast<const float4 *>(src + o + 4 * p))
+                                   : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    }
+
+    __device__ __forceinline__ void store(unsigned char *hi, unsigned char *lo) const {
+        using S = Split<KIND>;
+        bool fin = true;
+#pragma unroll
+        for (int j = 0; j < kPF; ++j) {
+            fin = fin && fabsf(v[j].x) < S::kFinite && fabsf(v[j].y) < S::kFinite && fabsf(v[j].z) < S::kFinite &&
+                  fabsf(v[j].w) < S::kFinite;
+        }
+        if (fin)
+            write<true>(hi, lo);
+        else
+            write<false>(hi, lo);
+    }
+
+    template <bool FINITE>
+    __device__ __forceinline__ void write(unsigned char *hi, unsigned char *lo) const {
+        using S = Split<KIND>;
+#pragma unroll
+        for (int j = 0; j < JMAX; ++j) {
+            if (at[j] < 0) continue;
+            float x[KC];
+#pragma unroll
+            for (int p = 0; p < Q; ++p) {
+                x[4 * p] = v[j * Q + p].x;
+                x[4 * p + 1] = v[j * Q + p].y;
+                x[4 * p + 2] = v[j * Q + p].z;
+                x[4 * p + 3] = v[j * Q + p].w;
             }
-            q += dq;
-            kc += dc;
-            if (kc >= nkc) {
-                kc -= nkc;
-                ++q;
+            typename S::T h[KC], l[KC];
+#pragma unroll
+            for (int p = 0; p < KC; ++p) {
+                if constexpr (FINITE)
+                    S::run_finite(x[p], h[p], l[p]);
+                else
+                    S::run(x[p], h[p], l[p]);
             }
+            *reinterpret_cast<uint4 *>(hi + to[j]) = *reinterpret_cast<const uint4 *>(h);
+            *reinterpret_cast<uint4 *>(lo + to[j]) = *reinterpret_cast<const uint4 *>(l);
+        }
+    }
+};
+
+// The same for rows that are not whole float4s (F not a multiple of 4): a
+// tile's spectra are one contiguous block, thread tid takes its elements
+// tid + 256 j, so the loads coalesce whatever F; element (row, column) advances
+// by 256's quotient and remainder by F with one carry.  At most kFlat per
+// thread (F <= 64).
+constexpr int kFlat = 32;
+
+template <int KIND>
+struct FlatPrefetch {
+    float v[kFlat];
+    int F, n, row, col, dr, dc;
+
+    __device__ __forceinline__ void init(int F_, int tid) {
+        F = F_;
+        n = kTM * F;
+        row = tid / F;
+        col = tid - row * F;
+        dr = kThreads / F;
+        dc = kThreads - dr * F;
+    }
+
+    __device__ __forceinline__ void load(const float *__restrict__ imh, int P, size_t row0) {
+        const float *src = imh + row0 * F;
+        const size_t left = ((size_t)P - row0) * F;
+        const int m = left < (size_t)n ? (int)left : n;
+#pragma unroll
+        for (int j = 0; j < kFlat; ++j) {
+            const int i = (int)threadIdx.x + j * kThreads;
+            v[j] = i < m ? __ldg(src + i) : 0.f;
         }
     }
 
     __device__ __forceinline__ void store(uint32_t sbo, unsigned char *hi, unsigned char *lo) const {
         using S = Split<KIND>;
-        const int jc = nkc * kTM / kThreads, r7 = threadIdx.x & 7;
-        const int dq = (pack >> 16) & 0xff, dc = pack >> 24;
-        int q = pack & 0xff, kc = (pack >> 8) & 0xff;
+        constexpr int KC = 16 / S::ES;
+        int r = row, c = col;
 #pragma unroll
-        for (int j = 0; j < JMAX; ++j) {
-            if (j < jc) {
-                const uint32_t o = (uint32_t)q * sbo + (uint32_t)kc * 128u + (uint32_t)r7 * 16u;
-                float x[KC];
-#pragma unroll
-                for (int p = 0; p < Q; ++p) {
-                    x[4 * p] = v[j * Q + p].x;
-                    x[4 * p + 1] = v[j * Q + p].y;
-                    x[4 * p + 2] = v[j * Q + p].z;
-                    x[4 * p + 3] = v[j * Q + p].w;
-                }
-                typename S::T h[KC], l[KC];
-#pragma unroll
-                for (int p = 0; p < KC; ++p) S::run(x[p], h[p], l[p]);
-                *reinterpret_cast<uint4 *>(hi + o) = *reinterpret_cast<const uint4 *>(h);
-                *reinterpret_cast<uint4 *>(lo + o) = *reinterpret_cast<const uint4 *>(l);
+        for (int j = 0; j < kFlat; ++j) {
+            if ((int)threadIdx.x + j * kThreads < n) {
+                const uint32_t o = (uint32_t)(r >> 3) * sbo + (uint32_t)(c / KC) * 128u + (uint32_t)(r & 7) * 16u +
+                                   (uint32_t)(c % KC) * S::ES;
+                typename S::T h, l;
+                S::run(v[j], h, l);
+                *reinterpret_cast<typename S::T *>(hi + o) = h;
+                *reinterpret_cast<typename S::T *>(lo + o) = l;
             }
-            q += dq;
-            kc += dc;
-            if (kc >= nkc) {
-                kc -= nkc;
-                ++q;
+            r += dr;
+            c += dc;
+            if (c >= F) {
+                c -= F;
+                ++r;
             }
         }
     }
 };
 
-template <int KIND>
-__global__ void __launch_bounds__(kThreads, KIND == 0 ? 2 : 3) gates_tc_kernel(TcArgs a) {
+// FLAT: the flat prefetch's registers (rows that are not whole float4s);
+// otherwise the float4 one's, or none when the tile does not fit them.
+// Software pipeline per CTA: once a tile's MMAs are done its operand buffer and
+// the other accumulator are free, so the next tile is converted into shared
+// memory and its MMAs issued, the spectra after it requested, and only then
+// this tile's accumulator read: the tensor core and the loads run under the
+// epilogue, one CTA barrier per tile.  2^20 spectra of 60 frequencies, TF32
+// split, likelihood: 182 -> 113 us (a tile's chain of stage, fence, MMA, wait
+// and epilogue took 14,600 cycles end to end; 8,700 warp instructions a tile
+// are left at 56 % issue, 2.2 TB/s).
+template <int KIND, bool FLAT>
+__global__ void __launch_bounds__(kThreads, KIND == 0 || FLAT ? 2 : 3) gates_tc_kernel(TcArgs a) {
     using S = Split<KIND>;
     constexpr int ES = S::ES;
     constexpr int KI = 32 / ES;  // K of one MMA: two core matrices
@@ -336,10 +457,11 @@ __global__ void __launch_bounds__(kThreads, KIND == 0 ? 2 : 3) gates_tc_kernel(T
     const uint32_t sbo = (uint32_t)NKC * 128u;  // same for A and B
     const uint32_t a_bytes = (uint32_t)kTM * a.KP * ES, b_bytes = (uint32_t)a.N * a.KP * ES;
     unsigned char *Ahi = base, *Alo = base + a_bytes, *Bhi = base + 2 * a_bytes, *Blo = Bhi + b_bytes;
-    float2 *ysplit = reinterpret_cast<float2 *>(Blo + b_bytes);  // [2][G]: the datum rows of this tile
-    float *ea2 = reinterpret_cast<float *>(ysplit + 2 * AEM_MAX_GATES);
-    float2 *llp = reinterpret_cast<float2 *>(ea2 + AEM_MAX_GATES);  // [kTM]: the second column half's sums
-    uint64_t *mbar_p = reinterpret_cast<uint64_t *>(llp + kTM);
+    // [2][N]: the datum rows of this tile, (y high, y low, eps_an^2, 0); past G
+    // (0, 0, 1, 0), which with the accumulator's zero there adds nothing
+    float4 *ysplit = reinterpret_cast<float4 *>(Blo + b_bytes);
+    float4 *llp = ysplit + 2 * AEM_MAX_GATES;  // [2][kTM]: the second column half's sums
+    uint64_t *mbar_p = reinterpret_cast<uint64_t *>(llp + 2 * kTM);
     uint32_t *slot_p = reinterpret_cast<uint32_t *>(mbar_p + 1);
     int *abort_p = reinterpret_cast<int *>(slot_p + 1);
     const uint32_t mbar = smem_u32(mbar_p);
@@ -351,15 +473,18 @@ __global__ void __launch_bounds__(kThreads, KIND == 0 ? 2 : 3) gates_tc_kernel(T
         *abort_p = 0;
     }
     __syncwarp();
-    if (warp == 0) tmem_alloc(smem_u32(slot_p), (uint32_t)a.ncols);
+    const uint32_t dcols = a.N <= 32 ? 32u : 64u;  // columns of one accumulator; two are allocated
+    if (warp == 0) tmem_alloc(smem_u32(slot_p), 2 * dcols);
     // B = T (rows: gates, zero-padded to N; columns: frequencies, zero-padded to KP)
     for (int c = tid; c < a.N * NKC; c += kThreads) {
         const int r = (c & 7) + 8 * ((c >> 3) / NKC), kc = (c >> 3) % NKC;
         const uint32_t o = (uint32_t)(r >> 3) * sbo + (uint32_t)kc * 128u + (uint32_t)(r & 7) * 16u;
         stage_chunk<KIND>(r < a.G ? a.T + (size_t)r * a.F : nullptr, a.F, kc, false, Bhi + o, Blo + o);
     }
-    if (a.eps_an)
-        for (int g = tid; g < a.G; g += kThreads) ea2[g] = (float)(a.eps_an[g] * a.eps_an[g]);
+    if (FLAT) {  // columns past F stay zero
+        for (uint32_t i = tid; i < 2 * a_bytes / 16; i += kThreads)
+            reinterpret_cast<uint4 *>(base)[i] = make_uint4(0u, 0u, 0u, 0u);
+    }
     tc_before_sync();
     __syncthreads();
     tc_after_sync();
@@ -368,132 +493,176 @@ __global__ void __launch_bounds__(kThreads, KIND == 0 ? 2 : 3) gates_tc_kernel(T
     const uint32_t ahi = smem_u32(Ahi), alo = smem_u32(Alo), bhi = smem_u32(Bhi), blo = smem_u32(Blo);
     const int ntiles = (a.P + kTM - 1) / kTM;
     const float em = (float)a.eps_mn;
-    uint32_t phase = 0;
-    bool pending = false;  // an MMA chain committed and not yet observed complete
-    bool first = true;
-    const bool pf_ok = vec4 && NKC * kTM / kThreads * TilePrefetch<KIND>::Q <= kPF;
-    TilePrefetch<KIND> pf;
-    if (pf_ok) pf.init(NKC, tid);
-    if (pf_ok && (int)blockIdx.x < ntiles) pf.load(a.imh, a.P, a.F, (size_t)blockIdx.x * kTM);
     // P < 2^31 and obs_per >= 1: the datum row of model m is m / obs_per in 32-bit arithmetic
     const unsigned int obs_per = (unsigned int)a.obs_per;
     const unsigned int last_row = (unsigned int)(a.P - 1) / obs_per;
+    const bool split_rows = a.y_obs && obs_per >= (unsigned int)kTM;
 
-    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        const size_t row0 = (size_t)tile * kTM;
-        // the datum rows this tile's models use, as float pairs (at most two
-        // when models_per_row >= the tile; otherwise the epilogue splits per model)
-        const unsigned int s0 = (unsigned int)row0 / obs_per;
-        const bool split_rows = a.y_obs && obs_per >= (unsigned int)kTM;
-        if (split_rows)
-            for (int i = tid; i < 2 * a.G; i += kThreads) {
-                const int two = i >= a.G ? 1 : 0;
-                const unsigned int srow = s0 + (unsigned int)two;
-                const double y = a.y_obs[(size_t)(srow <= last_row ? srow : last_row) * a.G + (i - two * a.G)];
-                const float hi = (float)y;
-                ysplit[i] = make_float2(hi, (float)(y - (double)hi));
-            }
-        // stage the tile's spectra (rows past P and columns past F are zero);
-        // consecutive lanes fill consecutive 16-byte rows of one core matrix
+    typename std::conditional<FLAT, FlatPrefetch<KIND>, TilePrefetch<KIND>>::type pf;
+    bool pf_ok = FLAT;
+    if constexpr (FLAT) {
+        pf.init(a.F, tid);
+    } else {
+        pf_ok = vec4 && NKC * kTM / kThreads * TilePrefetch<KIND>::Q <= kPF;
+        if (pf_ok) pf.init(NKC, a.F, sbo, tid);
+    }
+    auto request = [&](int tile) {
+        if (!pf_ok || tile >= ntiles) return;
+        if constexpr (FLAT)
+            pf.load(a.imh, a.P, (size_t)tile * kTM);
+        else
+            pf.load(a.imh, a.P, a.F, (size_t)tile * kTM);
+    };
+    // the tile's spectra as high / low operands (rows past P and columns past F
+    // are zero); consecutive lanes fill consecutive 16-byte rows of one core matrix
+    auto stage = [&](int tile) {
         if (pf_ok) {
-            pf.store(sbo, Ahi, Alo);
+            if constexpr (FLAT)
+                pf.store(sbo, Ahi, Alo);
+            else
+                pf.store(Ahi, Alo);
         } else {
             for (int c = tid; c < kTM * NKC; c += kThreads) {
                 const int r = (c & 7) + 8 * ((c >> 3) / NKC), kc = (c >> 3) % NKC;
-                const size_t m = row0 + r;
+                const size_t m = (size_t)tile * kTM + r;
                 const uint32_t o = (uint32_t)(r >> 3) * sbo + (uint32_t)kc * 128u + (uint32_t)(r & 7) * 16u;
                 stage_chunk<KIND>(m < (size_t)a.P ? a.imh + m * a.F : nullptr, a.F, kc, vec4, Ahi + o, Alo + o);
             }
         }
         fence_async_smem();
+    };
+    auto issue = [&](uint32_t acc) {
+        for (int ks = 0; ks < a.KP / KI; ++ks) {
+            const uint32_t off = (uint32_t)ks * 256u;
+            const uint64_t dah = smem_desc(ahi + off, 128u, sbo), dal = smem_desc(alo + off, 128u, sbo);
+            const uint64_t dbh = smem_desc(bhi + off, 128u, sbo), dbl = smem_desc(blo + off, 128u, sbo);
+            mma<KIND>(acc, dah, dbh, idesc, ks > 0 ? 1u : 0u);
+            mma<KIND>(acc, dah, dbl, idesc, 1u);
+            mma<KIND>(acc, dal, dbh, idesc, 1u);
+        }
+        mma_commit(mbar);
+    };
+
+    const int quarter = warp & 3, half = warp >> 2, row = quarter * 32 + lane;
+    uint32_t phase = 0;
+    const int first_tile = (int)blockIdx.x, step = (int)gridDim.x;
+    bool pending = !a.skip_mma;  // an MMA chain committed and not yet observed complete
+    request(first_tile);
+    stage(first_tile);
+    tc_before_sync();
+    __syncthreads();
+    tc_after_sync();
+    if (tid == 0 && pending) issue(tbase);
+    request(first_tile + step);
+    unsigned int have_row = 0xffffffffu;  // the datum row ysplit begins with
+    LlAcc acc;          // of the tile before, until its other half's sums are there
+    size_t acc_m = 0;
+    bool acc_valid = false;
+    // the two halves' sums meet in shared memory, added in a fixed order by the first half's thread
+    auto finish = [&](int buf) {
+        if (a.ll && half == 0 && acc_valid) {
+            const float4 o = llp[buf * kTM + row];
+            float s1, e1;
+            two_sum(acc.s, o.x, s1, e1);
+            acc.s = s1;
+            acc.e = (acc.e + o.y) + e1;
+            acc.prod *= o.z;
+            acc.ex += __float_as_int(o.w);
+            a.ll[acc_m] = acc.ll(a.gh, a.gl);
+        }
+    };
+    int buf = 0;
+    for (int tile = first_tile; tile < ntiles; tile += step, buf ^= 1) {
+        const size_t row0 = (size_t)tile * kTM;
+        const bool done = mbar_wait_bounded(mbar, phase, a.spins);
+        if (!done) atomicExch(abort_p, 1);
+        // the datum rows this tile's models use, as float pairs (at most two
+        // when models_per_row >= the tile; otherwise the epilogue splits per model)
+        const unsigned int s0 = last_row == 0 ? 0u : (unsigned int)row0 / obs_per;
+        const bool new_row = split_rows && s0 != have_row;  // CTA-uniform
+        const bool more = tile + step < ntiles;
+        if (done && more) stage(tile + step);
         tc_before_sync();
         __syncthreads();
         tc_after_sync();
-        const bool issue = !(first && a.skip_mma);
-        if (tid == 0 && issue) {
-            for (int ks = 0; ks < a.KP / KI; ++ks) {
-                const uint32_t off = (uint32_t)ks * 256u;
-                const uint64_t dah = smem_desc(ahi + off, 128u, sbo), dal = smem_desc(alo + off, 128u, sbo);
-                const uint64_t dbh = smem_desc(bhi + off, 128u, sbo), dbl = smem_desc(blo + off, 128u, sbo);
-                mma<KIND>(tbase, dah, dbh, idesc, ks > 0 ? 1u : 0u);
-                mma<KIND>(tbase, dah, dbl, idesc, 1u);
-                mma<KIND>(tbase, dal, dbh, idesc, 1u);
-            }
-            mma_commit(mbar);
-        }
-        first = false;
-        pending = issue;
-        // the next tile's loads go out while the MMA runs and the epilogue reads it
-        if (pf_ok && tile + (int)gridDim.x < ntiles)
-            pf.load(a.imh, a.P, a.F, (size_t)(tile + gridDim.x) * kTM);
-        const bool done = mbar_wait_bounded(mbar, phase, a.spins);
-        if (!done) atomicExch(abort_p, 1);
-        __syncthreads();
+        finish(buf ^ 1);
+        acc_valid = false;
         if (*abort_p) break;
-        pending = false;
         phase ^= 1u;
-        tc_after_sync();
+        pending = more;
+        if (tid == 0 && more) issue(tbase + (uint32_t)(buf ^ 1) * dcols);
+        request(tile + 2 * step);
+        if (new_row) {  // the epilogue before has been left by every thread
+            for (int i = tid; i < 2 * a.N; i += kThreads) {
+                const int two = i >= a.N ? 1 : 0, g = i - two * a.N;
+                const unsigned int srow = s0 + (unsigned int)two;
+                float4 rec = make_float4(0.f, 0.f, 1.f, 0.f);
+                if (g < a.G) {
+                    const double y = a.y_obs[(size_t)(srow <= last_row ? srow : last_row) * a.G + g];
+                    const float hi = (float)y;
+                    rec = make_float4(hi, (float)(y - (double)hi), (float)(a.eps_an[g] * a.eps_an[g]), 0.f);
+                }
+                ysplit[i] = rec;
+            }
+            have_row = s0;
+            __syncthreads();
+        }
         // epilogue: this thread's model is row 32 (warp mod 4) + lane of the
         // tile; warps 0-3 take the first half of the gate columns, 4-7 the second
-        const int quarter = warp & 3, half = warp >> 2;
-        const int row = quarter * 32 + lane;
         const size_t m = row0 + (size_t)row;
         const bool valid = m < (size_t)a.P;
         // with split rows the tile spans datum rows s0 and s0 + 1 at most
         const unsigned int srow =
             !valid ? 0u
                    : split_rows ? s0 + ((unsigned int)m >= (s0 + 1u) * obs_per ? 1u : 0u) : (unsigned int)m / obs_per;
-        const float2 *yrow = split_rows ? ysplit + (srow - s0) * a.G : nullptr;
+        const float4 *yrow = ysplit + (split_rows ? (srow - s0) * (unsigned int)a.N : 0u);
         const double *yd = (a.y_obs && !split_rows) ? a.y_obs + (size_t)srow * a.G : nullptr;
-        LlAcc acc;
         const int c_lo = half * (a.N / 2), c_hi = c_lo + a.N / 2;
-        for (int c = c_lo; c < c_hi; c += 8) {
-            float v[8];
-            tmem_ld8(tbase + ((uint32_t)(quarter * 32) << 16) + (uint32_t)c, v);
+        auto columns = [&](auto exact) {
+            constexpr bool EXACT = decltype(exact)::value;
+            acc = LlAcc();
+            for (int c = c_lo; c < c_hi; c += 8) {
+                float v[8];
+                tmem_ld8(tbase + (uint32_t)buf * dcols + ((uint32_t)(quarter * 32) << 16) + (uint32_t)c, v);
+                if (!EXACT && a.gates && valid) {
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                const int g = c + q;
-                if (valid && g < a.G) {
-                    if (a.gates) a.gates[m * a.G + g] = v[q];
-                    if (a.y_obs) {
-                        float2 y;
-                        if (yrow) {
-                            y = yrow[g];
-                        } else {
-                            const double yv = yd[g];
-                            y.x = (float)yv;
-                            y.y = (float)(yv - (double)y.x);
-                        }
-                        acc.add(v[q], y, ea2[g], em);
+                    for (int q = 0; q < 8; ++q)
+                        if (c + q < a.G) a.gates[m * a.G + c + q] = v[q];
+                }
+                if (split_rows) {  // columns past G and rows past P are harmless
+#pragma unroll
+                    for (int q = 0; q < 8; ++q) {
+                        const float4 y = yrow[c + q];
+                        if (!EXACT || c + q < a.G) acc.add<EXACT>(v[q], make_float2(y.x, y.y), y.z, em);
+                    }
+                } else if (yd && valid) {
+                    for (int q = 0; q < 8 && c + q < a.G; ++q) {
+                        const double yv = yd[c + q];
+                        const float hi = (float)yv, ea = (float)(a.eps_an[c + q] * a.eps_an[c + q]);
+                        acc.add<EXACT>(v[q], make_float2(hi, (float)(yv - (double)hi)), ea, em);
                     }
                 }
             }
-        }
-        if (a.ll) {
-            // the two halves' (sum, error) pairs meet in shared memory, added
-            // in a fixed order by the first half's thread
-            if (half == 1) llp[row] = make_float2(acc.s, acc.e);
-            __syncthreads();
-            if (half == 0 && valid) {
-                const float2 o = llp[row];
-                float s1, e1;
-                two_sum(acc.s, o.x, s1, e1);
-                acc.s = s1;
-                acc.e = (acc.e + o.y) + e1;
-                a.ll[m] = acc.ll(a.G);
-            }
-        }
-        tc_before_sync();
-        __syncthreads();  // every lane read before the next chain overwrites the accumulator
-    }
-    if (*abort_p) {
-        if (tid == 0) atomicExch(a.status, (int)AEM_ERR_TIMEOUT);
-        if (pending) mbar_wait_bounded(mbar, phase);  // our own MMAs, once more with the full limit
+        };
+        columns(std::false_type{});
+        if (__any_sync(0xffffffffu, acc.odd)) columns(std::true_type{});
+        acc_m = m;
+        acc_valid = valid;
+        if (a.ll && half == 1) llp[buf * kTM + row] = make_float4(acc.s, acc.e, acc.prod, __int_as_float(acc.ex));
     }
     tc_before_sync();
     __syncthreads();
     tc_after_sync();
-    if (warp == 0) tmem_dealloc(tbase, (uint32_t)a.ncols);
+    if (*abort_p) {
+        if (tid == 0) atomicExch(a.status, (int)AEM_ERR_TIMEOUT);
+        if (pending) mbar_wait_bounded(mbar, phase);  // our own MMAs, once more with the full limit
+    } else {
+        finish(buf ^ 1);
+    }
+    tc_before_sync();
+    __syncthreads();
+    tc_after_sync();
+    if (warp == 0) tmem_dealloc(tbase, 2 * dcols);
 }
 
 // FP32 CUDA-core form of the same transform (for comparison): one thread per
@@ -516,10 +685,10 @@ __global__ void gates_fp32_kernel(TcArgs a) {
             if (a.gates) a.gates[m * a.G + g] = s;
             if (y) {
                 const float hi = (float)y[g];
-                acc.add(s, make_float2(hi, (float)(y[g] - (double)hi)), ea2[g], em);
+                acc.add<true>(s, make_float2(hi, (float)(y[g] - (double)hi)), ea2[g], em);
             }
         }
-        if (a.ll) a.ll[m] = acc.ll(a.G);
+        if (a.ll) a.ll[m] = acc.ll(a.gh, a.gl);
     }
 }
 
@@ -560,8 +729,9 @@ int gates_from_spectrum(const aem_system *sys, const float *imh, int P, int mode
                         int obs_per, const double *eps_an, double eps_mn, float *gates, double *ll,
                         cudaStream_t stream) {
     const SystemTables &h = sys->host;
+    const double gconst = h.G * kLn2Pi;
     TcArgs a{imh, P, h.F, h.G, 0, 0, 0, sys->d_T_f, y_obs, obs_per > 0 ? obs_per : 1, eps_an, eps_mn, gates, ll,
-             sys->d_status, sys->wait_spins ? sys->wait_spins : kSpinLimit, sys->wait_skip_mma};
+             sys->d_status, (float)gconst, (float)(gconst - (double)(float)gconst), sys->wait_spins ? sys->wait_spins : kSpinLimit, sys->wait_skip_mma};
     if (mode == AEM_GATES_FP32) {
         const size_t smem = sizeof(float) * (size_t)h.G * h.F;
         int grid = (int)((P + 255) / 256);
@@ -574,10 +744,14 @@ int gates_from_spectrum(const aem_system *sys, const float *imh, int P, int mode
     const int ES = tf32 ? 4 : 2, KI = 32 / ES;
     a.KP = round_up(h.F, KI);
     a.N = round_up(h.G, 16);
-    a.ncols = a.N <= 32 ? 32 : 64;
-    const size_t smem = (size_t)2 * (kTM + a.N) * a.KP * ES + 1024 + sizeof(float2) * 2 * AEM_MAX_GATES +
-                        sizeof(float) * AEM_MAX_GATES + sizeof(float2) * kTM + 64;
-    auto kern = tf32 ? gates_tc_kernel<0> : gates_tc_kernel<1>;
+    a.ncols = 2 * (a.N <= 32 ? 32 : 64);
+    const size_t smem = (size_t)2 * (kTM + a.N) * a.KP * ES + 1024 + sizeof(float4) * 2 * AEM_MAX_GATES +
+                        sizeof(float4) * 2 * kTM + 64;
+    // rows of whole float4s take the float4 prefetch, others (up to 64
+    // frequencies, kFlat registers) the flat one
+    const bool flat = (h.F & 3) != 0 && h.F <= 2 * kFlat;
+    auto kern = tf32 ? (flat ? gates_tc_kernel<0, true> : gates_tc_kernel<0, false>)
+                     : (flat ? gates_tc_kernel<1, true> : gates_tc_kernel<1, false>);
     int per_sm = 0;
     if (const int rc = tc_resident(sys, mode, kern, smem, a.ncols, &per_sm)) return rc;
     if (per_sm < 1) return fail(AEM_ERR_UNSUPPORTED, "aem_gates_from_spectrum: tile does not fit in shared memory");
