@@ -7,29 +7,46 @@
 // log-likelihood.  Then one CTA per model (models claimed from a counter)
 // forms the adjoint seeds from those gates,
 //   a_f = sum_g T[g,f] dl/dyhat_g,  dl/dyhat = r/v + (e_mn^2 yhat / v)(r^2/v - 1),
-// and visits every (frequency, abscissa) item with weight a_f w_k: the
-// recursion is run bottom-up storing the reflection coefficients Gamma_j, then
-// top-down propagating dGamma_0/dGamma_j through the Moebius steps
-//   Gamma_j = (rho_j + Gamma_{j+1} E_j) / (1 + rho_j Gamma_{j+1} E_j),
-//   rho_j = (s_{j-1} - s_j) / (u_{j-1} + u_j)^2,  E_j = exp(-2 u_j h_j),
-//   u_j = sqrt(lambda^2 + s_j),
-// and emitting, for each layer, Im(dGamma_0/ds_n ds_n/dp) and Im(dGamma_0/dh_n)
-// into per-thread accumulators, reduced over the CTA at the end of the model.
-// R_0 is holomorphic in every s_n, so d Im R_0 / dp = Im(dR_0/ds_n ds_n/dp)
-// for the real parameters p.
+// and visits every (frequency, abscissa) item with weight a_f w_k.  Per item,
+// bottom-up, with w_n = sqrt(2 (lambda^2 + s_n)) and E_n = exp(-sqrt(2) w_n h_n),
+// the down- and upgoing amplitudes (D_n, N_n) at the bottom of every layer n
+// follow from the continuity of the field e and of h = w (D - P):
+//   D_n, N_n = e +- h / w_n,  P_n = N_n E_n,  e = D_n + P_n,  h = w_n (D_n - P_n)
+// from e = 1, h = w of the half-space, up to D_0 = e + h / (sqrt(2) lambda) of
+// the air (each interface doubles the scale).  The derivative of R_0 by s_n is
+// the integral of the squared field over the layer (the self-adjoint equation's
+// sensitivity; its closed form has no interface terms, and between layers only
+// the attenuation changes, c_{n+1} = 4 E_n c_n):
+//   dR_0/ds_n = -c_n [(1 - E_n)(D_n^2 + N_n P_n) 2 / w_n + 4 sqrt(2) h_n D_n P_n],
+//   dR_0/dh_n = -c_n sqrt(2) w_n^2 4 D_n P_n,  c_0 = 1 / (D_0^2 sqrt(2) lambda),
+//   dR_0/ds = -c 2 / w for the half-space.
+// For each layer Im(dR_0/ds_n ds_n/dp) and Im(dR_0/dh_n) go into per-thread
+// accumulators, reduced over the CTA at the end of the model.  R_0 is
+// holomorphic in every s_n, so d Im R_0 / dp = Im(dR_0/ds_n ds_n/dp) for the
+// real parameters p.
 //
 // Like the forward kernel, each thread carries two abscissae of one frequency
 // (k and k + K/2) through both passes in 64-bit register pairs on the paired
 // FP32 instructions (f32x2.h); the two abscissae's weighted adjoints are added
 // before they meet the per-(frequency, layer) derivatives ds_n/dp, which do
 // not depend on the abscissa.
+//
+// The bound is the instruction issue of the paired FP32 and special-function
+// units: about 100 paired operations and 20 special-function ones per pair and
+// layer for both passes.  Differentiating the Moebius chain interface by
+// interface took 163 and 28: 16384 models of 60 x 200 items with 1 to 10
+// layers, forward kernel included, 7.05 -> 4.89 ms.  E_n is formed again on the
+// way down: kept from the way up it costs 16 bytes of local memory per layer
+// each way, 5.58 against 5.23 ms.
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <type_traits>
 
 #include "aem_internal.h"
 #include "depth_cutoff.h"
 #include "f32x2.h"
+#include "te_roots.h"
 
 namespace aem {
 namespace {
@@ -58,9 +75,6 @@ __device__ __forceinline__ C2x2 c2(u64 re, u64 im) {
     r.im = im;
     return r;
 }
-__device__ __forceinline__ C2x2 c2add(C2x2 a, C2x2 b) { return c2(add2(a.re, b.re), add2(a.im, b.im)); }
-__device__ __forceinline__ C2x2 c2neg(C2x2 a) { return c2(sub2(kZero2, a.re), sub2(kZero2, a.im)); }
-__device__ __forceinline__ C2x2 c2add1(C2x2 a) { return c2(add2(kOne2, a.re), a.im); }         // 1 + a
 __device__ __forceinline__ C2x2 c2mul(C2x2 a, C2x2 b) {
     return c2(sub2(mul2(a.re, b.re), mul2(a.im, b.im)), fma2(a.re, b.im, mul2(a.im, b.re)));
 }
@@ -71,45 +85,49 @@ __device__ __forceinline__ C2x2 c2sq(C2x2 a) {
     const u64 t = mul2(a.re, a.im);
     return c2(mul2(sub2(a.re, a.im), add2(a.re, a.im)), add2(t, t));
 }
-__device__ __forceinline__ C2x2 c2scale(C2x2 a, u64 s) { return c2(mul2(a.re, s), mul2(a.im, s)); }
-constexpr u64 kMinus2 = 0xc0000000c0000000ull;  // (-2, -2)
-__device__ __forceinline__ C2x2 c2one_minus_sq(C2x2 a) {  // 1 - a^2
-    return c2(fma2(a.im, a.im, sub2(kOne2, mul2(a.re, a.re))), mul2(mul2(a.re, a.im), kMinus2));
+// The power of two next to 1 / max(|Re d|, |Im d|), per abscissa (2^-126 .. 2^126;
+// of zero, an infinity or a NaN one of the ends).
+__device__ __forceinline__ float pow2_inv(float a, float b) {
+    const int e = __float_as_int(fmaxf(fabsf(a), fabsf(b))) >> 23;
+    return __int_as_float(min(max(254 - e, 1), 253) << 23);
 }
-__device__ __forceinline__ u64 c2inorm(C2x2 a) {  // 1 / |a|^2
-    float m0, m1;
-    up2(fma2(a.re, a.re, mul2(a.im, a.im)), m0, m1);
-    return pk2(rcp_approx(m0), rcp_approx(m1));
+__device__ __forceinline__ u64 pow2_inv2(C2x2 d) {
+    float a0, a1, b0, b1;
+    up2(d.re, a0, a1);
+    up2(d.im, b0, b1);
+    return pk2(pow2_inv(a0, b0), pow2_inv(a1, b1));
 }
-__device__ __forceinline__ C2x2 c2div(C2x2 x, C2x2 a) { return c2scale(c2mulc(x, a), c2inorm(a)); }
+constexpr u64 kTwo2 = 0x4000000040000000ull, kQuarter2 = 0x3e8000003e800000ull;
+constexpr u64 kMinusHalf2 = 0xbf000000bf000000ull, kMinusOne2 = 0xbf800000bf800000ull;
 
-// Principal root u of z = lambda^2 + s (Im s > 0) for both abscissae, and
-// 1 / (2 |z|) (= 1 / (2 |u|^2), for du/ds = 1 / (2 u) = conj(u) / (2 |z|)).  With t = (|z| + |x|) / 2 the pair
-// (sqrt t, Im s / (2 sqrt t)) is (Re u, Im u) when x = Re z >= 0 and
-// (Im u, Re u) otherwise.  s = ((Re s, Re s), (Im s, Im s)), y2 = (Im s)^2.
-__device__ __forceinline__ C2x2 c2root(u64 lam2, ulonglong2 s, u64 y2, u64 &inv_mod) {
-    const u64 x = add2(lam2, s.x);
-    const u64 v = fma2(x, x, y2);
+// root2 and 1 / m (for dw/ds = 1 / w = conj(w) / (2 m)).
+__device__ __forceinline__ Root root2_inv(u64 lam2, ulonglong2 rec, u64 &inv_m) {
+    const u64 x = add2(lam2, rec.x);
+    const u64 v = fma2(x, x, mul2(rec.y, rec.y));
     float v0, v1, x0, x1;
     up2(v, v0, v1);
     up2(x, x0, x1);
-    const u64 rv = pk2(rsqrt_approx(v0), rsqrt_approx(v1));  // v = |z|^2
-    inv_mod = mul2(rv, kHalf2);
-    const u64 t = mul2(add2(mul2(v, rv), pk2(fabsf(x0), fabsf(x1))), kHalf2);
-    float t0, t1;
-    up2(t, t0, t1);
+    inv_m = pk2(rsqrt_approx(v0), rsqrt_approx(v1));
+    Root w;
+    w.m = mul2(v, inv_m);
+    float m0, m1;
+    up2(w.m, m0, m1);
+    const float t0 = m0 + fabsf(x0), t1 = m1 + fabsf(x1);
     const u64 rr = pk2(rsqrt_approx(t0), rsqrt_approx(t1));
     float p0, p1, o0, o1;
-    up2(mul2(t, rr), p0, p1);
-    up2(mul2(mul2(s.y, kHalf2), rr), o0, o1);
-    return c2(pk2(x0 >= 0.f ? p0 : o0, x1 >= 0.f ? p1 : o1), pk2(x0 >= 0.f ? o0 : p0, x1 >= 0.f ? o1 : p1));
+    up2(mul2(pk2(t0, t1), rr), p0, p1);
+    up2(mul2(rec.y, rr), o0, o1);
+    w.re = pk2(x0 >= 0.f ? p0 : o0, x1 >= 0.f ? p1 : o1);
+    w.im = pk2(x0 >= 0.f ? o0 : p0, x1 >= 0.f ? o1 : p1);
+    return w;
 }
 
-// E = exp(-2 h u) for both abscissae; he = ((-2 h log2 e) x 2, (-2 h) x 2)
-__device__ __forceinline__ C2x2 c2expm(ulonglong2 he, C2x2 u) {
+// E = exp(-sqrt(2) w h) for both abscissae (FOUR: 4 E); he = (e x 2, e ln2 x 2), e = -sqrt(2) h log2 e
+template <bool FOUR>
+__device__ __forceinline__ C2x2 c2expm(ulonglong2 he, const Root &w) {
     float a0, a1, f0, f1, s0, c0, s1, c1;
-    up2(mul2(he.x, u.re), a0, a1);
-    up2(reduce_2pi2(mul2(he.y, u.im)), f0, f1);
+    up2(FOUR ? fma2(he.x, w.re, kTwo2) : mul2(he.x, w.re), a0, a1);
+    up2(reduce_2pi2(mul2(he.y, w.im)), f0, f1);
     sincos_approx(f0, &s0, &c0);
     sincos_approx(f1, &s1, &c1);
     const u64 e = pk2(ex2_approx(a0), ex2_approx(a1));
@@ -130,39 +148,39 @@ struct GradModels {
 };
 
 // Shared memory (dynamic), in order: RS[F*LS] (ulonglong2: (Re s, Re s),
-// (Im s, Im s)), lamp[K2] (ulonglong2: (lam_a^2, lam_b^2), (lam_a, lam_b)),
-// DS[F*LS*4] (float2 ds/dp for log10 sigma, m, log10 tau, c), RY2[F*LS] (u64:
-// (Im s)^2 twice), hwp[K2] (float2 weights of the pair), af[F], T[G*F],
+// (Im s, Im s)), lamp[K2] (ulonglong2: (lam_a^2, lam_b^2), 1 / (sqrt(2) lambda)),
+// DS[F*LS*2] (float4: ds/dp for log10 sigma and m, then for log10 tau and c),
+// hwp[K2] (float2 weights of the pair over sqrt(2) lambda), af[F], T[G*F],
 // part[kGW * LS * kNP], TH[F*LS] (float: the depth cutoff's thresholds).
 size_t grad_smem_bytes(int F, int G, int K, int LS) {
     const size_t K2 = (size_t)(K + 1) / 2, FL = (size_t)F * LS;
-    return sizeof(ulonglong2) * (FL + K2) + sizeof(float2) * (FL * 4) + sizeof(u64) * FL + sizeof(float2) * K2 +
+    return sizeof(ulonglong2) * (FL + K2) + sizeof(float4) * (FL * 2) + sizeof(float2) * K2 +
            sizeof(float) * ((size_t)F + (size_t)G * F + (size_t)kGW * LS * kNP + FL);
 }
 
 // MAXL: the largest layer count the per-thread arrays hold (10 or
 // AEM_MAX_LAYERS), so the common lmax <= 10 keeps them half as large.  Three
-// resident CTAs per SM (80 registers) measured faster than two (128
-// registers, no spills) and four (64 registers, 200 bytes spilled).
+// resident CTAs per SM (80 registers) measure faster than two (120 registers,
+// 5.9 against 5.2 ms of the workload above) and like four (64, spilling).
 template <int MAXL>
 __global__ void __launch_bounds__(kGT, 3) loglik_grad_kernel(GradModels mv, int F, int G, int K, int LS, int cc_form,
-                                                          const float *__restrict__ g_omega,
-                                                          const float *__restrict__ g_lam,
-                                                          const float *__restrict__ g_hw,
-                                                          const float *__restrict__ g_T,
-                                                          const double *__restrict__ y_obs, int obs_per,
-                                                          const double *__restrict__ eps_an, double eps_mn,
-                                                          const float *__restrict__ g_gates, float *__restrict__ grad,
-                                                          int *__restrict__ work_counter, float att0,
-                                                          const int8_t *__restrict__ valid) {
+                                                             float len,
+                                                             const float *__restrict__ g_omega,
+                                                             const float *__restrict__ g_lam,
+                                                             const float *__restrict__ g_hw,
+                                                             const float *__restrict__ g_T,
+                                                             const double *__restrict__ y_obs, int obs_per,
+                                                             const double *__restrict__ eps_an, double eps_mn,
+                                                             const float *__restrict__ g_gates, float *__restrict__ grad,
+                                                             int *__restrict__ work_counter, float att0,
+                                                             const int8_t *__restrict__ valid) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int K2 = (K + 1) / 2;
     const size_t FL = (size_t)F * LS;
     ulonglong2 *RS = reinterpret_cast<ulonglong2 *>(smem_raw);
     ulonglong2 *lamp = RS + FL;
-    float2 *DS = reinterpret_cast<float2 *>(lamp + K2);
-    u64 *RY2 = reinterpret_cast<u64 *>(DS + FL * 4);
-    float2 *hwp = reinterpret_cast<float2 *>(RY2 + FL);
+    float4 *DS = reinterpret_cast<float4 *>(lamp + K2);
+    float2 *hwp = reinterpret_cast<float2 *>(DS + FL * 2);
     float *af = reinterpret_cast<float *>(hwp + K2);
     float *Ts = af + F;
     float *part = Ts + (size_t)G * F;
@@ -173,14 +191,16 @@ __global__ void __launch_bounds__(kGT, 3) loglik_grad_kernel(GradModels mv, int 
     __shared__ double dldy[AEM_MAX_GATES];
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const float mu0 = (float)kMu0, ln10 = 2.302585092994046f;
+    // lengths in the forward kernel's unit (aem_system::len)
+    const float mu0 = (float)kMu0 * len * len, ilen = 1.f / len, ln10 = 2.302585092994046f;
     for (int i = tid; i < G * F; i += blockDim.x) Ts[i] = g_T[i];
     // abscissa pairs (k, k + K2); an odd K pads the last pair with a zero weight
     for (int k = tid; k < K2; k += blockDim.x) {
         const int kb = k + K2 < K ? k + K2 : K - 1;
         const float la = g_lam[k], lb = g_lam[kb];
-        lamp[k] = make_ulonglong2(pk2(la * la, lb * lb), pk2(la, lb));
-        hwp[k] = make_float2(g_hw[k], k + K2 < K ? g_hw[kb] : 0.f);
+        lamp[k] = make_ulonglong2(pk2(la * la, lb * lb), pk2(0.70710678118654752f / la, 0.70710678118654752f / lb));
+        hwp[k] = make_float2(0.70710678118654752f / la * g_hw[k],
+                             k + K2 < K ? 0.70710678118654752f / lb * g_hw[kb] : 0.f);
     }
     const int FK2 = F * K2;
 
@@ -198,10 +218,10 @@ __global__ void __launch_bounds__(kGT, 3) loglik_grad_kernel(GradModels mv, int 
         if (tid < L) {
             const size_t o = (size_t)p * mv.lmax + tid;
             sig_s[tid] = exp10f(mv.logsig[o]);
-            const float h = exp10f(mv.logh[o]);
+            const float h = exp10f(mv.logh[o]) * ilen;
             thick[tid] = h;
-            const float a = -2.f * 1.44269504088896341f * h, b = -2.f * h;
-            HE[tid] = make_ulonglong2(pk2(a, a), pk2(b, b));
+            const float e = -1.41421356237309505f * 1.44269504088896341f * h;
+            HE[tid] = make_ulonglong2(pk2(e, e), pk2(e * 0.69314718055994531f, e * 0.69314718055994531f));
             m_s[tid] = mv.m[o];
             tau_s[tid] = exp10f(mv.logtau[o]);
             c_s[tid] = mv.c[o];
@@ -249,12 +269,11 @@ __global__ void __launch_bounds__(kGT, 3) loglik_grad_kernel(GradModels mv, int 
             const float2 iwm = make_float2(0.f, w * mu0);                 // i w mu0
             const float2 sv = cmul(iwm, sg);
             RS[(size_t)f * LS + n] = make_ulonglong2(pk2(sv.x, sv.x), pk2(sv.y, sv.y));
-            RY2[(size_t)f * LS + n] = pk2(sv.y * sv.y, sv.y * sv.y);
-            float2 *d = DS + ((size_t)f * LS + n) * 4;
-            d[0] = cmul(iwm, cscale(sg, ln10));
-            d[1] = cmul(iwm, dsg_dm);
-            d[2] = cmul(iwm, cmul(dsg_dx, dx_dlt));
-            d[3] = cmul(iwm, cmul(dsg_dx, dx_dc));
+            const float2 d0 = cmul(iwm, cscale(sg, ln10)), d1 = cmul(iwm, dsg_dm);
+            const float2 d2 = cmul(iwm, cmul(dsg_dx, dx_dlt)), d3 = cmul(iwm, cmul(dsg_dx, dx_dc));
+            float4 *d = DS + ((size_t)f * LS + n) * 2;
+            d[0] = make_float4(d0.x, d0.y, d1.x, d1.y);
+            d[1] = make_float4(d2.x, d2.y, d3.x, d3.y);
         }
         __syncthreads();
 
@@ -290,127 +309,108 @@ __global__ void __launch_bounds__(kGT, 3) loglik_grad_kernel(GradModels mv, int 
         }
         __syncthreads();
 
-        // ---- reverse sweep per pair of items, per-thread accumulators; the
-        // log10 h entries hold sum w Im(u_j tb_j) until the reduction applies
-        // -2 h_j ln10 (d Gamma_0 / d h_j = -2 u_j tb_j, tb_j as below)
-        float acc[MAXL * kNP];
-        for (int v = 0; v < L * kNP; ++v) acc[v] = 0.f;
-        C2x2 Gam[MAXL];
+        // ---- reverse sweep per pair of items, per-thread accumulators (one
+        // 16-byte access for the four that come together); acc_h holds the sum
+        // of Im(c 4 D P (lambda^2 + s)) until the reduction applies
+        // -2 sqrt(2) h_n ln10
+        float4 acc_s[MAXL];
+        float acc_h[MAXL];
+        for (int v = 0; v < L; ++v) {
+            acc_s[v] = make_float4(0.f, 0.f, 0.f, 0.f);
+            acc_h[v] = 0.f;
+        }
+        C2x2 Ns[MAXL], Ds[MAXL];
+        u64 Sc[MAXL];  // the powers of two of the scaled sweep
         int f = tid / K2, k = tid - (tid / K2) * K2;
         for (int item = tid; item < FK2; item += blockDim.x) {
-            const ulonglong2 lp = lamp[k];  // (lam^2 pair, lam pair)
-            const float2 hw = hwp[k];
-            const float a = af[f];
-            const u64 wgt = pk2(a * hw.x, a * hw.y);
+            const ulonglong2 lp = lamp[k];  // (lam^2 pair, 1 / (sqrt(2) lam) pair)
             const ulonglong2 *Sf = RS + (size_t)f * LS;
-            const u64 *Yf = RY2 + (size_t)f * LS;
-            const float2 *Df = DS + (size_t)f * LS * 4;
-            const C2x2 air = c2(lp.y, kZero2);  // u of the air: lambda
+            const float4 *Df = DS + (size_t)f * LS * 2;
             int Li = L;  // the layers this item runs
             if (cut) {
                 float l2, lb2;
                 up2(lp.x, l2, lb2);
                 Li = depth_layers(l2, TH + (size_t)f * LS, L);
             }
-            u64 imod;
-            // bottom-up: Gamma_j for every interface j
-            {
-                C2x2 ub = c2root(lp.x, Sf[Li - 1], Yf[Li - 1], imod);
-                for (int j = Li - 1; j >= 0; --j) {
-                    const ulonglong2 sb = Sf[j];
-                    C2x2 ua, dsab;  // u above the interface; s above minus s below
-                    if (j > 0) {
-                        const ulonglong2 sa = Sf[j - 1];
-                        ua = c2root(lp.x, sa, Yf[j - 1], imod);
-                        dsab = c2(sub2(sa.x, sb.x), sub2(sa.y, sb.y));
-                    } else {
-                        ua = air;
-                        dsab = c2(sub2(kZero2, sb.x), sub2(kZero2, sb.y));
-                    }
-                    const C2x2 rho = c2div(dsab, c2sq(c2add(ua, ub)));
-                    if (j == Li - 1) {
-                        Gam[j] = rho;
-                    } else {
-                        const C2x2 b = c2mul(Gam[j + 1], c2expm(HE[j], ub));
-                        Gam[j] = c2div(c2add(rho, b), c2add1(c2mul(rho, b)));
-                    }
-                    ub = ua;
-                }
-            }
-            // top-down: adjoints.  gbar = d Gamma_0 / d Gamma_j; sbar_p, ubar_p
-            // collect d Gamma_0 / d s_{j-1}, d / d u_{j-1} of the layer above
-            C2x2 gbar = c2(kOne2, kZero2), up = air, sbar_p = c2(kZero2, kZero2), ubar_p = sbar_p;
-            u64 imod_up = kZero2;
-            ulonglong2 sp = make_ulonglong2(kZero2, kZero2);
-            C2x2 uj = c2root(lp.x, Sf[0], Yf[0], imod);
-            for (int j = 0; j < Li; ++j) {
-                const ulonglong2 sj = Sf[j];
-                const C2x2 q = c2add(up, uj);
-                const u64 iqn = c2inorm(q);
-                const C2x2 iqc = c2scale(q, iqn);  // conj(1 / q)
-                const C2x2 iq2c = c2sq(iqc);       // conj(1 / q^2)
-                const C2x2 rho = c2mulc(c2(sub2(sp.x, sj.x), sub2(sp.y, sj.y)), iq2c);
-                C2x2 rbar, ubar_j = c2(kZero2, kZero2), gnext = ubar_j;
-                if (j < Li - 1) {
-                    const ulonglong2 he = HE[j];
-                    const C2x2 E = c2expm(he, uj);
-                    const C2x2 b = c2mul(Gam[j + 1], E);
-                    // d Gamma_j / d rho = (1 - b^2) / den^2, d Gamma_j / d b = (1 - rho^2) / den^2
-                    const C2x2 g2 = c2div(gbar, c2sq(c2add1(c2mul(rho, b))));
-                    rbar = c2mul(g2, c2one_minus_sq(b));
-                    const C2x2 tbar = c2mul(g2, c2one_minus_sq(rho));
-                    // tb = tbar b = (d Gamma_0 / d E_j) E_j: d / d u_j through E_j is -2 h tb
-                    const C2x2 tb = c2mul(tbar, b);
-                    gnext = c2mul(tbar, E);
-                    float h0, h1;
-                    up2(mul2(wgt, fma2(uj.re, tb.im, mul2(uj.im, tb.re))), h0, h1);
-                    acc[j * kNP + 1] += h0 + h1;
-                    ubar_j = c2scale(tb, he.y);
-                } else {
-                    rbar = gbar;
-                }
-                // d rho / d u_{j-1} = d rho / d u_j = -2 rho / q; d rho / d s_{j-1} = 1 / q^2 = -d rho / d s_j
-                // dq2 = rbar rho / q, so the rho term of d / d u is -2 dq2
-                const C2x2 dq2 = c2mul(rbar, c2mulc(rho, iqc));
-                const C2x2 rbi = c2mulc(rbar, iq2c);
-                if (j > 0) {
-                    // layer j-1 complete: s enters through u as well, du/ds = 1 / (2 u) = conj(u) / (2 |z|)
-                    ubar_p = c2(fma2(dq2.re, kMinus2, ubar_p.re), fma2(dq2.im, kMinus2, ubar_p.im));
-                    sbar_p = c2add(c2add(sbar_p, rbi), c2scale(c2mulc(ubar_p, up), imod_up));
-                    float x0, x1, y0, y1;
-                    up2(mul2(wgt, sbar_p.re), x0, x1);
-                    up2(mul2(wgt, sbar_p.im), y0, y1);
-                    const float swx = x0 + x1, swy = y0 + y1;
-                    const float4 *d = reinterpret_cast<const float4 *>(Df + (size_t)(j - 1) * 4);
-                    const float4 d01 = d[0], d23 = d[1];
-                    float *ac = acc + (j - 1) * kNP;
-                    ac[0] += fmaf(swx, d01.y, swy * d01.x);
-                    ac[2] += fmaf(swx, d01.w, swy * d01.z);
-                    ac[3] += fmaf(swx, d23.y, swy * d23.x);
-                    ac[4] += fmaf(swx, d23.w, swy * d23.z);
-                }
-                sbar_p = c2neg(rbi);
-                ubar_p = c2(fma2(dq2.re, kMinus2, ubar_j.re), fma2(dq2.im, kMinus2, ubar_j.im));
-                up = uj;
-                imod_up = imod;
-                sp = sj;
-                gbar = gnext;
-                if (j + 1 < Li) uj = c2root(lp.x, Sf[j + 1], Yf[j + 1], imod);
-            }
-            {
-                sbar_p = c2add(sbar_p, c2scale(c2mulc(ubar_p, up), imod_up));
+            auto emit = [&](int n, C2x2 t) {
                 float x0, x1, y0, y1;
-                up2(mul2(wgt, sbar_p.re), x0, x1);
-                up2(mul2(wgt, sbar_p.im), y0, y1);
+                up2(t.re, x0, x1);
+                up2(t.im, y0, y1);
                 const float swx = x0 + x1, swy = y0 + y1;
-                const float4 *d = reinterpret_cast<const float4 *>(Df + (size_t)(Li - 1) * 4);
-                const float4 d01 = d[0], d23 = d[1];
-                float *ac = acc + (Li - 1) * kNP;
-                ac[0] += fmaf(swx, d01.y, swy * d01.x);
-                ac[2] += fmaf(swx, d01.w, swy * d01.z);
-                ac[3] += fmaf(swx, d23.y, swy * d23.x);
-                ac[4] += fmaf(swx, d23.w, swy * d23.z);
-            }
+                const float4 d01 = Df[2 * n], d23 = Df[2 * n + 1];
+                float4 ac = acc_s[n];
+                ac.x += fmaf(swx, d01.y, swy * d01.x);
+                ac.y += fmaf(swx, d01.w, swy * d01.z);
+                ac.z += fmaf(swx, d23.y, swy * d23.x);
+                ac.w += fmaf(swx, d23.w, swy * d23.z);
+                acc_s[n] = ac;
+            };
+            // false: D_0 has left the range in which the squares of every
+            // layer's amplitudes stay normal FP32 numbers, and nothing was
+            // added: many thick layers of alternating contrast, where each
+            // interface multiplies D by up to the contrast of w.  The scaled
+            // sweep then brings every (N_n, D_n) back to about one by a power
+            // of two; done always, it costs 5 %.
+            auto sweep = [&](auto sc) -> bool {
+                constexpr bool SCALED = decltype(sc)::value;
+                // bottom-up
+                u64 im;
+                Root w = root2_inv(lp.x, Sf[Li - 1], im);
+                C2x2 e = c2(kOne2, kZero2), h = c2(w.re, w.im);
+                for (int n = Li - 2; n >= 0; --n) {
+                    w = root2_inv(lp.x, Sf[n], im);
+                    const C2x2 g = c2mulc(h, c2(mul2(w.re, im), mul2(w.im, im)));
+                    C2x2 N = c2(fma2(kMinusHalf2, g.re, e.re), fma2(kMinusHalf2, g.im, e.im));
+                    C2x2 D = c2(fma2(kHalf2, g.re, e.re), fma2(kHalf2, g.im, e.im));
+                    if constexpr (SCALED) {
+                        const u64 q = pow2_inv2(D);
+                        N = c2(mul2(N.re, q), mul2(N.im, q));
+                        D = c2(mul2(D.re, q), mul2(D.im, q));
+                        Sc[n] = q;
+                    }
+                    Ns[n] = N;
+                    Ds[n] = D;
+                    const C2x2 P = c2mul(N, c2expm<false>(HE[n], w));
+                    e = c2(add2(D.re, P.re), add2(D.im, P.im));
+                    h = c2mul(c2(w.re, w.im), c2(sub2(D.re, P.re), sub2(D.im, P.im)));
+                }
+                const C2x2 D0 = c2(fma2(h.re, lp.y, e.re), fma2(h.im, lp.y, e.im));
+                float d0, d1;
+                up2(fma2(D0.re, D0.re, mul2(D0.im, D0.im)), d0, d1);
+                if (!SCALED && !(d0 > 1e-24f && d1 > 1e-24f && d0 < 1e30f && d1 < 1e30f)) return false;
+                const float2 hw = hwp[k];
+                const float a = af[f];
+                const u64 i = pk2(rcp_approx(d0), rcp_approx(d1)), wgt = pk2(a * hw.x, a * hw.y);
+                C2x2 c = c2sq(c2(mul2(D0.re, i), sub2(kZero2, mul2(D0.im, i))));
+                c = c2(mul2(c.re, wgt), mul2(c.im, wgt));
+                // top-down
+                for (int n = 0; n < Li - 1; ++n) {
+                    const ulonglong2 he = HE[n], sv = Sf[n];
+                    w = root2_inv(lp.x, sv, im);
+                    const C2x2 E4 = c2expm<true>(he, w), N = Ns[n], D = Ds[n];
+                    const C2x2 P4 = c2mul(N, E4), D2 = c2sq(D), NP4 = c2mul(N, P4), T4 = c2mul(D, P4);
+                    // -(1 - E) (D^2 + N P) 2 / w - sqrt(2) h 4 T
+                    C2x2 A = c2mul(c2(fma2(NP4.re, kQuarter2, D2.re), fma2(NP4.im, kQuarter2, D2.im)),
+                                   c2(fma2(E4.re, kQuarter2, kMinusOne2), mul2(E4.im, kQuarter2)));
+                    A = c2mulc(A, c2(mul2(w.re, im), mul2(w.im, im)));
+                    A = c2(fma2(he.y, T4.re, A.re), fma2(he.y, T4.im, A.im));
+                    emit(n, c2mul(c, A));
+                    const C2x2 cT = c2mul(c, T4);
+                    float h0, h1;
+                    up2(fma2(cT.im, add2(lp.x, sv.x), mul2(cT.re, sv.y)), h0, h1);
+                    acc_h[n] += h0 + h1;
+                    c = c2mul(c, E4);
+                    if constexpr (SCALED) {
+                        const u64 q = mul2(Sc[n], Sc[n]);
+                        c = c2(mul2(c.re, q), mul2(c.im, q));
+                    }
+                }
+                w = root2_inv(lp.x, Sf[Li - 1], im);
+                const u64 ni = sub2(kZero2, im);
+                emit(Li - 1, c2mulc(c, c2(mul2(w.re, ni), mul2(w.im, ni))));
+                return true;
+            };
+            if (!sweep(std::false_type{})) sweep(std::true_type{});
             k += blockDim.x;
             while (k >= K2) {
                 k -= K2;
@@ -418,16 +418,25 @@ __global__ void __launch_bounds__(kGT, 3) loglik_grad_kernel(GradModels mv, int 
             }
         }
         // CTA reduction of the per-thread accumulators (fixed order)
-        for (int v = 0; v < L * kNP; ++v) {
-            const float s = wsum<float>(acc[v]);
-            if (lane == 0) part[warp * LS * kNP + v] = s;
+        for (int n = 0; n < L; ++n) {
+            const float4 ac = acc_s[n];
+            const float s0 = wsum<float>(ac.x), s1 = wsum<float>(acc_h[n]), s2 = wsum<float>(ac.y),
+                        s3 = wsum<float>(ac.z), s4 = wsum<float>(ac.w);
+            if (lane == 0) {
+                float *q = part + (warp * LS + n) * kNP;
+                q[0] = s0;
+                q[1] = s1;
+                q[2] = s2;
+                q[3] = s3;
+                q[4] = s4;
+            }
         }
         __syncthreads();
         for (int v = tid; v < mv.lmax * kNP; v += blockDim.x) {
             float s = 0.f;
             if (v < L * kNP) {
                 for (int w = 0; w < kGW; ++w) s += part[w * LS * kNP + v];
-                if (v % kNP == 1) s *= -2.f * thick[v / kNP] * ln10;
+                if (v % kNP == 1) s *= -2.f * 1.41421356237309505f * thick[v / kNP] * ln10;
             }
             grad[(size_t)p * mv.lmax * kNP + v] = s;
         }
@@ -471,8 +480,8 @@ int loglik_grad_f32_soundings(const aem_system *sys, const aem_models_f32 *model
     if (rc == AEM_OK) {
         e = cudaMemsetAsync(counter, 0, sizeof(int), stream);
         if (e == cudaSuccess) {
-            kern<<<(unsigned)grid, kGT, smem, stream>>>(gm, h.F, h.G, h.K, LS, h.cc_form, sys->d_omega_f, sys->d_lam_f,
-                                                        sys->d_hw_f, sys->d_T_f, y_obs, models_per_sounding, eps_an,
+            kern<<<(unsigned)grid, kGT, smem, stream>>>(gm, h.F, h.G, h.K, LS, h.cc_form, sys->len, sys->d_omega_f,
+                                                        sys->d_lamu_f, sys->d_hw_f, sys->d_T_f, y_obs, models_per_sounding, eps_an,
                                                         eps_mn, gates, grad, counter, sys->depth_att, valid);
             e = cudaGetLastError();
         }
