@@ -618,7 +618,8 @@ __global__ void __launch_bounds__(kGroupThreads) reweight_kernel(const RwArgs a)
         double s1 = 0.0, s2 = 0.0;
         if (tid < M) {
             const int qa = max(so[tid], lo_pos) - lo_pos, qb = min(so[tid + 1], hi_pos) - lo_pos;
-            for (int i = qa >> 5; 32 * i < qb; ++i) {
+            // a model that begins past the slice's end, in its last block, has no entry there
+            for (int i = qa >> 5; qa < qb && 32 * i < qb; ++i) {
                 s1 += b1[i + tid];
                 s2 += b2[i + tid];
             }

@@ -97,3 +97,41 @@ def test_resample_edges(n, models, kind):
         thr = np.array([(j * one + int(u40[k])) // m for j in range(m)], dtype=np.int64)
         ref[idx] = idx[np.searchsorted(C, thr, side="right")]
     assert np.array_equal(got, ref)
+
+
+@pytest.mark.parametrize("n", [1024, 1300, 1396, 4001, 9600])
+@pytest.mark.parametrize("shift", [0, 1, 7, 31])
+def test_models_beginning_past_a_slice(n, shift):
+    """Models that begin `shift` positions past the end of each of the eight
+    cluster slices, after another population's sums went through the same
+    shared memory: such a model has no share in that slice."""
+    import torch
+    from paper_2109_00661_gb300 import smc as S
+    rng = np.random.default_rng(n)
+    at = np.unique(np.minimum(np.arange(1, 8) * n // 8 + shift, n - 1))
+    models = at.size + 1
+    model = np.searchsorted(at, np.arange(n), side="right")
+    ll = -20.0 / rng.random(n)
+
+    def call(ll, model, models, alpha):
+        return S.reweight(torch.as_tensor(ll, device="cuda"), torch.as_tensor(model.astype(np.int32), device="cuda"),
+                          models, 0.0, alpha)
+
+    def sums(x):
+        top = np.full(models, -np.inf)
+        np.maximum.at(top, model, ll)
+        e = np.exp(x * (ll - top[model]))
+        return e, np.bincount(model, e, models), np.bincount(model, e * e, models)
+
+    lo, hi = 0.0, 1.0
+    for _ in range(60):
+        mid = 0.5 * (lo + hi)
+        _, s1, s2 = sums(mid)
+        lo, hi = (mid, hi) if np.sum(s1**2 / s2) >= 0.9 * n else (lo, mid)
+    big = -rng.random(16384)  # leaves exponentials near one behind on every SM
+    for _ in range(64):
+        call(big, rng.integers(0, 20, 16384), 20, 0.5)
+        dg, _, _, W = call(ll, model, models, 0.9)
+        assert abs(dg.item() - lo) <= 1e-10 * lo
+    e, s1, _ = sums(lo)
+    assert np.allclose(W.cpu().numpy(), e / s1[model], rtol=1e-8, atol=1e-14)
