@@ -13,6 +13,7 @@ namespace aem {
 
 constexpr double kPi = 3.14159265358979323846;
 constexpr double kMu0 = 4e-7 * kPi;
+constexpr int kTab64Turn = 1024, kTab64Octave = 256;  // entries of the FP64 forward kernel's tables (d_tab64)
 
 // Records the message returned by aem_last_error() and passes the code through.
 int fail(int code, const std::string &msg);
@@ -71,6 +72,9 @@ struct aem_system {
     // the FP32 forward kernel's length unit (a power of two, metres) and its
     // abscissae in it
     float len = 1.f, *d_lamu_f = nullptr;
+    // the FP64 forward kernel's tables: sine and cosine of 2 pi j / kTab64Turn in
+    // pairs, then 2^(j / kTab64Octave)
+    double *d_tab64 = nullptr;
     double *d_omega_d = nullptr, *d_lam_d = nullptr, *d_hw_d = nullptr, *d_T_d = nullptr;
     int num_sms = 0;
     // device status word: kernels record AEM_ERR_TIMEOUT here when a bounded

@@ -56,156 +56,144 @@ struct ModelsView {
 // of FP64 operations, and everything else is free: roots and reciprocals take
 // the hardware's 20-bit estimates and one third-order step, the exponential and
 // the sine and cosine a table in shared memory and a short polynomial, signs,
-// exponents and table indices integer instructions.  About 70 FP64 operations
-// per layer-step (154 with the library's sqrt, rsqrt, division, exp and
-// sincos): 1,024 models of 1..10 layers, 60 frequencies, 200 abscissae, 20.0
-// -> 9.06 ms, at the rate the FP64 pipe allows (71 operations of 19.4 cycles a
-// warp: 9.2 ms).
+// exponents and table indices integer instructions.  53 FP64 operations per
+// layer-step (154 with the library's sqrt, rsqrt, division, exp and sincos, 71
+// with interface coefficients and 64-entry tables): 1,024 models of 1..10
+// layers, 60 frequencies, 200 abscissae, 20.0 -> 9.06 -> 7.06 ms, at the rate the
+// FP64 pipe allows.
 //
-// The recursion is the FP32 kernel's (w = sqrt(2) u, the interface coefficient
-// from the roots and their moduli).
+// The recursion carries the tangential field e and h = w (D - P) upwards, with
+// w = sqrt(2) u, D and N = R D the down- and upgoing amplitudes at the bottom
+// of a layer and P = N E: both are continuous across an interface, where
+//   D = w e + h,  N = w e - h,  then  e = D + N E,  h = w (D - N E)
+// (scaled by w at every interface, which 64-bit exponents hold; no interface
+// coefficient and no division), and R_0 = (w_air e - h) / (w_air e + h).
 namespace f64 {
 
-// 1 / sqrt(v) and 1 / v, v > 0 normal: y (1 + e (1/2 + 3/8 e)), e = 1 - v y^2,
-// and y (1 + e + e^2), e = 1 - v y, leave 5/16 e^3 and e^3 of e < 2^-18.
-__device__ __forceinline__ double rsq(double v) {
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(v));
-    const double e = fma(-(v * y), y, 1.0);
-    return fma(fma(e, 0.375, 0.5), e * y, y);
-}
-__device__ __forceinline__ double rcp(double v) {
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(v));
-    const double e = fma(-v, y, 1.0);
-    return fma(fma(e, e, e), y, y);
-}
-
-// Tables of the complex exponential (Tang 1989's scheme): 2^(j/64), and sine
-// and cosine of j pi / 32.
-struct Tables {
-    double ex[64];
-    double2 sc[64];
-};
-__device__ inline void fill(Tables *t) {
-    for (int j = threadIdx.x; j < 64; j += blockDim.x) {
-        t->ex[j] = exp2(j * 0.015625);
-        sincospi(j * 0.03125, &t->sc[j].x, &t->sc[j].y);
-    }
-}
-
+constexpr int kExN = kTab64Octave, kScN = kTab64Turn;
 constexpr double kShift = 6755399441055744.0;  // 1.5 * 2^52: the low word of x + kShift is round(x)
 
-// exp(x) for x <= 0 (0 below -700): x = k ln2 / 64 + r, |r| < 0.0055, and
-// e^r - 1 to r^5 (the next term is 4e-17).
-__device__ __forceinline__ double exp_neg(double x, const Tables *t) {
-    const double n = fma(x, 92.332482616893657, kShift);  // 64 / ln 2
-    const int k = __double2loint(n);
-    const double kd = n - kShift;
-    // ln2 / 64, its leading 32 bits and the rest
-    double r = fma(kd, -1.08304246932675596326e-02, x);
-    r = fma(kd, -2.98158582698529370e-12, r);
-    const double r2 = r * r;
-    double q = fma(r, 1.0 / 120.0, 1.0 / 24.0);
-    q = fma(q, r, 1.0 / 6.0);
-    q = fma(q, r, 0.5);
-    const double T = t->ex[k & 63];
-    const double e = fma(fma(r2, q, r), T, T);
-    // -inf <= x <= -700, from the high word's range
-    const bool gone = (unsigned)__double2hiint(x) - 0xc085e000u <= 0xfff00000u - 0xc085e000u;
-    const unsigned hi = (unsigned)__double2hiint(e) + ((unsigned)(k >> 6) << 20);
-    return gone ? 0.0 : __hiloint2double((int)hi, __double2loint(e));
-}
-
-// sine and cosine of x = k pi / 32 + r, |r| < 0.0491: r's to r^7 and r^8, then
-// the table's angle by the addition theorems.
-__device__ __forceinline__ void sincos_tab(double x, const Tables *t, double *s, double *c) {
-    const double n = fma(x, 10.185916357881302, kShift);  // 32 / pi
-    const int k = __double2loint(n);
-    const double kd = n - kShift;
-    // pi / 32 as two doubles; the first product is exact in the fused step
-    double r = fma(kd, -0.098174770424681035, x);
-    r = fma(kd, -3.8270212473354788e-18, r);
-    const double r2 = r * r;
-    double p = fma(r2, -1.0 / 5040.0, 1.0 / 120.0);
-    p = fma(p, r2, -1.0 / 6.0);
-    const double sr = fma(p * r2, r, r);
-    double q = fma(r2, 1.0 / 40320.0, -1.0 / 720.0);
-    q = fma(q, r2, 1.0 / 24.0);
-    q = fma(q, r2, -0.5);
-    const double cr = q * r2;  // cos r - 1
-    const double2 a = t->sc[k & 63];
-    *s = fma(a.y, sr, fma(a.x, cr, a.x));
-    *c = fma(-a.x, sr, fma(a.y, cr, a.y));
-}
-
-struct Root {  // w = sqrt(2 (x + i y)), m = |w|^2 / 2
-    double re, im, m;
+// Tables of the complex exponential (Tang 1989's scheme): 2^(j / kExN), sine
+// and cosine of 2 pi j / kScN (kTabDoubles in this order, forward_f64_tables).
+struct Tables {
+    double2 sc[kScN];
+    double ex[kExN];
 };
+
+// Per layer: -sqrt(2) h, and it in the tables' steps (times kExN / ln 2 and
+// kScN / (2 pi)).
+struct Thick {
+    double h, he, hp;
+};
+
+// E = exp(-sqrt(2) h w).  With k the nearest step, the fused x h' - k is the
+// exact remainder f, |f| <= 1/2; e^(f ln2 / 256) - 1 to f^4 (the next term is
+// 4e-17), sin and cos of f pi / 512 to f^5 and f^4 (5e-22, 1e-18).
+__device__ __forceinline__ void exp_c(double wre, double wim, const Thick &t, const Tables *tab, double &Ex,
+                                      double &Ey) {
+    constexpr double a = 0.69314718055994530942 / kExN, b = 6.28318530717958647693 / kScN;
+    const double n = fma(t.he, wre, kShift);
+    const int k = __double2loint(n);
+    const double f = fma(t.he, wre, kShift - n);
+    double q = fma(f, a * a * a * a / 24.0, a * a * a / 6.0);
+    q = fma(q, f, a * a / 2.0);
+    q = fma(q, f, a);
+    const double T = tab->ex[k & (kExN - 1)];
+    double e = fma(q * f, T, T);
+    e = __hiloint2double(__double2hiint(e) + (int)((unsigned)(k >> 8) << 20), __double2loint(e));
+    // below exp(-700): the steps themselves, from n's bits (a NaN stays)
+    constexpr long long kGone = 0x4338000000000000ll - 258530;
+    const bool gone = __double_as_longlong(n) < kGone;
+    const double m = fma(t.hp, wim, kShift);
+    double sn, cs;
+    if ((unsigned)(__double2hiint(m) - 0x43380000 + 0x20000) < 0x40000u) {  // |steps| < 2^49
+        const double g = fma(t.hp, wim, kShift - m), g2 = g * g;
+        double p = fma(g2, b * b * b * b * b / 120.0, -b * b * b / 6.0);
+        p = fma(p, g2, b);
+        const double sr = p * g;
+        const double cr = fma(g2, b * b * b * b / 24.0, -b * b / 2.0) * g2;  // cos - 1
+        const double2 v = tab->sc[__double2loint(m) & (kScN - 1)];
+        sn = fma(v.y, sr, fma(v.x, cr, v.x));
+        cs = fma(-v.x, sr, fma(v.y, cr, v.y));
+    } else {
+        sincos(t.h * wim, &sn, &cs);
+    }
+    Ex = gone ? 0.0 : e * cs;
+    Ey = gone ? 0.0 : e * sn;
+}
+
 struct Rec {  // per frequency and layer
     double sx, sy, sy2;
 };
-
-__device__ __forceinline__ Root root(double lam2, const Rec &s) {
-    const double x = lam2 + s.sx;
-    const double v = fma(x, x, s.sy2);
-    Root w;
-    w.m = v * rsq(v);
-    const double t = w.m + fabs(x), rr = rsq(t), p = t * rr, o = s.sy * rr;
-    const bool pos = __double2hiint(x) >= 0;
-    w.re = pos ? p : o;
-    w.im = pos ? o : p;
-    return w;
-}
-
 struct C {
     double x, y;
 };
 
-// (u_a - u_b) / (u_a + u_b)
-__device__ __forceinline__ C coef(const Root &a, const Root &b) {
-    const double i = rcp(fma(a.im, b.im, fma(a.re, b.re, a.m + b.m)));
-    return {(a.m - b.m) * i, fma(a.im, b.re, -(a.re * b.im)) * i};
+// w = sqrt(2 (x + i y)).  From the 20-bit estimate y of 1 / sqrt(v), g = v y and
+// e = 1 - g y: sqrt(v) = g (1 + c) and 1 / sqrt(v) = y (1 + c) with c = e (1/2 +
+// 3/8 e), up to 5/16 e^3 < 2^-55.
+__device__ __forceinline__ double rsq_est(double v) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(v));
+    return y;
+}
+__device__ __forceinline__ C root(double lam2, const Rec &s) {
+    const double x = lam2 + s.sx;
+    const double v = fma(x, x, s.sy2);
+    const double y1 = rsq_est(v), g1 = v * y1, e1 = fma(-g1, y1, 1.0);
+    const double m = fma(e1 * fma(e1, 0.375, 0.5), g1, g1);
+    const double t = m + fabs(x);
+    const double y2 = rsq_est(t), g2 = t * y2, e2 = fma(-g2, y2, 1.0);
+    const double c = e2 * fma(e2, 0.375, 0.5);
+    const double p = fma(c, g2, g2), o = s.sy * fma(c, y2, y2);
+    const bool pos = __double2hiint(x) >= 0;
+    return {pos ? p : o, pos ? o : p};
 }
 
-// Im R_0 of one (lambda, frequency); rec: the frequency's layers, ha: -sqrt(2) h.
+// Im R_0 of one (lambda, frequency); rec: the frequency's layers.
 __device__ __forceinline__ double im_r0(double lam2, double wair, const Rec *__restrict__ rec,
-                                        const double *__restrict__ ha, int L, const Tables *t) {
-    Root b = root(lam2, rec[L - 1]);
-    C N = {0.0, 0.0}, D = {1.0, 0.0};
+                                        const Thick *__restrict__ th, int L, const Tables *tab) {
+    C h = root(lam2, rec[L - 1]), D, N;
+    if (L == 1) {
+        D = {wair + h.x, h.y};
+        N = {wair - h.x, -h.y};
+    } else {
+        C w = root(lam2, rec[L - 2]), e;
+        D = {w.x + h.x, w.y + h.y};
+        N = {w.x - h.x, w.y - h.y};
 #pragma unroll 1
-    for (int n = L - 2; n >= -1; --n) {
-        Root a;
-        if (n >= 0)
-            a = root(lam2, rec[n]);
-        else
-            a = {wair, 0.0, lam2};
-        const C r = coef(a, b);
-        if (n == L - 2) {
-            N = r;
-        } else {
-            const double h = ha[n + 1], ph = h * b.im;
-            const double e = exp_neg(h * b.re, t);
-            double sn, cs;
-            if ((__double2hiint(ph) & 0x7fffffff) < 0x41900000)  // |phase| < 2^26
-                sincos_tab(ph, t, &sn, &cs);
-            else
-                sincos(ph, &sn, &cs);
-            const C E = {e * cs, e * sn};
-            const C P = {fma(N.x, E.x, -(N.y * E.y)), fma(N.x, E.y, N.y * E.x)};
-            const C N1 = {fma(r.x, D.x, fma(-r.y, D.y, P.x)), fma(r.x, D.y, fma(r.y, D.x, P.y))};
-            D = {fma(r.x, P.x, fma(-r.y, P.y, D.x)), fma(r.x, P.y, fma(r.y, P.x, D.y))};
-            N = N1;
+        for (int n = L - 2;; --n) {
+            double Ex, Ey;
+            exp_c(w.x, w.y, th[n], tab, Ex, Ey);
+            e = {fma(N.x, Ex, fma(-N.y, Ey, D.x)), fma(N.x, Ey, fma(N.y, Ex, D.y))};
+            const C b = {fma(2.0, D.x, -e.x), fma(2.0, D.y, -e.y)};
+            h = {fma(w.x, b.x, -(w.y * b.y)), fma(w.x, b.y, w.y * b.x)};
+            if (n == 0) break;
+            w = root(lam2, rec[n - 1]);
+            D = {fma(w.x, e.x, fma(-w.y, e.y, h.x)), fma(w.x, e.y, fma(w.y, e.x, h.y))};
+            N = {fma(-2.0, h.x, D.x), fma(-2.0, h.y, D.y)};
         }
-        b = a;
+        D = {fma(wair, e.x, h.x), fma(wair, e.y, h.y)};
+        N = {fma(-2.0, h.x, D.x), fma(-2.0, h.y, D.y)};
     }
-    return fma(N.y, D.x, -(N.x * D.y)) * rcp(fma(D.x, D.x, D.y * D.y));
+    // |D| to about one by a power of two: the squares stay in range
+    const int top = max(__double2hiint(D.x) & 0x7ff00000, __double2hiint(D.y) & 0x7ff00000);
+    const double z = __hiloint2double(min(max(0x7fe00000 - top, 0x00100000), 0x7fd00000), 0);
+    D = {D.x * z, D.y * z};
+    N = {N.x * z, N.y * z};
+    const double v = fma(D.x, D.x, D.y * D.y);
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(v));
+    const double r = fma(-v, y, 1.0);  // 1 / v = y (1 + r + r^2 + ..)
+    return fma(N.y, D.x, -(N.x * D.y)) * fma(fma(r, r, r), y, y);
 }
 
 }  // namespace f64
 
 constexpr int kThreads64 = 256;
 constexpr int kChunk64 = 8;  // frequencies whose items share the value buffer
+constexpr int kTab64Doubles = (int)(sizeof(f64::Tables) / sizeof(double));
+static_assert(kTab64Doubles == 2 * kTab64Turn + kTab64Octave && kTab64Octave == 256, "");
 
 // Shared memory (dynamic): vals [kChunk64 * K], lam2 [K], wair [K], hw [K],
 // rec [kChunk64 * lmax], imh [F].
@@ -223,6 +211,7 @@ __global__ void __launch_bounds__(kThreads64) forward_f64_kernel(ModelsView<doub
                                                                const double *__restrict__ g_lam,
                                                                const double *__restrict__ g_hw,
                                                                const double *__restrict__ g_T,
+                                                               const double *__restrict__ g_tab,
                                                                double *__restrict__ gates_out,
                                                                double *__restrict__ imh_out,
                                                                const double *__restrict__ y_obs, int obs_per,
@@ -241,12 +230,12 @@ __global__ void __launch_bounds__(kThreads64) forward_f64_kernel(ModelsView<doub
     double *lam2 = vals + (size_t)kChunk64 * K, *wair = lam2 + K, *hw = wair + K, *imh = hw + K;
     f64::Rec *rec = reinterpret_cast<f64::Rec *>(imh + F);
     __shared__ f64::Tables tab;
-    __shared__ double lsig[AEM_MAX_LAYERS], lm[AEM_MAX_LAYERS], ltau[AEM_MAX_LAYERS], lc[AEM_MAX_LAYERS],
-        ha[AEM_MAX_LAYERS];
+    __shared__ double lsig[AEM_MAX_LAYERS], lm[AEM_MAX_LAYERS], ltau[AEM_MAX_LAYERS], lc[AEM_MAX_LAYERS];
+    __shared__ f64::Thick th[AEM_MAX_LAYERS];
     __shared__ double ll_part[2];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int L = mv.nlayers[p];
-    f64::fill(&tab);
+    for (int j = tid; j < kTab64Doubles; j += kThreads64) reinterpret_cast<double *>(&tab)[j] = g_tab[j];
     for (int k = tid; k < K; k += kThreads64) {
         const double l = g_lam[k];
         lam2[k] = l * l;
@@ -256,7 +245,8 @@ __global__ void __launch_bounds__(kThreads64) forward_f64_kernel(ModelsView<doub
     if (tid < L) {
         const size_t o = (size_t)p * mv.lmax + tid;
         lsig[tid] = exp10(mv.logsig[o]);
-        ha[tid] = -1.4142135623730951 * exp10(mv.logh[o]);
+        const double h = -1.4142135623730951 * exp10(mv.logh[o]);
+        th[tid] = {h, h * (f64::kExN / 0.69314718055994530942), h * (f64::kScN / 6.28318530717958647693)};
         lm[tid] = mv.m[o];
         ltau[tid] = exp10(mv.logtau[o]);
         lc[tid] = mv.c[o];
@@ -302,7 +292,7 @@ __global__ void __launch_bounds__(kThreads64) forward_f64_kernel(ModelsView<doub
         __syncthreads();
         int f = tid / K, k = tid - f * K;
         for (int item = tid; item < nf * K; item += kThreads64) {
-            vals[item] = hw[k] * f64::im_r0(lam2[k], wair[k], rec + f * L, ha, L, &tab);
+            vals[item] = hw[k] * f64::im_r0(lam2[k], wair[k], rec + f * L, th, L, &tab);
             k += kThreads64;
             while (k >= K) {
                 k -= K;
@@ -400,7 +390,8 @@ int launch_forward_f64(const aem_system *sys, const aem_models_f64 *models, doub
     cfg.numAttrs = C > 1 ? 1 : 0;
     AEM_CUDA_TRY(cudaLaunchKernelEx(&cfg, forward_f64_kernel, mv, h.F, h.G, h.K, h.cc_form,
                                     (const double *)sys->d_omega_d, (const double *)sys->d_lam_d,
-                                    (const double *)sys->d_hw_d, (const double *)sys->d_T_d, gates, imh, y_obs, obs_per,
+                                    (const double *)sys->d_hw_d, (const double *)sys->d_T_d, (const double *)sys->d_tab64, gates,
+                                    imh, y_obs, obs_per,
                                     eps_an, eps_mn, ll, active, valid));
     return AEM_OK;
 }

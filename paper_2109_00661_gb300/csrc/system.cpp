@@ -306,10 +306,18 @@ extern "C" int aem_system_create(const aem_system_desc *desc, aem_system **out) 
     std::vector<double> lamu(h.lam);
     for (double &l : lamu) l *= len;
     s->len = (float)len;
+    std::vector<double> tab64(2 * kTab64Turn + kTab64Octave);
+    for (int j = 0; j < kTab64Turn; ++j) {
+        const long double a = 6.283185307179586476925286766559L * j / kTab64Turn;
+        tab64[2 * j] = (double)std::sin(a);
+        tab64[2 * j + 1] = (double)std::cos(a);
+    }
+    for (int j = 0; j < kTab64Octave; ++j)
+        tab64[2 * kTab64Turn + j] = (double)std::exp2((long double)j / kTab64Octave);
     if ((rc = upload(&s->d_omega_f, h.omega)) || (rc = upload(&s->d_lam_f, h.lam)) || (rc = upload(&s->d_hw_f, h.hw)) ||
         (rc = upload(&s->d_T_f, h.T)) || (rc = upload(&s->d_omega_d, h.omega)) || (rc = upload(&s->d_lam_d, h.lam)) ||
         (rc = upload(&s->d_hw_d, h.hw)) || (rc = upload(&s->d_T_d, h.T)) ||
-        (rc = upload(&s->d_lamu_f, lamu))) {
+        (rc = upload(&s->d_lamu_f, lamu)) || (rc = upload(&s->d_tab64, tab64))) {
         aem_system_destroy(s);
         return rc;
     }
@@ -326,7 +334,7 @@ extern "C" int aem_system_create(const aem_system_desc *desc, aem_system **out) 
 extern "C" int aem_system_destroy(aem_system *s) {
     if (!s) return AEM_OK;
     void *ptrs[] = {s->d_omega_f, s->d_lam_f, s->d_hw_f, s->d_T_f,
-                    s->d_omega_d, s->d_lam_d, s->d_hw_d, s->d_T_d, s->d_lamu_f, s->d_status};
+                    s->d_omega_d, s->d_lam_d, s->d_hw_d, s->d_T_d, s->d_lamu_f, s->d_tab64, s->d_status};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     delete s;
