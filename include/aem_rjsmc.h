@@ -156,11 +156,15 @@ int aem_loglik_f64(const aem_system *sys, const aem_models_f64 *models, const do
  * 1 = 128 x 8, 2 = 512 x 2, 3 = 256 x 3, 4 = 128 x 6 (the register budget per
  * thread follows from the pair), each with a fixed grid-stride order of
  * models (a recorded 0, the default, stands for "none chosen": launches take
- * shape 2 for at most two models per SM and shape 1 above); 5..9 = the same five with dynamic scheduling (a CTA claims its
- * next model from a counter in stream-ordered scratch when it finishes one).  aem_autotune_forward times every shape that
- * fits on an SM on the caller's sample batch (one untimed launch, then
- * `repeats` launches timed with CUDA events on `stream`; synchronous), and
- * records the fastest for the sample's lmax in the system: later launches
+ * shape 2 for at most two models per SM, and above that the one of 0 and 1 of
+ * which more threads are resident, its CTAs taking their models dynamically
+ * from the grid once there are more models than resident CTAs); 5..9 = the
+ * same five with dynamic scheduling (a CTA claims its next model from a counter
+ * in stream-ordered scratch when it finishes one).  aem_autotune_forward times
+ * every shape that fits on an SM on the caller's sample batch (one untimed
+ * launch, then `repeats` launches timed with CUDA events on `stream`;
+ * synchronous), and records the fastest for the sample's lmax in the system:
+ * later launches
  * with that lmax use it.  shape_out (may be NULL) receives the choice; ms_out
  * (may be NULL, AEM_F32_SHAPES floats) the mean time per launch of each shape, -1 for a
  * shape that does not fit.  It takes P x G floats of stream-ordered scratch

@@ -210,9 +210,13 @@ __global__ void __launch_bounds__(kGT, 3) loglik_grad_kernel(GradModels mv, int 
     for (int p = blockIdx.x; p < mv.n; p = next_model) {
         const int L = mv.nlayers[p];
         __syncthreads();
-        if (tid == 0) next_model = (int)gridDim.x + atomicAdd(work_counter, 1);
+        // when this model's items are done, not before (forward.cu)
+        auto ask = [&] {
+            if (tid == 0) next_model = (int)gridDim.x + atomicAdd(work_counter, 1);
+        };
         if (valid && !valid[p]) {  // a proposal the caller will not use (CTA-uniform)
-            __syncthreads();       // next_model visible to every thread
+            ask();
+            __syncthreads();  // next_model visible to every thread
             continue;
         }
         if (tid < L) {
@@ -417,6 +421,7 @@ __global__ void __launch_bounds__(kGT, 3) loglik_grad_kernel(GradModels mv, int 
                 ++f;
             }
         }
+        ask();
         // CTA reduction of the per-thread accumulators (fixed order)
         for (int n = 0; n < L; ++n) {
             const float4 ac = acc_s[n];

@@ -89,7 +89,7 @@ struct aem_system {
     int f32_shape[AEM_MAX_LAYERS + 1] = {};
     // CTAs per SM of each kernel, asked once (resident_ctas): the FP32 forward
     // shapes and the adjoint per lmax, the tensor-core transform per mode
-    mutable std::atomic<int> fwd_ctas[AEM_F32_SHAPES][AEM_MAX_LAYERS + 1] = {};
+    mutable std::atomic<int> fwd_ctas[AEM_F32_SHAPES + 2][AEM_MAX_LAYERS + 1] = {};
     mutable std::atomic<int> grad_ctas[AEM_MAX_LAYERS + 1] = {};
     mutable std::atomic<int> tc_ctas[3] = {};
     // the FP32 forward kernel's depth cutoff (aem_system_set_depth_cutoff):

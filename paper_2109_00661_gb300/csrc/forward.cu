@@ -562,6 +562,63 @@ __device__ __forceinline__ void im_r0_pair(u64 lam2, u64 nwair, unsigned rec, un
     out1 = n1 * rcp_approx(d1);
 }
 
+// Claiming the next model from the grid itself (cluster launch control): with
+// one CTA per model in the grid, a running CTA cancels the next one that has
+// not been started yet and takes over its index, so CTAs stay resident and
+// whichever is free takes the next model, with no counter in memory to
+// allocate, reset or keep apart between streams (a launch without a recorded
+// shape allocates nothing).  One thread asks (asynchronously, answered into
+// shared memory) and later reads the answer.  A counter is about 1 % faster
+// (9.19 against 9.27 ms for 2^17 models of the 60 x 200 system), so the
+// recorded dynamic shapes and the callers that own one keep it.
+struct alignas(16) Claim {
+    unsigned long long answer[2];
+    unsigned long long bar;
+    unsigned parity;
+};
+constexpr int kClaimSpins = 1 << 22;  // a bound on the wait; an answer takes about a microsecond
+
+__device__ __forceinline__ void claim_init(Claim *c) {
+    c->parity = 0;
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((unsigned)__cvta_generic_to_shared(&c->bar)) : "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+}
+__device__ __forceinline__ void claim_ask(Claim *c) {
+    const unsigned a = (unsigned)__cvta_generic_to_shared(c->answer), b = (unsigned)__cvta_generic_to_shared(&c->bar);
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the last answer has been read
+    asm volatile("{\n\t.reg .b64 t;\n\tmbarrier.arrive.expect_tx.shared::cta.b64 t, [%0], 16;\n\t}" ::"r"(b) : "memory");
+    asm volatile(
+        "clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];" ::"r"(a),
+        "r"(b)
+        : "memory");
+}
+// The index taken over, or n when none is left (or the bound ran out: recorded in *status).
+__device__ __forceinline__ int claim_answer(Claim *c, int n, int *status) {
+    const unsigned a = (unsigned)__cvta_generic_to_shared(c->answer), b = (unsigned)__cvta_generic_to_shared(&c->bar);
+    const unsigned parity = c->parity;
+    c->parity = parity ^ 1;
+    unsigned ok = 0;
+    for (int i = 0; i < kClaimSpins && !ok; ++i)
+        asm volatile(
+            "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+            : "=r"(ok)
+            : "r"(b), "r"(parity)
+            : "memory");
+    if (!ok) {
+        atomicExch(status, (int)AEM_ERR_TIMEOUT);
+        return n;
+    }
+    unsigned got, x;
+    asm volatile(
+        "{\n\t.reg .b128 r;\n\t.reg .pred p;\n\t.reg .b32 y, z, w;\n\tld.shared.b128 r, [%2];\n\t"
+        "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, r;\n\tselp.u32 %0, 1, 0, p;\n\tmov.u32 %1, 0;\n\t"
+        "@p clusterlaunchcontrol.query_cancel.get_first_ctaid.v4.b32.b128 {%1, y, z, w}, r;\n\t}"
+        : "=r"(got), "=&r"(x)
+        : "r"(a)
+        : "memory");
+    return got ? (int)x : n;
+}
+
 // The per-item value buffer: kValsWords floats (24 KB), the same for every
 // launch shape, so that the Hankel sums come out identical whatever the
 // shape, the scheduling or the row stride (lmax) of the models.
@@ -587,7 +644,9 @@ __host__ __device__ inline int vals_words(int F, int K2) {
 // partial sums, two levels by shuffles) and added to imh[f], rounds in order.
 // The order of every sum is fixed by the item indices alone.  (The throughput
 // system's 60 x 100 items take one round.)
-template <int NT, int MINB, bool DYN, bool SPEC>
+// DYN: models in a fixed order (0), claimed from work_counter (1) or from the
+// grid, which then has a CTA per model (2).
+template <int NT, int MINB, int DYN, bool SPEC>
 __global__ void __launch_bounds__(NT, MINB) forward_f32_kernel(ModelsView<float> mv, int F, int G, int K,
                                                                int cc_form, int LS, float len,
                                                                const float *__restrict__ g_omega,
@@ -600,6 +659,7 @@ __global__ void __launch_bounds__(NT, MINB) forward_f32_kernel(ModelsView<float>
                                                                const double *__restrict__ eps_an, double eps_mn,
                                                                double *__restrict__ ll_out,
                                                                int *__restrict__ work_counter,
+                                                               int *__restrict__ status,
                                                                const int *__restrict__ active, float att0,
                                                                unsigned long long *__restrict__ steps_out,
                                                                const int8_t *__restrict__ valid) {
@@ -636,13 +696,26 @@ __global__ void __launch_bounds__(NT, MINB) forward_f32_kernel(ModelsView<float>
     const bool wide = K2 >= 32;  // 32 consecutive items span two frequencies at most
 
     __shared__ int next_model;
+    __shared__ Claim claim;
+    if (DYN == 2 && tid == 0) claim_init(&claim);
     unsigned int nsteps = 0;  // layer-steps of the groups this lane bucketed (steps_out)
     for (int p = blockIdx.x; p < mv.n; p = DYN ? next_model : p + gridDim.x) {
         const int L = mv.nlayers[p];
         __syncthreads();
-        // claimed now, read after this model's later barriers
-        if (DYN && tid == 0) next_model = (int)gridDim.x + atomicAdd(work_counter, 1);
+        // The next model is claimed when this one's items are done, not before:
+        // what is left at the end then goes to whichever CTA is free, not to
+        // those that started first (1,300 models on 1,216 resident CTAs: 75 us
+        // claimed at the model's start, 60 us).
+        auto ask = [&] {
+            if (DYN == 1 && tid == 0) next_model = (int)gridDim.x + atomicAdd(work_counter, 1);
+            if (DYN == 2 && tid == 0) claim_ask(&claim);
+        };
+        auto claimed = [&] {  // into next_model, before a barrier
+            if (DYN == 2 && tid == 0) next_model = claim_answer(&claim, mv.n, status);
+        };
         if (valid && !valid[p]) {  // a proposal the caller will not use (CTA-uniform)
+            ask();
+            claimed();
             if (DYN) __syncthreads();  // next_model visible to every thread
             continue;
         }
@@ -800,6 +873,7 @@ __global__ void __launch_bounds__(NT, MINB) forward_f32_kernel(ModelsView<float>
                     }
                 }
             }
+            if (r1 == FK2) ask();
             __syncthreads();
             // the round's share of each frequency's Hankel sum, in a fixed
             // order: four consecutive lanes per frequency; lane s adds the
@@ -829,6 +903,7 @@ __global__ void __launch_bounds__(NT, MINB) forward_f32_kernel(ModelsView<float>
                 acc += __shfl_xor_sync(kFull, acc, 2);
                 if (s == 0 && j <= fb) imh[j] += acc;
             }
+            if (r1 == FK2) claimed();
             __syncthreads();
         }
 
@@ -907,8 +982,11 @@ constexpr F32Shape kF32Shapes[] = {AEM_SHAPES(AEM_SHAPE)};
 // shapes kNumBase .. 2 kNumBase - 1 are the same with dynamic model scheduling
 constexpr int kNumBase = sizeof(kF32Shapes) / sizeof(kF32Shapes[0]);
 constexpr int kNumF32Shapes = 2 * kNumBase;
+// shapes 0 and 1 taking their models from the grid, for launches without a recorded shape
+constexpr int kFromGrid = kNumF32Shapes;
+static_assert(kNumF32Shapes == AEM_F32_SHAPES, "");
 
-template <int IDX, int NT, int MINB, bool DYN, bool SPEC>
+template <int IDX, int NT, int MINB, int DYN, bool SPEC>
 int launch_shape(const aem_system *sys, const ModelsView<float> &mv, int LS, float *gates, float *imh,
                  const double *y_obs, int obs_per, const double *eps_an, double eps_mn, double *ll,
                  cudaStream_t stream, int *counter_ext, const int *active, unsigned long long *steps,
@@ -920,15 +998,15 @@ int launch_shape(const aem_system *sys, const ModelsView<float> &mv, int LS, flo
     if (const int rc = resident_ctas(&sys->fwd_ctas[IDX][LS], kern, NT, smem, sys->device, &per_sm)) return rc;
     if (per_sm < 1) return fail(AEM_ERR_UNSUPPORTED, "forward kernel: launch shape does not fit on an SM");
     long long grid = (long long)sys->num_sms * per_sm;
-    if (grid > mv.n) grid = mv.n;
+    if (grid > mv.n || DYN == 2) grid = mv.n;
     int *counter = counter_ext;
-    const bool own = DYN && !counter_ext;
+    const bool own = DYN == 1 && !counter_ext;
     if (own)  // stream-ordered: one counter per launch, so launches on other streams never share it
         AEM_CUDA_TRY(cudaMallocAsync((void **)&counter, sizeof(int), stream));
-    if (DYN) AEM_CUDA_TRY(cudaMemsetAsync(counter, 0, sizeof(int), stream));
+    if (DYN == 1) AEM_CUDA_TRY(cudaMemsetAsync(counter, 0, sizeof(int), stream));
     kern<<<(unsigned)grid, NT, smem, stream>>>(mv, h.F, h.G, h.K, h.cc_form, LS, sys->len, sys->d_omega_f, sys->d_lamu_f,
                                                sys->d_hw_f, sys->d_T_f, gates, imh, y_obs, obs_per, eps_an, eps_mn,
-                                               ll, counter, active, sys->depth_att, steps, valid);
+                                               ll, counter, sys->d_status, active, sys->depth_att, steps, valid);
     const cudaError_t e = cudaGetLastError();
     if (own) cudaFreeAsync(counter, stream);
     AEM_CUDA_TRY(e);
@@ -939,18 +1017,21 @@ int launch_shape_index(int idx, const aem_system *sys, const ModelsView<float> &
                        float *imh, const double *y_obs, int obs_per, const double *eps_an, double eps_mn, double *ll,
                        cudaStream_t stream, int *counter_ext = nullptr, const int *active = nullptr,
                        unsigned long long *steps = nullptr, const int8_t *valid = nullptr) {
-#define AEM_SHAPE(I, NT, MINB, SPEC)                                                                                 \
+#define AEM_SHAPE_CASE(I, NT, MINB, DYN, SPEC)                                                                     \
     case I:                                                                                                        \
-        return launch_shape<I, NT, MINB, false, SPEC>(sys, mv, LS, gates, imh, y_obs, obs_per, eps_an, eps_mn, ll, stream, \
-                                             counter_ext, active, steps, valid);                                   \
-    case I + kNumBase:                                                                                             \
-        return launch_shape<I + kNumBase, NT, MINB, true, SPEC>(sys, mv, LS, gates, imh, y_obs, obs_per, eps_an, eps_mn, ll, stream,  \
-                                            counter_ext, active, steps, valid);
+        return launch_shape<I, NT, MINB, DYN, SPEC>(sys, mv, LS, gates, imh, y_obs, obs_per, eps_an, eps_mn, ll,   \
+                                                    stream, counter_ext, active, steps, valid);
+#define AEM_SHAPE(I, NT, MINB, SPEC)         \
+    AEM_SHAPE_CASE(I, NT, MINB, 0, SPEC)     \
+    AEM_SHAPE_CASE(I + kNumBase, NT, MINB, 1, SPEC)
     switch (idx) {
         AEM_SHAPES(AEM_SHAPE)
+        AEM_SHAPE_CASE(kFromGrid, 256, 4, 2, false)
+        AEM_SHAPE_CASE(kFromGrid + 1, 128, 8, 2, false)
         default: return fail(AEM_ERR_INVALID_ARG, "forward kernel: launch shape");
     }
 #undef AEM_SHAPE
+#undef AEM_SHAPE_CASE
 }
 
 template <class Models>
@@ -969,10 +1050,32 @@ int launch_forward_f32(const aem_system *sys, const Models *models, float *gates
     ModelsView<float> mv{models->n_models, models->lmax, models->nlayers, models->logsig, models->logh,
                            models->m, models->logtau, models->c};
     const int LS = models->lmax;
-    // No shape recorded: the smallest CTAs for batches that fill the chip;
-    // with at most two models per SM the largest, which finish a model soonest.
+    // No shape recorded.  At most two models per SM: the largest CTAs, which
+    // finish a model soonest.  Otherwise the looped shape of which more threads
+    // are resident (the value buffer of many frequencies and abscissae leaves
+    // room for fewer CTAs), the smaller one on a tie, with dynamic scheduling
+    // once there are more models than resident CTAs.  3,001 and 20,000 models of
+    // up to 10 layers of the 60 x 200 system: 340 and 1889 us at 128 x 8 in
+    // fixed order, 254 and 1472 us; up to 8 layers of the 40 x 120 system, where
+    // 128 x 8 stays: 117 and 671 us, 109 and 555 us.
     int shape = sys->f32_shape[LS];
-    if (shape == 0) shape = models->n_models <= 2 * sys->num_sms ? 2 : 1;
+    if (shape == 0) {
+        if (models->n_models <= 2 * sys->num_sms) {
+            shape = 2;
+        } else {
+            const size_t smem = smem_bytes_f32(sys->host.F, sys->host.G, sys->host.K, LS);
+            int n0 = 0, n1 = 0;
+            if (const int rc = resident_ctas(&sys->fwd_ctas[kFromGrid][LS], forward_f32_kernel<256, 4, 2, false>, 256,
+                                             smem, sys->device, &n0))
+                return rc;
+            if (const int rc = resident_ctas(&sys->fwd_ctas[kFromGrid + 1][LS], forward_f32_kernel<128, 8, 2, false>,
+                                             128, smem, sys->device, &n1))
+                return rc;
+            shape = n1 >= 2 * n0 ? 1 : 0;
+            if (models->n_models > (long long)sys->num_sms * (shape ? n1 : n0))
+                shape += counter_ext ? kNumBase : kFromGrid;
+        }
+    }
     return launch_shape_index(shape, sys, mv, LS, gates, imh, y_obs, obs_per, eps_an, eps_mn, ll,
                               (cudaStream_t)stream, counter_ext, active, steps, valid);
 }

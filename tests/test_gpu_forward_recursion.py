@@ -47,3 +47,39 @@ def test_length_scales(height, radius):
     _, ref, absh = O.forward(models, so, mode=O.HANKEL_RULE, want_imh=True, want_absh=True)
     imh = L.spectrum_f32(sysg, I.to_torch(models, torch.float32)).cpu().numpy().astype(np.float64)
     assert spectrum_err(imh, ref, absh).max() < DELTA_S32
+
+
+@pytest.mark.parametrize("name, lmax, models", [("sounding-g20-f40-k120", 8, 305), ("sounding-g20-f40-k120", 8, 1217),
+                                                ("sounding-g20-f40-k120", 20, 5001), ("throughput", 10, 609),
+                                                ("throughput", 1, 3000), ("throughput", 10, 4100)])
+def test_models_taken_from_the_grid(name, lmax, models):
+    """Launches without a recorded shape claim their models from the grid once
+    there are more of them than resident CTAs: the fixed order's results bit
+    for bit, also under capture and from two streams at once."""
+    import torch
+    import paper_2109_00661_gb300 as L
+    kw = I.system_kwargs("sounding-g20-f40-k120")
+    if name == "throughput":
+        kw = dict(kw, n_freq=60, n_hankel=200)
+    sysg, fixed = L.System(**kw), L.System(**kw)
+    fixed.set_forward_shape(lmax, 1)
+    m = I.to_torch(I.random_models(models, seed=models, lmax=lmax, layers_max=lmax), torch.float32)
+    want = L.spectrum_f32(fixed, m)
+    assert torch.equal(L.spectrum_f32(sysg, m), want)
+    side = [torch.cuda.Stream(), torch.cuda.Stream()]
+    out = []
+    torch.cuda.synchronize()
+    for _ in range(3):
+        for s in side:
+            with torch.cuda.stream(s):
+                out.append(L.spectrum_f32(sysg, m))
+    torch.cuda.synchronize()
+    assert all(torch.equal(o, want) for o in out)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        got = L.spectrum_f32(sysg, m)
+    for _ in range(2):
+        got.zero_()
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(got, want)
