@@ -1261,6 +1261,60 @@ __device__ inline bool ordered_open(const float *z, int n, double zmax) {
     return n == 0 || (double)z[n - 1] < zmax;
 }
 
+// The Langevin kernels give a particle kLanes lanes, each every kLanes-th
+// component of theta (up to 39): one thread's chain of that many FP64
+// Box-Muller draws took 143 us for 4,096 particles (61 now; the accept test's 66
+// and 22), the chip's FP64 rate alone about 40.  Sums over the components keep their order (every lane adds the
+// others' terms in turn), so proposals and decisions are the serial ones.
+constexpr int kLanes = 8;
+
+struct Lanes {
+    int i, sub;     // particle, lane of it
+    unsigned mask;  // its lanes in the warp
+};
+__device__ inline Lanes lanes_of_thread() {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    return {t / kLanes, t % kLanes, ((1u << kLanes) - 1u) << (threadIdx.x & 31 & ~(kLanes - 1))};
+}
+
+__device__ inline void copy_particle_lanes(PState d, PState s, const Lanes &l) {
+    const int i = l.i;
+    if (l.sub == 0) {
+        d.kappa[i] = s.kappa[i];
+        d.lam[i] = s.lam[i];
+        d.phib[i] = s.phib[i];
+        d.tau[i] = s.tau[i];
+        d.c[i] = s.c[i];
+        d.ll[i] = s.ll[i];
+    }
+    for (int q = i * KS + l.sub; q < (i + 1) * KS; q += kLanes) {
+        d.zc[q] = s.zc[q];
+        d.phic[q] = s.phic[q];
+        d.zm[q] = s.zm[q];
+        d.mv[q] = s.mv[q];
+    }
+}
+
+// ordered_open for this lane's interfaces
+__device__ inline bool ordered_open_lanes(const float *z, int n, double zmax, int sub) {
+    bool ok = true;
+    for (int q = sub; q < n; q += kLanes) {
+        const double lo = q > 0 ? (double)z[q - 1] : 0.0;
+        ok = ok && (double)z[q] > lo && (q < n - 1 || (double)z[q] < zmax);
+    }
+    return ok;
+}
+
+// acc - sum over the kLanes components from j0 of x^2 / 2, in their order
+__device__ inline double minus_half_squares(double acc, double x, int j0, int d, unsigned mask) {
+    const int n = min(kLanes, d - j0);
+    for (int q = 0; q < n; ++q) {
+        const double v = __shfl_sync(mask, x, q, kLanes);
+        acc -= 0.5 * v * v;
+    }
+    return acc;
+}
+
 // Preconditioned Langevin proposal at gamma_t:
 //   theta' = theta + (h^2 / 2) D gamma_t grad l(theta) + h D^(1/2) xi,
 //   D = diag(scale_j^2), xi ~ N(0, I);
@@ -1269,42 +1323,53 @@ __device__ inline bool ordered_open(const float *z, int n, double zmax) {
 __global__ void langevin_propose_kernel(PState cur, PState prop, const float *gcur, const double *gamma,
                                         const double *lang_h, Params pr, int stage_arg, int sweep, int8_t *valid_out,
                                         double *lq, const int *stage_dev) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= pr.S * pr.N) return;
+    const Lanes l = lanes_of_thread();
+    const int i = l.i;
+    if (i >= pr.S * pr.N) return;  // all lanes of the particle
     const int stage = stage_dev ? *stage_dev : stage_arg;
     const int s = i / pr.N, jp = i - s * pr.N;
     const Key key = stream_key(pr.seed, s);
-    copy_particle(prop, i, cur, i);
+    copy_particle_lanes(prop, cur, l);
+    __syncwarp(l.mask);
     const int kappa = cur.kappa[i], lam = cur.lam[i];
     const int d = 3 + 2 * kappa + 2 * lam;
     const double gm = gamma[s], h = lang_h[s];
     double lqf = 0.0;
-    uint32_t w[4];
-    for (int j = 0; j < d; ++j) {
-        if ((j & 1) == 0)
+    for (int j0 = 0; j0 < d; j0 += kLanes) {
+        const int j = j0 + l.sub;
+        double xi = 0.0;
+        if (j < d) {
+            uint32_t w[4];
             block_draws(w, key, (uint32_t)jp, (uint32_t)(kPurposeLangevin0 + j / 2), (uint32_t)stage,
                         (uint32_t)sweep);
-        const double xi = gauss(w[2 * (j & 1)], w[2 * (j & 1) + 1]);
-        const ThetaRef rc = theta_ref(cur, i, j, kappa, lam, pr);
-        const ThetaRef rp = theta_ref(prop, i, j, kappa, lam, pr);
-        const double sc = rc.scale;
-        const double th = theta_value(rc, pr) + 0.5 * h * h * sc * sc * gm * (double)gcur[(size_t)i * GD + rc.slot] +
-                          h * sc * xi;
-        *rp.x = (float)((rp.is_tau && pr.tau_log_prior) ? pow(10.0, th) : th);
-        lqf -= 0.5 * xi * xi;
+            xi = (j & 1) ? gauss(w[2], w[3]) : gauss(w[0], w[1]);
+            const ThetaRef rc = theta_ref(cur, i, j, kappa, lam, pr);
+            const ThetaRef rp = theta_ref(prop, i, j, kappa, lam, pr);
+            const double sc = rc.scale;
+            const double th = theta_value(rc, pr) +
+                              0.5 * h * h * sc * sc * gm * (double)gcur[(size_t)i * GD + rc.slot] + h * sc * xi;
+            *rp.x = (float)((rp.is_tau && pr.tau_log_prior) ? pow(10.0, th) : th);
+        }
+        lqf = minus_half_squares(lqf, xi, j0, d, l.mask);
     }
+    __syncwarp(l.mask);  // the lanes' components, before the others read them
     bool ok = in_bounds_open(prop.phib[i], pr.phi_lo, pr.phi_hi) && in_bounds_open(prop.c[i], 0.0, 1.0);
-    for (int q = 0; q < kappa; ++q) ok = ok && in_bounds_open(prop.phic[i * KS + q], pr.phi_lo, pr.phi_hi);
-    for (int q = 0; q < lam; ++q) ok = ok && in_bounds_open(prop.mv[i * KS + q], 0.0, 1.0);
-    ok = ok && ordered_open(prop.zc + (size_t)i * KS, kappa, pr.zmax) &&
-         ordered_open(prop.zm + (size_t)i * KS, lam, pr.zmax);
-    if (pr.tau_log_prior)
-        ok = ok && prop.tau[i] > 0.f && in_bounds_open(log10((double)prop.tau[i]), pr.logtau_lo, pr.logtau_hi);
-    else
-        ok = ok && in_bounds_open(prop.tau[i], 0.0, 1.0);
-    if (!ok) copy_particle(prop, i, cur, i);
-    valid_out[i] = ok ? 1 : 0;
-    lq[i] = lqf;
+    for (int q = l.sub; q < kappa; q += kLanes) ok = ok && in_bounds_open(prop.phic[i * KS + q], pr.phi_lo, pr.phi_hi);
+    for (int q = l.sub; q < lam; q += kLanes) ok = ok && in_bounds_open(prop.mv[i * KS + q], 0.0, 1.0);
+    ok = ok && ordered_open_lanes(prop.zc + (size_t)i * KS, kappa, pr.zmax, l.sub) &&
+         ordered_open_lanes(prop.zm + (size_t)i * KS, lam, pr.zmax, l.sub);
+    if (l.sub == 0) {
+        if (pr.tau_log_prior)
+            ok = ok && prop.tau[i] > 0.f && in_bounds_open(log10((double)prop.tau[i]), pr.logtau_lo, pr.logtau_hi);
+        else
+            ok = ok && in_bounds_open(prop.tau[i], 0.0, 1.0);
+    }
+    ok = __all_sync(l.mask, ok);
+    if (!ok) copy_particle_lanes(prop, cur, l);
+    if (l.sub == 0) {
+        valid_out[i] = ok ? 1 : 0;
+        lq[i] = lqf;
+    }
 }
 
 // Metropolis-Hastings test of the Langevin proposal at gamma_t:
@@ -1314,32 +1379,42 @@ __global__ void langevin_accept_kernel(PState cur, PState prop, float *gcur, con
                                        const int8_t *valid, const double *lq, const double *gamma,
                                        const double *lang_h, Params pr, int stage_arg, int sweep, int *lacc,
                                        int *lprop, const int *stage_dev) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const Lanes l = lanes_of_thread();
+    const int i = l.i;
     if (i >= pr.S * pr.N) return;
     const int stage = stage_dev ? *stage_dev : stage_arg;
     const int s = i / pr.N, jp = i - s * pr.N;
-    atomicAdd(&lprop[s], 1);
-    if (!valid[i]) return;
+    if (l.sub == 0) atomicAdd(&lprop[s], 1);
+    if (!valid[i]) return;  // all lanes of the particle
     const int kappa = cur.kappa[i], lam = cur.lam[i];
     const int d = 3 + 2 * kappa + 2 * lam;
     const double gm = gamma[s], h = lang_h[s];
     double lqr = 0.0;
-    for (int j = 0; j < d; ++j) {
-        const ThetaRef rc = theta_ref(cur, i, j, kappa, lam, pr);
-        const ThetaRef rp = theta_ref(prop, i, j, kappa, lam, pr);
-        const double sc = rc.scale;
-        const double mean = theta_value(rp, pr) + 0.5 * h * h * sc * sc * gm * (double)gprop[(size_t)i * GD + rp.slot];
-        const double zz = (theta_value(rc, pr) - mean) / (h * sc);
-        lqr -= 0.5 * zz * zz;
+    for (int j0 = 0; j0 < d; j0 += kLanes) {
+        const int j = j0 + l.sub;
+        double zz = 0.0;
+        if (j < d) {
+            const ThetaRef rc = theta_ref(cur, i, j, kappa, lam, pr);
+            const ThetaRef rp = theta_ref(prop, i, j, kappa, lam, pr);
+            const double sc = rc.scale;
+            const double mean =
+                theta_value(rp, pr) + 0.5 * h * h * sc * sc * gm * (double)gprop[(size_t)i * GD + rp.slot];
+            zz = (theta_value(rc, pr) - mean) / (h * sc);
+        }
+        lqr = minus_half_squares(lqr, zz, j0, d, l.mask);
     }
-    uint32_t w[4];
-    block_draws(w, stream_key(pr.seed, s), (uint32_t)jp, (uint32_t)kPurposeLangevinAccept, (uint32_t)stage,
-                (uint32_t)sweep);
-    const double u = u01_53(w[0], w[1]);
-    if (log(u) < gm * (prop.ll[i] - cur.ll[i]) + lqr - lq[i]) {
-        copy_particle(cur, i, prop, i);
-        for (int q = 0; q < GD; ++q) gcur[(size_t)i * GD + q] = gprop[(size_t)i * GD + q];
-        atomicAdd(&lacc[s], 1);
+    bool take = false;
+    if (l.sub == 0) {
+        uint32_t w[4];
+        block_draws(w, stream_key(pr.seed, s), (uint32_t)jp, (uint32_t)kPurposeLangevinAccept, (uint32_t)stage,
+                    (uint32_t)sweep);
+        const double u = u01_53(w[0], w[1]);
+        take = log(u) < gm * (prop.ll[i] - cur.ll[i]) + lqr - lq[i];
+    }
+    if (__shfl_sync(l.mask, (int)take, 0, kLanes)) {  // every lane has read cur
+        copy_particle_lanes(cur, prop, l);
+        for (int q = l.sub; q < GD; q += kLanes) gcur[(size_t)i * GD + q] = gprop[(size_t)i * GD + q];
+        if (l.sub == 0) atomicAdd(&lacc[s], 1);
     }
 }
 
@@ -2121,7 +2196,7 @@ struct smc_state {
 // serial chain, with FP64 logarithms that cost an SM 19 cycles per warp
 // operation, so while the population's warps fit the chip at once (32 CTAs per
 // SM) every warp is a CTA of its own: 4,096 particles are 128 warps on 128 SMs,
-// not 32 CTAs of four on 32 (merge 62 -> 40 us, Langevin proposal 152 -> 143).
+// not 32 CTAs of four on 32 (merge 62 -> 40 us).
 static unsigned particle_threads(const smc_state *st) { return st->P <= 1024LL * st->sys->num_sms ? 32 : 128; }
 static unsigned particle_ctas(const smc_state *st) { return blocks_for(st->P, (int)particle_threads(st)); }
 
@@ -2573,11 +2648,11 @@ static int langevin_sweeps(smc_state *st, int n, const int *stage_dev = nullptr)
     if ((rc = run_grad(st, st->cur, st->gcur))) return rc;
     st->gcur_valid = true;
     for (int l = 0; l < n; ++l) {
-        langevin_propose_kernel<<<particle_ctas(st), particle_threads(st), 0, st->stream>>>(
+        langevin_propose_kernel<<<blocks_for((long long)st->P * kLanes, 128), 128, 0, st->stream>>>(
             st->cur, st->prop, st->gcur, st->gamma, st->lang_h, st->pr, st->stage, l, st->valid, st->lq, stage_dev);
         AEM_CUDA_TRY(cudaGetLastError());
         if ((rc = run_grad(st, st->prop, st->gprop, st->valid))) return rc;
-        langevin_accept_kernel<<<particle_ctas(st), particle_threads(st), 0, st->stream>>>(
+        langevin_accept_kernel<<<blocks_for((long long)st->P * kLanes, 128), 128, 0, st->stream>>>(
             st->cur, st->prop, st->gcur, st->gprop, st->valid, st->lq, st->gamma, st->lang_h, st->pr, st->stage, l,
             st->lacc, st->lprop, stage_dev);
         AEM_CUDA_TRY(cudaGetLastError());
@@ -2901,7 +2976,7 @@ extern "C" int smc_langevin_propose(smc_state *st, int stage, int sweep) {
     if (!st) return fail(AEM_ERR_INVALID_ARG, "smc_langevin_propose: NULL state");
     if (!st->gcur_valid)
         return fail(AEM_ERR_INVALID_ARG, "smc_langevin_propose: no gradient of the current particles (smc_grad_current)");
-    langevin_propose_kernel<<<particle_ctas(st), particle_threads(st), 0, st->stream>>>(
+    langevin_propose_kernel<<<blocks_for((long long)st->P * kLanes, 128), 128, 0, st->stream>>>(
         st->cur, st->prop, st->gcur, st->gamma, st->lang_h, st->pr, stage, sweep, st->valid, st->lq, nullptr);
     AEM_CUDA_TRY(cudaGetLastError());
     return AEM_OK;
