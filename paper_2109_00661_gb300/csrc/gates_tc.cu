@@ -18,15 +18,16 @@
 // shared memory in the canonical K-major layout without swizzle (core
 // matrices of 8 rows x 16 bytes), each lane converting one 16-byte core-matrix
 // row so that a warp's stores cover 512 contiguous bytes; one thread issues
-// the tcgen05.mma chain into a TMEM accumulator (row m of the tile in TMEM
-// lane m, gate n in column n) and commits it to an mbarrier; every warp then
-// reads its 32 lanes (warps w and w + 4 the same lanes, each half of the
-// columns) with tcgen05.ld and forms the gates and the likelihood terms of
-// its 32 models, the two halves' sums meeting in shared memory.  The likelihood terms are FP32 (Section 2.3.2's Gaussian:
-// the residual from a float pair holding the FP64 datum, the variance, one
-// logarithm and one division per gate) and their sum is carried as an
-// unevaluated FP32 pair (Knuth's TwoSum), exact to about 2^-48 of the sum of
-// magnitudes, so no FP64 arithmetic is left per gate.  Every wait is bounded:
+// the tcgen05.mma chain into one of two TMEM accumulators (row m of the tile
+// in TMEM lane m, gate n in column n) and commits it to an mbarrier; while the
+// next tile's chain runs into the other one, every warp reads its 32 lanes
+// (warps w and w + 4 the same lanes, each half of the columns) with tcgen05.ld
+// and forms the gates and the likelihood terms of its 32 models, the two
+// halves' sums meeting in shared memory.  The likelihood terms are FP32
+// (Section 2.3.2's Gaussian: the residual from a float pair holding the FP64
+// datum, the variance, a division, and the logarithm of a product of variances,
+// see LlAcc) and their sum is carried as an unevaluated FP32 pair (Knuth's
+// TwoSum), so no FP64 arithmetic is left per gate.  Every wait is bounded:
 // on a timeout the CTA records AEM_ERR_TIMEOUT in the system's status word,
 // waits (bounded) once more for its own MMAs, frees its TMEM and returns.  If
 // that second wait also gives up, the MMAs it issued may still be in flight
