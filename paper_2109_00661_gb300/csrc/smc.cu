@@ -799,7 +799,7 @@ __global__ void __launch_bounds__(kGroupThreads) reweight_kernel(const RwArgs a)
             else
                 a.logz[(size_t)s * M + k] = z;
         }
-        if (tid == 0) {  // warp 0: `done` is the driver's
+        if (tid == 0) {  // warp 0, which holds `done`
             if (a.gamma_out) a.gamma_out[s] = done ? 1.0 : g0 + dg;
             a.dgamma_out[s] = dg;
             a.done_out[s] = done;
