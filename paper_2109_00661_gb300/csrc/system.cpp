@@ -274,6 +274,23 @@ using namespace aem;
 
 extern "C" const char *aem_last_error(void) { return g_last_error.c_str(); }
 
+// The FP64 forward kernel's tables (aem_system::d_tab64), formed once: the
+// same for every system, rounded from extended precision.
+static const std::vector<double> &f64_tables() {
+    static const std::vector<double> tab = [] {
+        std::vector<double> t(2 * kTab64Turn + kTab64Octave);
+        for (int j = 0; j < kTab64Turn; ++j) {
+            const long double a = 6.283185307179586476925286766559L * j / kTab64Turn;
+            t[2 * j] = (double)std::sin(a);
+            t[2 * j + 1] = (double)std::cos(a);
+        }
+        for (int j = 0; j < kTab64Octave; ++j)
+            t[2 * kTab64Turn + j] = (double)std::exp2((long double)j / kTab64Octave);
+        return t;
+    }();
+    return tab;
+}
+
 template <class T>
 static int upload(T **dst, const std::vector<double> &src) {
     std::vector<T> tmp(src.begin(), src.end());
@@ -306,14 +323,7 @@ extern "C" int aem_system_create(const aem_system_desc *desc, aem_system **out) 
     std::vector<double> lamu(h.lam);
     for (double &l : lamu) l *= len;
     s->len = (float)len;
-    std::vector<double> tab64(2 * kTab64Turn + kTab64Octave);
-    for (int j = 0; j < kTab64Turn; ++j) {
-        const long double a = 6.283185307179586476925286766559L * j / kTab64Turn;
-        tab64[2 * j] = (double)std::sin(a);
-        tab64[2 * j + 1] = (double)std::cos(a);
-    }
-    for (int j = 0; j < kTab64Octave; ++j)
-        tab64[2 * kTab64Turn + j] = (double)std::exp2((long double)j / kTab64Octave);
+    const std::vector<double> &tab64 = f64_tables();
     if ((rc = upload(&s->d_omega_f, h.omega)) || (rc = upload(&s->d_lam_f, h.lam)) || (rc = upload(&s->d_hw_f, h.hw)) ||
         (rc = upload(&s->d_T_f, h.T)) || (rc = upload(&s->d_omega_d, h.omega)) || (rc = upload(&s->d_lam_d, h.lam)) ||
         (rc = upload(&s->d_hw_d, h.hw)) || (rc = upload(&s->d_T_d, h.T)) ||
