@@ -121,6 +121,13 @@ __device__ __forceinline__ u64 fma2(u64 a, u64 b, u64 c) {
     return d;
 }
 
+// Knuth's TwoSum: s + e == a + b exactly (round to nearest, no overflow).
+__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
+    const float t = a + b, bb = t - a;
+    e = (a - (t - bb)) + (b - bb);
+    s = t;
+}
+
 struct C2x2 {  // two complex numbers: re = (re_a, re_b), im = (im_a, im_b)
     u64 re, im;
 };

@@ -11,8 +11,8 @@
 // kernel also drops the layers under its depth cutoff (depth_cutoff.h).  The
 // epilogue applies the G x F step-off transform and, for
 // the likelihood entry points, the Gaussian log-likelihood of Section 2.3.2
-// (FP32 terms with an FP64 sum in the FP32 kernel, FP64 throughout in the
-// FP64 one).
+// (gates in float pairs, FP32 terms and an FP64 sum in the FP32 kernel, FP64
+// throughout in the FP64 one).
 //
 // Recursion used (quasi-static TE mode, exp(+i w t)):
 //   u_n = sqrt(lambda^2 + s_n), Re u_n > 0
@@ -418,7 +418,8 @@ int launch_forward_f64(const aem_system *sys, const aem_models_f64 *models, doub
 // with the layer's own signal, and Im r keeps its relative accuracy, so the
 // spectrum's error is lower than with the differenced s (FP32 emulation on 150
 // random and 100 alternating stacks, relative to sum |w_k| |R_0|: largest
-// 6.3e-7 against 1.4e-6, rms 4.0e-8 against 7.5e-8).
+// 6.3e-7 against 1.4e-6, rms 4.0e-8 against 7.5e-8); the log-likelihood's by
+// itself is not (see forward_f32_kernel's sums).
 //   E = exp(-2 u h) = exp2(e w.x) (cos(e ln2 w.y) + i sin(e ln2 w.y)),
 //   e = -sqrt(2) h log2(e).
 // The Moebius step (N, D) <- (r D + N E, D + r N E) keeps R_0 = N / D.
@@ -429,6 +430,10 @@ int launch_forward_f64(const aem_system *sys, const aem_models_f64 *models, doub
 using namespace f32x2;  // paired FP32 helpers and the hardware approximations (f32x2.h)
 
 constexpr double kLn2Pi = 1.83787706640934548356;  // ln(2 pi)
+constexpr int kDotParts = 4;  // warps that share a model's gate transform (every launch shape has them)
+
+// The low part of a float pair; none beside an infinity or a NaN.
+__device__ __forceinline__ float rest(float hi, float lo) { return fabsf(hi) <= 3.402823466e38f ? lo : 0.f; }
 
 // rcoef2 for the air above the top layer: w_air = sqrt(2) lambda is real,
 // m_air = lambda^2; nwair = -w_air.
@@ -632,16 +637,25 @@ __host__ __device__ inline int vals_words(int F, int K2) {
 }
 
 // Shared memory (dynamic), in order: REC[F*LS] (ulonglong2: per frequency and
-// layer the (Re s, Re s) and (Im s, Im s) pairs), KR[2*K2] (ulonglong2: per
-// abscissa pair the (lambda^2, -sqrt(2) lambda) pairs, then the two Hankel
-// weights), vals[kValsWords], imh[F], T[G*F], TH[F*LS] (float: the depth
-// cutoff's thresholds), MS[F] (float: max_n(-Re s_n), the lambda^2 under which
-// some root has a negative real part).  The items (frequency major, F*K2 of
+// layer the (Re s, Re s) and (Im s, Im s) pairs), KR[K2] (ulonglong2: per
+// abscissa pair the (lambda^2, -sqrt(2) lambda) pairs), HW[K2] (the pairs'
+// Hankel weights), vals[vals_words], imh[F] (float pairs), Ts[(F+1)*G] (float
+// pairs: T by frequency, then the bounds of d_T_pair), TH[F*LS] (float: the
+// depth cutoff's thresholds).  The items (frequency major, F*K2 of
 // them) are taken in rounds of kValsWords: every item stores its weighted pair
 // value at its own index in the buffer; after the round each frequency the
 // round touched is summed by four consecutive lanes (lane s adds the values at
 // s + 4 i into four accumulators by i mod 4, then a tree over the sixteen
 // partial sums, two levels by shuffles) and added to imh[f], rounds in order.
+// From the sixteen partial sums on the sums are float pairs (TwoSum), and so
+// is the transform: the gates cancel to about a hundredth of their terms, and
+// with the spectrum and T rounded to a float and a plain dot product these
+// three made most of the log-likelihood's error.  On 256 models about one
+// earth (40 frequencies, 120 abscissae, up to 8 layers) it is 5.4e-7 of the
+// norm against 64 bits, 1.1e-6 without (1.3e-6 with the differenced s before
+// that); on the 60 x 200 system 4.4e-7 against 1.3e-6, and the gradient's
+// error falls with it by 2 to 4.  32,768 models of the former: 0.94 ms, 0.92
+// without (0.95 with TwoProd and TwoSum).
 // The order of every sum is fixed by the item indices alone.  (The throughput
 // system's 60 x 100 items take one round.)
 // DYN: models in a fixed order (0), claimed from work_counter (1) or from the
@@ -650,9 +664,10 @@ template <int NT, int MINB, int DYN, bool SPEC>
 __global__ void __launch_bounds__(NT, MINB) forward_f32_kernel(ModelsView<float> mv, int F, int G, int K,
                                                                int cc_form, int LS, float len,
                                                                const float *__restrict__ g_omega,
+                                                               const float2 *__restrict__ g_wmu,
                                                                const float *__restrict__ g_lam,
                                                                const float *__restrict__ g_hw,
-                                                               const float *__restrict__ g_T,
+                                                               const float2 *__restrict__ g_T,
                                                                float *__restrict__ gates_out,
                                                                float *__restrict__ imh_out,
                                                                const double *__restrict__ y_obs, int obs_per,
@@ -671,17 +686,22 @@ __global__ void __launch_bounds__(NT, MINB) forward_f32_kernel(ModelsView<float>
     ulonglong2 *KR = REC + (size_t)F * LS;
     u64 *HW = reinterpret_cast<u64 *>(KR + K2);
     float *vals = reinterpret_cast<float *>(HW + K2);
-    float *imh = vals + vals_words(F, K2);
-    float *Ts = imh + F;
-    float *TH = Ts + (size_t)G * F;  // depth-cutoff thresholds, [F][LS]
+    float2 *imh = reinterpret_cast<float2 *>(vals + vals_words(F, K2));
+    float2 *Ts = imh + F;
+    float *TH = reinterpret_cast<float *>(Ts + (size_t)G * (F + 1));  // depth-cutoff thresholds, [F][LS]
     __shared__ ulonglong2 HE[AEM_MAX_LAYERS];
     __shared__ float lh[AEM_MAX_LAYERS];
     __shared__ float lsig[AEM_MAX_LAYERS], lm[AEM_MAX_LAYERS], ltau[AEM_MAX_LAYERS], lc[AEM_MAX_LAYERS];
     __shared__ float lsp[AEM_MAX_LAYERS], lcp[AEM_MAX_LAYERS];
-    __shared__ double ll_part[NW];
+    __shared__ double ll_part[2];
+    __shared__ float2 gate_part[kDotParts][AEM_MAX_GATES];
+    __shared__ unsigned imh_max;  // the largest |Im H| of the model, as its bits
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int i = tid; i < G * F; i += blockDim.x) Ts[i] = g_T[i];
+    for (int i = tid; i < G * (F + 1); i += blockDim.x) {
+        const int g = i / F;
+        Ts[g < G ? (i - g * F) * G + g : i] = g_T[i];
+    }
     // abscissa pairs (k, k + K2); an odd K pads the last pair with a zero weight
     for (int k = tid; k < K2; k += blockDim.x) {
         const int kb = k + K2 < K ? k + K2 : K - 1;
@@ -691,7 +711,7 @@ __global__ void __launch_bounds__(NT, MINB) forward_f32_kernel(ModelsView<float>
         HW[k] = pk2(g_hw[k], k + K2 < K ? g_hw[kb] : 0.f);
     }
     const unsigned rec_a = (unsigned)__cvta_generic_to_shared(REC), he_a = (unsigned)__cvta_generic_to_shared(HE);
-    const float mu0 = (float)kMu0 * len * len, ilen = 1.f / len;
+    const float ilen = 1.f / len;
     const int FK2 = F * K2;
     const bool wide = K2 >= 32;  // 32 consecutive items span two frequencies at most
 
@@ -733,7 +753,8 @@ __global__ void __launch_bounds__(NT, MINB) forward_f32_kernel(ModelsView<float>
             lsp[tid] = sp;
             lcp[tid] = cp;
         }
-        for (int j = tid; j < F; j += blockDim.x) imh[j] = 0.f;
+        for (int j = tid; j < F; j += blockDim.x) imh[j] = make_float2(0.f, 0.f);
+        if (tid == 0) imh_max = 0u;
         __syncthreads();
         // Cole-Cole per (frequency, layer): x = (w tau)^c e^{i pi c / 2}, s = i w mu0 sigma
         for (int i = tid; i < F * L; i += blockDim.x) {
@@ -769,7 +790,9 @@ __global__ void __launch_bounds__(NT, MINB) forward_f32_kernel(ModelsView<float>
                     si = sig * (mm * xi / bd);
                 }
             }
-            const float sx = -w * mu0 * si, sy = w * mu0 * sr;
+            // w mu0 as a float pair: one rounding is left, that of the product
+            const float2 wm = g_wmu[f];
+            const float sx = -fmaf(wm.x, si, wm.y * si), sy = fmaf(wm.x, sr, wm.y * sr);
             REC[(size_t)f * LS + n] = make_ulonglong2(pk2(sx, sx), pk2(sy, sy));
         }
         __syncthreads();
@@ -886,7 +909,7 @@ __global__ void __launch_bounds__(NT, MINB) forward_f32_kernel(ModelsView<float>
             const int fa = r0 == 0 ? 0 : r0 / K2, fb = r1 == FK2 ? F - 1 : (r1 - 1) / K2;
             for (int t0 = 0; t0 < 4 * (fb - fa + 1); t0 += blockDim.x) {  // CTA-uniform trip count
                 const int t = t0 + tid, j = fa + (t >> 2), s = t & 3;
-                float acc = 0.f;
+                float acc = 0.f, err = 0.f;
                 if (j <= fb) {
                     const int a = j * K2 > r0 ? j * K2 : r0, b = (j + 1) * K2 < r1 ? (j + 1) * K2 : r1;
                     const float *vq = vals - r0;
@@ -897,34 +920,83 @@ __global__ void __launch_bounds__(NT, MINB) forward_f32_kernel(ModelsView<float>
                         if (q + 8 < b) c2 += vq[q + 8];
                         if (q + 12 < b) c3 += vq[q + 12];
                     }
-                    acc = (c0 + c1) + (c2 + c3);
+                    float e0, e1;
+                    two_sum(c0, c1, c0, e0);
+                    two_sum(c2, c3, c2, e1);
+                    two_sum(c0, c2, acc, err);
+                    err += e0 + e1;
                 }
-                acc += __shfl_xor_sync(kFull, acc, 1);
-                acc += __shfl_xor_sync(kFull, acc, 2);
-                if (s == 0 && j <= fb) imh[j] += acc;
+#pragma unroll
+                for (int o = 1; o <= 2; o <<= 1) {
+                    float e;
+                    two_sum(acc, __shfl_xor_sync(kFull, acc, o), acc, e);
+                    err += __shfl_xor_sync(kFull, err, o);
+                    err += e;
+                }
+                unsigned bits = 0u;
+                if (s == 0 && j <= fb) {
+                    const float2 had = imh[j];
+                    float h, e;
+                    two_sum(had.x, acc, h, e);
+                    imh[j] = make_float2(h, rest(h, had.y + (err + e)));
+                    bits = __float_as_uint(fabsf(h));
+                }
+                bits = __reduce_max_sync(kFull, bits);
+                if (lane == 0) atomicMax(&imh_max, bits);
             }
             if (r1 == FK2) claimed();
             __syncthreads();
         }
 
+        // gates: dot products in float pairs, a quarter of the frequencies per
+        // warp, lane = gate.  The sum begins at a power of two above all its
+        // partial sums, so that what it rounds off of a product is exact (Dekker's
+        // Fast2Sum): t x - (sum after - sum before), six operations a term
+        // where TwoProd and TwoSum take thirteen.
+        if (warp < kDotParts && (gates_out || ll_out)) {
+            const int j0 = F * warp / kDotParts, j1 = F * (warp + 1) / kDotParts;
+            const float xmax = __uint_as_float(imh_max);
+            for (int g = lane; g < G; g += 32) {
+                const float top = Ts[G * F + g].x * xmax;  // >= sum_j |t_j x_j|
+                const float base = __uint_as_float(min((__float_as_uint(top) >> 23) + 2u, 254u) << 23);
+                float acc = base, err = 0.f;
+#pragma unroll 4
+                for (int j = j0; j < j1; ++j) {
+                    const float2 t = Ts[j * G + g], x = imh[j];
+                    const float sum = fmaf(t.x, x.x, acc);
+                    err = fmaf(t.x, x.y, fmaf(t.y, x.x, err)) + fmaf(t.x, x.x, acc - sum);
+                    acc = sum;
+                }
+                gate_part[warp][g] = make_float2(acc - base, err);
+            }
+        }
+        __syncthreads();
         double term = 0.0;
-        if (tid < G) {
-            float acc = 0.f;
-            for (int j = 0; j < F; ++j) acc = fmaf(Ts[tid * F + j], imh[j], acc);
-            if (gates_out) gates_out[(size_t)p * G + tid] = acc;
+        if (tid < G && (gates_out || ll_out)) {
+            float acc = 0.f, err = 0.f;
+#pragma unroll
+            for (int w = 0; w < kDotParts; ++w) {
+                const float2 v = gate_part[w][tid];
+                float e;
+                two_sum(acc, v.x, acc, e);
+                err += v.y + e;
+            }
+            err = rest(acc, err);
+            const float gate = acc + err;
+            if (gates_out) gates_out[(size_t)p * G + tid] = gate;
             if (ll_out) {
                 const double *yo = y_obs + (obs_per > 0 ? (size_t)(p / obs_per) * G : 0);
                 // FP32 terms (the residual from an FP64 difference, the
                 // variance, one division and one logarithm), FP64 sum: FP64
                 // terms cost this serial epilogue 1 % of the whole launch
-                const float r = (float)(yo[tid] - (double)acc);
-                const float ea = (float)eps_an[tid], q = (float)eps_mn * acc;
+                const float r = (float)(yo[tid] - (double)acc) - err;
+                const float ea = (float)eps_an[tid], q = (float)eps_mn * gate;
                 const float v = fmaf(q, q, ea * ea);
                 term = (double)(__fdiv_rn(r * r, v) + logf(v)) + kLn2Pi;
             }
         }
         if (imh_out)
-            for (int j = tid; j < F; j += blockDim.x) imh_out[(size_t)p * F + j] = imh[j];
+            for (int j = tid; j < F; j += blockDim.x) imh_out[(size_t)p * F + j] = imh[j].x + imh[j].y;
         if (ll_out) {
             if (G <= 32) {
                 // every term is in warp 0: its tree is the whole sum (0 + t = t
@@ -956,7 +1028,7 @@ __global__ void __launch_bounds__(NT, MINB) forward_f32_kernel(ModelsView<float>
 size_t smem_bytes_f32(int F, int G, int K, int LS) {
     const int K2 = (K + 1) / 2;
     return sizeof(ulonglong2) * ((size_t)F * LS + K2) + sizeof(u64) * (size_t)K2 +
-           sizeof(float) * (vals_words(F, K2) + (size_t)F + (size_t)G * F + (size_t)F * LS);
+           sizeof(float) * (vals_words(F, K2) + 2 * (size_t)F + 2 * (size_t)G * (F + 1) + (size_t)F * LS);
 }
 
 // Launch shapes of forward_f32_kernel: threads per CTA, resident CTAs per SM
@@ -1004,8 +1076,8 @@ int launch_shape(const aem_system *sys, const ModelsView<float> &mv, int LS, flo
     if (own)  // stream-ordered: one counter per launch, so launches on other streams never share it
         AEM_CUDA_TRY(cudaMallocAsync((void **)&counter, sizeof(int), stream));
     if (DYN == 1) AEM_CUDA_TRY(cudaMemsetAsync(counter, 0, sizeof(int), stream));
-    kern<<<(unsigned)grid, NT, smem, stream>>>(mv, h.F, h.G, h.K, h.cc_form, LS, sys->len, sys->d_omega_f, sys->d_lamu_f,
-                                               sys->d_hw_f, sys->d_T_f, gates, imh, y_obs, obs_per, eps_an, eps_mn,
+    kern<<<(unsigned)grid, NT, smem, stream>>>(mv, h.F, h.G, h.K, h.cc_form, LS, sys->len, sys->d_omega_f,
+                                               sys->d_wmu_f, sys->d_lamu_f, sys->d_hw_f, sys->d_T_pair, gates, imh, y_obs, obs_per, eps_an, eps_mn,
                                                ll, counter, sys->d_status, active, sys->depth_att, steps, valid);
     const cudaError_t e = cudaGetLastError();
     if (own) cudaFreeAsync(counter, stream);

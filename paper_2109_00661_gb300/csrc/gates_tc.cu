@@ -41,9 +41,12 @@
 #include <type_traits>
 
 #include "aem_internal.h"
+#include "f32x2.h"
 
 namespace aem {
 namespace {
+
+using f32x2::two_sum;
 
 constexpr int kTM = 128;       // models per tile = MMA M
 constexpr int kThreads = 256;  // warps w and w + 4 read TMEM lanes 32 (w mod 4) .., one half of the columns each
@@ -109,13 +112,6 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t mbar, uint32_t parity
     for (uint32_t i = 0; i < limit; ++i)
         if (mbar_try_wait(mbar, parity)) return true;
     return false;
-}
-
-// Knuth's TwoSum: s + e == a + b exactly (round to nearest, no overflow).
-__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
-    s = a + b;
-    const float bb = s - a;
-    e = (a - (s - bb)) + (b - bb);
 }
 
 __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }

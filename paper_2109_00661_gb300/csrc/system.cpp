@@ -299,6 +299,19 @@ static int upload(T **dst, const std::vector<double> &src) {
     return AEM_OK;
 }
 
+// Every value as a float pair: the nearest float and the rest.
+static int upload_pairs(float2 **dst, const std::vector<double> &src) {
+    std::vector<float2> tmp;
+    for (double v : src) {
+        const float hi = (float)v;
+        tmp.push_back(make_float2(hi, (float)(v - (double)hi)));
+    }
+    cudaError_t e = cudaMalloc((void **)dst, sizeof(float2) * tmp.size());
+    if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(table)");
+    e = cudaMemcpy(*dst, tmp.data(), sizeof(float2) * tmp.size(), cudaMemcpyHostToDevice);
+    return e == cudaSuccess ? AEM_OK : cuda_fail(e, "cudaMemcpy(table)");
+}
+
 extern "C" int aem_system_create(const aem_system_desc *desc, aem_system **out) {
     if (!out) return fail(AEM_ERR_INVALID_ARG, "aem_system_create: out is NULL");
     *out = nullptr;
@@ -323,11 +336,20 @@ extern "C" int aem_system_create(const aem_system_desc *desc, aem_system **out) 
     std::vector<double> lamu(h.lam);
     for (double &l : lamu) l *= len;
     s->len = (float)len;
+    std::vector<double> wmu(h.omega);
+    for (double &w : wmu) w *= kMu0 * len * len;
+    std::vector<double> Tb(h.T);  // T, then for every gate F max_f |T| (a bound on its sums, with a margin)
+    for (int g = 0; g < h.G; ++g) {
+        double top = 0;
+        for (int f = 0; f < h.F; ++f) top = std::max(top, std::fabs(h.T[(size_t)g * h.F + f]));
+        Tb.push_back(1.001 * h.F * top);
+    }
     const std::vector<double> &tab64 = f64_tables();
     if ((rc = upload(&s->d_omega_f, h.omega)) || (rc = upload(&s->d_lam_f, h.lam)) || (rc = upload(&s->d_hw_f, h.hw)) ||
         (rc = upload(&s->d_T_f, h.T)) || (rc = upload(&s->d_omega_d, h.omega)) || (rc = upload(&s->d_lam_d, h.lam)) ||
         (rc = upload(&s->d_hw_d, h.hw)) || (rc = upload(&s->d_T_d, h.T)) ||
-        (rc = upload(&s->d_lamu_f, lamu)) || (rc = upload(&s->d_tab64, tab64))) {
+        (rc = upload(&s->d_lamu_f, lamu)) || (rc = upload_pairs(&s->d_wmu_f, wmu)) ||
+        (rc = upload_pairs(&s->d_T_pair, Tb)) || (rc = upload(&s->d_tab64, tab64))) {
         aem_system_destroy(s);
         return rc;
     }
@@ -344,7 +366,7 @@ extern "C" int aem_system_create(const aem_system_desc *desc, aem_system **out) 
 extern "C" int aem_system_destroy(aem_system *s) {
     if (!s) return AEM_OK;
     void *ptrs[] = {s->d_omega_f, s->d_lam_f, s->d_hw_f, s->d_T_f,
-                    s->d_omega_d, s->d_lam_d, s->d_hw_d, s->d_T_d, s->d_lamu_f, s->d_tab64, s->d_status};
+                    s->d_omega_d, s->d_lam_d, s->d_hw_d, s->d_T_d, s->d_lamu_f, s->d_wmu_f, s->d_T_pair, s->d_tab64, s->d_status};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     delete s;
