@@ -155,26 +155,29 @@ int aem_loglik_f64(const aem_system *sys, const aem_models_f64 *models, const do
  * Shapes: 0 = 256 threads per CTA with 4 resident CTAs per SM,
  * 1 = 128 x 8, 2 = 512 x 2, 3 = 256 x 3, 4 = 128 x 6 (the register budget per
  * thread follows from the pair), each with a fixed grid-stride order of
- * models (a recorded 0, the default, stands for "none chosen": launches take
- * shape 2 for at most two models per SM, and above that the one of 0 and 1 of
- * which more threads are resident, its CTAs taking their models dynamically
- * from the grid once there are more models than resident CTAs); 5..9 = the
- * same five with dynamic scheduling (a CTA claims its next model from a counter
- * in stream-ordered scratch when it finishes one).  aem_autotune_forward times
- * every shape that fits on an SM on the caller's sample batch (one untimed
+ * models; 5..9 = the same five with dynamic scheduling (a CTA claims its next
+ * model from a counter in stream-ordered scratch when it finishes one).  While
+ * no shape is recorded for an lmax (the default), launches take shape 2 for at
+ * most two models per SM, and above that the one of 0 and 1 of which more
+ * threads are resident, its CTAs taking their models dynamically once there
+ * are more models than resident CTAs: from the grid itself, without scratch
+ * (10 and 11, the forms of 0 and 1; neither tuned nor recorded, as 5 and 6
+ * are as fast), or from the counter a sampler holds.  aem_autotune_forward times
+ * every shape 0..9 that fits on an SM on the caller's sample batch (one untimed
  * launch, then `repeats` launches timed with CUDA events on `stream`;
  * synchronous), and records the fastest for the sample's lmax in the system:
- * later launches
- * with that lmax use it.  shape_out (may be NULL) receives the choice; ms_out
+ * later launches with that lmax use it.  shape_out (may be NULL) receives the choice; ms_out
  * (may be NULL, AEM_F32_SHAPES floats) the mean time per launch of each shape, -1 for a
  * shape that does not fit.  It takes P x G floats of stream-ordered scratch
  * (cudaMallocAsync) for the duration of the call.  aem_forward_shape sets the
- * shape for an lmax directly.  Not thread-safe against concurrent launches on
+ * shape for an lmax directly; aem_forward_launch_shape reports the shape, 0..11,
+ * that aem_forward_f32 takes for n_models models of that lmax.  Not thread-safe against concurrent launches on
  * the same system. */
 #define AEM_F32_SHAPES 10
 int aem_autotune_forward(aem_system *sys, const aem_models_f32 *sample, int repeats, void *stream, int *shape_out,
                          float *ms_out);
 int aem_forward_shape(aem_system *sys, int lmax, int shape);
+int aem_forward_launch_shape(const aem_system *sys, int lmax, int n_models, int *shape);
 
 /* Depth cutoff of the FP32 forward kernel (aem_forward_f32, aem_loglik_f32,
  * the tensor-core and gradient entries' forward pass and every sampler call

@@ -121,6 +121,14 @@ class System:
         """aem_forward_shape: the FP32 forward kernel's launch shape for lmax."""
         check(_lib.load().aem_forward_shape(self._h, int(lmax), int(shape)), "aem_forward_shape")
 
+    def forward_shape(self, lmax, n_models):
+        """aem_forward_launch_shape: the launch shape (0..11) that forward_f32
+        takes for n_models models of row stride lmax."""
+        shape = ctypes.c_int()
+        check(_lib.load().aem_forward_launch_shape(self._h, int(lmax), int(n_models), ctypes.byref(shape)),
+              "aem_forward_launch_shape")
+        return shape.value
+
     def set_depth_cutoff(self, attenuation):
         """aem_system_set_depth_cutoff: the FP32 forward kernel drops the layers
         below the depth where the round-trip attenuation exceeds

@@ -88,8 +88,11 @@ struct aem_system {
     unsigned int wait_spins = 0;
     int wait_skip_mma = 0;
     // launch shape of the FP32 forward kernel per lmax (index into its shape
-    // table, 0 = default), set by aem_autotune_forward / aem_forward_shape
-    int f32_shape[AEM_MAX_LAYERS + 1] = {};
+    // table, -1 = none recorded), set by aem_autotune_forward / aem_forward_shape
+    int f32_shape[AEM_MAX_LAYERS + 1];
+    aem_system() {
+        for (int &s : f32_shape) s = -1;
+    }
     // CTAs per SM of each kernel, asked once (resident_ctas): the FP32 forward
     // shapes and the adjoint per lmax, the tensor-core transform per mode
     mutable std::atomic<int> fwd_ctas[AEM_F32_SHAPES + 2][AEM_MAX_LAYERS + 1] = {};

@@ -1106,6 +1106,39 @@ int launch_shape_index(int idx, const aem_system *sys, const ModelsView<float> &
 #undef AEM_SHAPE_CASE
 }
 
+// The launch shape of n_models models with row stride LS: the recorded one, or
+// else the rule's.  counter: the caller has a work counter.
+int shape_of_launch(const aem_system *sys, int LS, int n_models, bool counter, int *out) {
+    // No shape recorded.  At most two models per SM: the largest CTAs, which
+    // finish a model soonest.  Otherwise the looped shape of which more threads
+    // are resident (the value buffer of many frequencies and abscissae leaves
+    // room for fewer CTAs), the smaller one on a tie, with dynamic scheduling
+    // once there are more models than resident CTAs.  3,001 and 20,000 models of
+    // up to 10 layers of the 60 x 200 system: 340 and 1889 us at 128 x 8 in
+    // fixed order, 254 and 1472 us; up to 8 layers of the 40 x 120 system, where
+    // 128 x 8 stays: 117 and 671 us, 109 and 555 us.
+    int shape = sys->f32_shape[LS];
+    if (shape < 0) {
+        if (n_models <= 2 * sys->num_sms) {
+            shape = 2;
+        } else {
+            const size_t smem = smem_bytes_f32(sys->host.F, sys->host.G, sys->host.K, LS);
+            int n0 = 0, n1 = 0;
+            if (const int rc = resident_ctas(&sys->fwd_ctas[kFromGrid][LS], forward_f32_kernel<256, 4, 2, false>, 256,
+                                             smem, sys->device, &n0))
+                return rc;
+            if (const int rc = resident_ctas(&sys->fwd_ctas[kFromGrid + 1][LS], forward_f32_kernel<128, 8, 2, false>,
+                                             128, smem, sys->device, &n1))
+                return rc;
+            shape = n1 >= 2 * n0 ? 1 : 0;
+            if (n_models > (long long)sys->num_sms * (shape ? n1 : n0))
+                shape += counter ? kNumBase : kFromGrid;
+        }
+    }
+    *out = shape;
+    return AEM_OK;
+}
+
 template <class Models>
 int launch_forward_f32(const aem_system *sys, const Models *models, float *gates, float *imh, const double *y_obs,
                        int obs_per, const double *eps_an, double eps_mn, double *ll, void *stream, const char *name,
@@ -1122,32 +1155,8 @@ int launch_forward_f32(const aem_system *sys, const Models *models, float *gates
     ModelsView<float> mv{models->n_models, models->lmax, models->nlayers, models->logsig, models->logh,
                            models->m, models->logtau, models->c};
     const int LS = models->lmax;
-    // No shape recorded.  At most two models per SM: the largest CTAs, which
-    // finish a model soonest.  Otherwise the looped shape of which more threads
-    // are resident (the value buffer of many frequencies and abscissae leaves
-    // room for fewer CTAs), the smaller one on a tie, with dynamic scheduling
-    // once there are more models than resident CTAs.  3,001 and 20,000 models of
-    // up to 10 layers of the 60 x 200 system: 340 and 1889 us at 128 x 8 in
-    // fixed order, 254 and 1472 us; up to 8 layers of the 40 x 120 system, where
-    // 128 x 8 stays: 117 and 671 us, 109 and 555 us.
-    int shape = sys->f32_shape[LS];
-    if (shape == 0) {
-        if (models->n_models <= 2 * sys->num_sms) {
-            shape = 2;
-        } else {
-            const size_t smem = smem_bytes_f32(sys->host.F, sys->host.G, sys->host.K, LS);
-            int n0 = 0, n1 = 0;
-            if (const int rc = resident_ctas(&sys->fwd_ctas[kFromGrid][LS], forward_f32_kernel<256, 4, 2, false>, 256,
-                                             smem, sys->device, &n0))
-                return rc;
-            if (const int rc = resident_ctas(&sys->fwd_ctas[kFromGrid + 1][LS], forward_f32_kernel<128, 8, 2, false>,
-                                             128, smem, sys->device, &n1))
-                return rc;
-            shape = n1 >= 2 * n0 ? 1 : 0;
-            if (models->n_models > (long long)sys->num_sms * (shape ? n1 : n0))
-                shape += counter_ext ? kNumBase : kFromGrid;
-        }
-    }
+    int shape = 0;
+    if (const int rc = shape_of_launch(sys, LS, models->n_models, counter_ext != nullptr, &shape)) return rc;
     return launch_shape_index(shape, sys, mv, LS, gates, imh, y_obs, obs_per, eps_an, eps_mn, ll,
                               (cudaStream_t)stream, counter_ext, active, steps, valid);
 }
@@ -1278,4 +1287,10 @@ extern "C" int aem_forward_shape(aem_system *sys, int lmax, int shape) {
         return fail(AEM_ERR_INVALID_ARG, "aem_forward_shape: invalid lmax or shape");
     sys->f32_shape[lmax] = shape;
     return AEM_OK;
+}
+
+extern "C" int aem_forward_launch_shape(const aem_system *sys, int lmax, int n_models, int *shape) {
+    if (!sys || lmax < 1 || lmax > AEM_MAX_LAYERS || n_models < 0 || !shape)
+        return fail(AEM_ERR_INVALID_ARG, "aem_forward_launch_shape: NULL pointer, invalid lmax or n_models < 0");
+    return shape_of_launch(sys, lmax, n_models, false, shape);
 }
