@@ -125,7 +125,11 @@ typedef struct {
  * optionally Im Hz_s at the frequency nodes (imh [device, P*F], may be NULL;
  * gates may be NULL if only imh is wanted).  The f32 entry computes the
  * layer recursion, Hankel sum and gate transform in FP32; the f64 entry is
- * the plain double-precision form of the same arithmetic. */
+ * the plain double-precision form of the same arithmetic.  Asynchronous.  The
+ * f32 entry, and every call that evaluates the FP32 forward model, records
+ * AEM_ERR_TIMEOUT in the system's status word (aem_system_status) should a
+ * CTA's bounded wait for its next model give up; it then waits once more and
+ * evaluates that model all the same. */
 int aem_forward_f32(const aem_system *sys, const aem_models_f32 *models, float *gates, float *imh, void *stream);
 /* aem_forward_f32 that also adds to *layer_steps ([device] unsigned long
  * long, caller-initialised) the number of (layer, abscissa pair) steps its
@@ -230,17 +234,23 @@ int aem_loglik_f32_tc(const aem_system *sys, const aem_models_f32 *models, const
  * AEM_ERR_TIMEOUT a kernel recorded since the last call. */
 int aem_system_status(const aem_system *sys, int *status);
 
-/* Diagnostics of the bounded device wait (for tests; no counterpart in the
+/* Diagnostics of the bounded device waits (for tests; no counterpart in the
  * paper).  spins > 0 sets the iteration limit of the tensor-core transform's
- * completion wait (0 restores the default, 2^22 polls); skip_first_mma = 1
- * makes each CTA of that kernel issue no MMA and no commit for its first
+ * completion wait and of the FP32 forward kernel's wait for the next model
+ * when its CTAs take their models from the grid (launch shapes 10 and 11; 1
+ * polls not at all, so that wait runs out: the kernel records
+ * AEM_ERR_TIMEOUT in the status word, waits again with the default limit and
+ * goes on with the answer, every output written).  0 restores the default,
+ * 2^22 polls.  skip_first_mma = 1
+ * makes each CTA of the transform issue no MMA and no commit for its first
  * tile, so its wait runs out with no tensor-core work in flight: the CTA then
  * records AEM_ERR_TIMEOUT in the status word, frees its tensor memory and
  * returns, leaving the outputs of its tiles unwritten.  The limit applies to
- * the first wait only; the wait for a CTA's own MMAs after a timeout keeps the
- * full limit (should that one also run out, the MMAs may still be in flight
- * when the tensor memory is freed, which is undefined: treat a context that
- * reported a timeout as unreliable).  Not thread-safe against launches on the
+ * the first wait only; the wait for a CTA's own MMAs (or model request) after a
+ * timeout keeps the full limit (should that one also run out, the MMAs may
+ * still be in flight when the tensor memory is freed, or the request when the
+ * CTA leaves, which is undefined: treat a context that reported a timeout as
+ * unreliable).  Not thread-safe against launches on the
  * same system.  skip_first_mma must be 0 or 1 (AEM_ERR_INVALID_ARG). */
 int aem_debug_bounded_wait(aem_system *sys, unsigned int spins, int skip_first_mma);
 

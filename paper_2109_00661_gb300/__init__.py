@@ -265,7 +265,8 @@ def loglik_f32_tc(system, models, y_obs, eps_an, eps_mn, mode=GATES_TF32_SPLIT, 
 
 
 def debug_bounded_wait(system, spins=0, skip_first_mma=False):
-    """aem_debug_bounded_wait: the tensor-core transform's completion-wait limit
+    """aem_debug_bounded_wait: the limit of the tensor-core transform's completion
+    wait and of the forward kernel's wait for its next model
     (0: the default) and whether its CTAs skip the first tile's MMAs (tests)."""
     check(_lib.load().aem_debug_bounded_wait(system.handle, int(spins), int(skip_first_mma)),
           "aem_debug_bounded_wait")

@@ -83,8 +83,8 @@ struct aem_system {
     // device status word: kernels record AEM_ERR_TIMEOUT here when a bounded
     // wait gives up (read and cleared by aem_system_status)
     int *d_status = nullptr;
-    // diagnostics of the tensor-core transform's bounded wait (aem_debug_bounded_wait):
-    // iteration limit (0: the default) and whether CTAs issue nothing for their first tile
+    // diagnostics of the bounded waits (aem_debug_bounded_wait): their iteration limit (0: the
+    // default) and whether the tensor-core transform's CTAs issue nothing for their first tile
     unsigned int wait_spins = 0;
     int wait_skip_mma = 0;
     // launch shape of the FP32 forward kernel per lmax (index into its shape

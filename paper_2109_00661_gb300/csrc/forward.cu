@@ -581,7 +581,7 @@ struct alignas(16) Claim {
     unsigned long long bar;
     unsigned parity;
 };
-constexpr int kClaimSpins = 1 << 22;  // a bound on the wait; an answer takes about a microsecond
+constexpr unsigned kClaimSpins = 1u << 22;  // a bound on the wait; an answer takes about a microsecond
 
 __device__ __forceinline__ void claim_init(Claim *c) {
     c->parity = 0;
@@ -597,21 +597,29 @@ __device__ __forceinline__ void claim_ask(Claim *c) {
         "r"(b)
         : "memory");
 }
-// The index taken over, or n when none is left (or the bound ran out: recorded in *status).
-__device__ __forceinline__ int claim_answer(Claim *c, int n, int *status) {
-    const unsigned a = (unsigned)__cvta_generic_to_shared(c->answer), b = (unsigned)__cvta_generic_to_shared(&c->bar);
-    const unsigned parity = c->parity;
-    c->parity = parity ^ 1;
+// At most limit - 1 polls of the answer's barrier.
+__device__ __forceinline__ bool claim_wait(unsigned bar, unsigned parity, unsigned limit) {
     unsigned ok = 0;
-    for (int i = 0; i < kClaimSpins && !ok; ++i)
+    for (unsigned i = 1; i < limit && !ok; ++i)
         asm volatile(
             "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
             : "=r"(ok)
-            : "r"(b), "r"(parity)
+            : "r"(bar), "r"(parity)
             : "memory");
-    if (!ok) {
+    return ok != 0;
+}
+// The index taken over, or n when none is left.  A wait that runs out is
+// recorded in *status and waited for once more: the request is in flight
+// into this CTA's shared memory, and the CTA it cancels has left its model to
+// this one.  Should that wait run out too, the launch ends without the models
+// of this CTA's answer (and the context should be treated as unreliable).
+__device__ __forceinline__ int claim_answer(Claim *c, int n, int *status, unsigned limit) {
+    const unsigned a = (unsigned)__cvta_generic_to_shared(c->answer), b = (unsigned)__cvta_generic_to_shared(&c->bar);
+    const unsigned parity = c->parity;
+    c->parity = parity ^ 1;
+    if (!claim_wait(b, parity, limit)) {
         atomicExch(status, (int)AEM_ERR_TIMEOUT);
-        return n;
+        if (!claim_wait(b, parity, kClaimSpins)) return n;
     }
     unsigned got, x;
     asm volatile(
@@ -674,7 +682,7 @@ __global__ void __launch_bounds__(NT, MINB) forward_f32_kernel(ModelsView<float>
                                                                const double *__restrict__ eps_an, double eps_mn,
                                                                double *__restrict__ ll_out,
                                                                int *__restrict__ work_counter,
-                                                               int *__restrict__ status,
+                                                               int *__restrict__ status, unsigned claim_limit,
                                                                const int *__restrict__ active, float att0,
                                                                unsigned long long *__restrict__ steps_out,
                                                                const int8_t *__restrict__ valid) {
@@ -731,7 +739,7 @@ __global__ void __launch_bounds__(NT, MINB) forward_f32_kernel(ModelsView<float>
             if (DYN == 2 && tid == 0) claim_ask(&claim);
         };
         auto claimed = [&] {  // into next_model, before a barrier
-            if (DYN == 2 && tid == 0) next_model = claim_answer(&claim, mv.n, status);
+            if (DYN == 2 && tid == 0) next_model = claim_answer(&claim, mv.n, status, claim_limit);
         };
         if (valid && !valid[p]) {  // a proposal the caller will not use (CTA-uniform)
             ask();
@@ -1078,7 +1086,8 @@ int launch_shape(const aem_system *sys, const ModelsView<float> &mv, int LS, flo
     if (DYN == 1) AEM_CUDA_TRY(cudaMemsetAsync(counter, 0, sizeof(int), stream));
     kern<<<(unsigned)grid, NT, smem, stream>>>(mv, h.F, h.G, h.K, h.cc_form, LS, sys->len, sys->d_omega_f,
                                                sys->d_wmu_f, sys->d_lamu_f, sys->d_hw_f, sys->d_T_pair, gates, imh, y_obs, obs_per, eps_an, eps_mn,
-                                               ll, counter, sys->d_status, active, sys->depth_att, steps, valid);
+                                               ll, counter, sys->d_status,
+                                               sys->wait_spins ? sys->wait_spins : kClaimSpins, active, sys->depth_att, steps, valid);
     const cudaError_t e = cudaGetLastError();
     if (own) cudaFreeAsync(counter, stream);
     AEM_CUDA_TRY(e);
