@@ -367,9 +367,14 @@ __device__ inline T warp_sum_t(T v) {
 // FP64 only where TESS is close to alpha N: each probe is evaluated in FP32
 // first (error about 3e-6 of TESS) and decided there while it is further than
 // kScreen from the target; at the first probe that is not, the crossing itself
-// is found by Newton's method on the FP64 TESS with the FP32 slope (kept inside
-// the bracket) in about three evaluations, and the remaining halvings compare
-// their midpoint with it.  Where that does not settle, the remaining probes are
+// is found on the FP64 TESS in two to four evaluations: a Newton step with the
+// FP32 slope, then secant steps through the last two evaluations (kept inside
+// the bracket), and the remaining halvings compare their midpoint with it.
+// The FP32 slope alone, which cancels where the weights are nearly uniform,
+// left the crossing 10 to 20 times as far off as FP64 halvings do (4,096
+// particles in 20 models: 1.1e-14 at alpha 0.5, 2.5e-12 at 0.999; with the
+// secant 1.0e-15 and 3.3e-13, FP64 halvings 5.4e-16 and 2.9e-13: what the
+// rounding of TESS leaves).  Where that does not settle, the remaining probes are
 // evaluated in FP64 one by one.  One more FP64 evaluation at the step taken
 // gives the weights and log Z.
 //
@@ -385,7 +390,12 @@ __device__ inline T warp_sum_t(T v) {
 // 9,600 particles in 20 models, alpha 0.5: 3.9 ms with every probe in FP64 on
 // one SM, 116 us now (16 FP32 probes of 2.6 us, three FP64 ones of 13.7 us).
 constexpr double kScreen = 1e-4;    // of alpha N
-constexpr double kSettled = 1e-10;  // relative step after which the next one is below 2^-49 (slope to 1e-5)
+// The relative step after which no other is made.  The last one leaves its
+// length times the slope's relative error: the secant's is about 1e-5 where the
+// two TESS differ by more than kSecant (their rounding, 1e-15, is all there is
+// to it), and the FP32 slope, kept where they do not, is good to 1e-3.
+constexpr double kSettled = 1e-10;
+constexpr double kSecant = 1e-10;  // of alpha N
 constexpr int kNewton = 8;
 constexpr int kMaxCluster = 8;
 
@@ -718,7 +728,7 @@ __global__ void __launch_bounds__(kGroupThreads) reweight_kernel(const RwArgs a)
     };
     if (warp == 0) ask_screen(hi);
     __syncthreads();
-    float slope = 0.f;
+    double slope = 0.0, xp = 0.0, tp = 0.0;  // xp, tp: the evaluation before
     for (;;) {
         const int op = s_op;
         if (op == kOpScreen)
@@ -728,12 +738,12 @@ __global__ void __launch_bounds__(kGroupThreads) reweight_kernel(const RwArgs a)
         if (op == kOpFinal) break;
         if (warp == 0) {
             if (op == kOpScreen) {
-                float t = 0.f;
-                slope = 0.f;
+                float t = 0.f, d = 0.f;
                 for (int w = 0; w < nw; ++w) {
                     t += s_fred[0][w];
-                    slope += s_fred[1][w];
+                    d += s_fred[1][w];
                 }
+                slope = (double)d;
                 const double off = (double)t - target;
                 if (fabs(off) > kScreen * target) {
                     next(off >= 0.0);
@@ -743,7 +753,7 @@ __global__ void __launch_bounds__(kGroupThreads) reweight_kernel(const RwArgs a)
                         newton = 0;
                         xa = lo;
                         xb = hi;
-                        y = x - off / (double)slope;  // FP32's own step first
+                        y = x - off / slope;  // FP32's own step first
                         if (!(y > xa && y < xb)) y = x;
                     }
                     ask(kOpEvaluate, y);
@@ -755,14 +765,21 @@ __global__ void __launch_bounds__(kGroupThreads) reweight_kernel(const RwArgs a)
                     if (it >= 0) how = 2;
                     next(t >= target);
                 } else {
-                    // Newton's method for the crossing, started at this halving's midpoint
+                    // the crossing, started at this halving's midpoint
+                    if (newton > 0 && fabs(t - tp) > kSecant * target) {
+                        const double s = (t - tp) / (x - xp);
+                        if (s < 0.0) slope = s;
+                    }
+                    tp = t;
+                    xp = x;
                     if (t >= target)
                         xa = x;
                     else
                         xb = x;
-                    double y = x - (t - target) / (double)slope;
-                    const bool in = y > xa && y < xb;  // false for NaN
-                    const bool settled = in && fabs(y - x) <= kSettled * x;
+                    double y = x - (t - target) / slope;
+                    const bool in = y > xa && y < xb;                 // false for NaN, as the next
+                    const bool settled = fabs(y - x) <= kSettled * x;  // t = target among them: y = x, an end of the bracket
+                    if (settled) y = fmin(fmax(y, xa), xb);
                     if (!settled && ++newton < kNewton) {
                         ask(kOpEvaluate, in ? y : 0.5 * (xa + xb));
                     } else {
