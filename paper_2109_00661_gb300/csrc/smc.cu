@@ -477,13 +477,17 @@ __global__ void __launch_bounds__(kGroupThreads) reweight_kernel(const RwArgs a)
         return k;
     };
     // per-model maxima: this slice's by integer comparison (the doubles' bits in
-    // an order-preserving form), then the cluster's
+    // an order-preserving form; a NaN of either sign is the largest, so that its
+    // model's terms are NaN and its ESS 0 in every evaluation), then the cluster's
     for (int i = tid; i < own; i += kGroupThreads) {
         const double v = a.ll[perm[lo_pos + i]];
         const int k = first_model(lo_pos + i);
         v64[i] = v;
         md[i] = (unsigned char)k;
-        const long long b = __double_as_longlong(v);
+        long long b = __double_as_longlong(v);
+        // a constant: the sign of a NaN cleared in its bits came back set (the
+        // compiler may take that for a floating-point absolute value)
+        if ((b & 0x7fffffffffffffffll) > 0x7ff0000000000000ll) b = 0x7fffffffffffffffll;
         atomicMax(&p_key[k], b ^ ((b >> 63) & 0x7fffffffffffffffll));
     }
     __syncthreads();
