@@ -101,9 +101,10 @@ __device__ __forceinline__ void exp_c(double wre, double wim, const Thick &t, co
     const double T = tab->ex[k & (kExN - 1)];
     double e = fma(q * f, T, T);
     e = __hiloint2double(__double2hiint(e) + (int)((unsigned)(k >> 8) << 20), __double2loint(e));
-    // below exp(-700): the steps themselves, from n's bits (a NaN stays)
+    // below exp(-700): the steps themselves, from n's bits (a NaN of either sign
+    // stays, and so does a thickness of infinity: exp(-inf) (cos, sin)(-inf))
     constexpr long long kGone = 0x4338000000000000ll - 258530;
-    const bool gone = __double_as_longlong(n) < kGone;
+    const bool gone = __double_as_longlong(n) < kGone && (unsigned)__double2hiint(n) < 0xfff00000u;
     const double m = fma(t.hp, wim, kShift);
     double sn, cs;
     if ((unsigned)(__double2hiint(m) - 0x43380000 + 0x20000) < 0x40000u) {  // |steps| < 2^49
