@@ -56,18 +56,20 @@ struct ModelsView {
 // of FP64 operations, and everything else is free: roots and reciprocals take
 // the hardware's 20-bit estimates and one third-order step, the exponential and
 // the sine and cosine a table in shared memory and a short polynomial, signs,
-// exponents and table indices integer instructions.  53 FP64 operations per
-// layer-step (154 with the library's sqrt, rsqrt, division, exp and sincos, 71
-// with interface coefficients and 64-entry tables): 1,024 models of 1..10
-// layers, 60 frequencies, 200 abscissae, 20.0 -> 9.06 -> 7.06 ms, at the rate the
-// FP64 pipe allows.
+// exponents and table indices integer instructions.  61 FP64 operations per
+// layer-step (154 with the library's sqrt, rsqrt, division, exp and sincos):
+// 1,024 models of 1..10 layers, 60 frequencies, 200 abscissae, 19.4 -> 7.71 ms,
+// at the rate the FP64 pipe allows.
 //
-// The recursion carries the tangential field e and h = w (D - P) upwards, with
-// w = sqrt(2) u, D and N = R D the down- and upgoing amplitudes at the bottom
-// of a layer and P = N E: both are continuous across an interface, where
-//   D = w e + h,  N = w e - h,  then  e = D + N E,  h = w (D - N E)
-// (scaled by w at every interface, which 64-bit exponents hold; no interface
-// coefficient and no division), and R_0 = (w_air e - h) / (w_air e + h).
+// The recursion is the FP32 kernel's, (N, D) <- (r D + N E, D + r N E) in w =
+// sqrt(2) u with the interface coefficient from the roots and their moduli.
+// Carrying the field (e = D + P, h = w (D - P)) in place of r takes 53
+// operations (7.0 ms), but e and h then keep the phase of the layers below,
+// which Im R_0 has to cancel even where the layers above hide them: an error of
+// 2^-53 times the conductivity contrast, 3e-12 of the spectrum on layers of
+// 1e-4 and 1 S/m under a small loop near the ground and 1e-7 at a contrast of
+// 1e16.  Here it is 5e-16 and 1e-14, on all stacks tried no more than with
+// the library's functions and the differenced s.
 namespace f64 {
 
 constexpr int kExN = kTab64Octave, kScN = kTab64Turn;
@@ -129,6 +131,9 @@ struct Rec {  // per frequency and layer
 struct C {
     double x, y;
 };
+struct Root {  // w = sqrt(2 (lambda^2 + s)) and m = |w|^2 / 2
+    double x, y, m;
+};
 
 // w = sqrt(2 (x + i y)).  From the 20-bit estimate y of 1 / sqrt(v), g = v y and
 // e = 1 - g y: sqrt(v) = g (1 + c) and 1 / sqrt(v) = y (1 + c) with c = e (1/2 +
@@ -138,7 +143,7 @@ __device__ __forceinline__ double rsq_est(double v) {
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(v));
     return y;
 }
-__device__ __forceinline__ C root(double lam2, const Rec &s) {
+__device__ __forceinline__ Root root(double lam2, const Rec &s) {
     const double x = lam2 + s.sx;
     const double v = fma(x, x, s.sy2);
     const double y1 = rsq_est(v), g1 = v * y1, e1 = fma(-g1, y1, 1.0);
@@ -148,45 +153,51 @@ __device__ __forceinline__ C root(double lam2, const Rec &s) {
     const double c = e2 * fma(e2, 0.375, 0.5);
     const double p = fma(c, g2, g2), o = s.sy * fma(c, y2, y2);
     const bool pos = __double2hiint(x) >= 0;
-    return {pos ? p : o, pos ? o : p};
+    return {pos ? p : o, pos ? o : p, m};
+}
+__device__ __forceinline__ double rcp(double v) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(v));
+    const double r = fma(-v, y, 1.0);  // 1 / v = y (1 + r + r^2 + ..)
+    return fma(fma(r, r, r), y, y);
+}
+// The interface coefficient between a (above) and b from the roots and their
+// moduli (the form of te_roots.h), and that of the air above the top layer, whose
+// root is the real wair and modulus lam2.
+__device__ __forceinline__ C rcoef(const Root &a, const Root &b) {
+    const double i = rcp(fma(a.y, b.y, fma(a.x, b.x, a.m + b.m)));
+    return {(a.m - b.m) * i, fma(a.y, b.x, -(a.x * b.y)) * i};
+}
+__device__ __forceinline__ C rcoef_air(double lam2, double wair, const Root &b) {
+    const double i = rcp(fma(wair, b.x, lam2 + b.m));
+    return {(lam2 - b.m) * i, -(wair * b.y) * i};
 }
 
 // Im R_0 of one (lambda, frequency); rec: the frequency's layers.
 __device__ __forceinline__ double im_r0(double lam2, double wair, const Rec *__restrict__ rec,
                                         const Thick *__restrict__ th, int L, const Tables *tab) {
-    C h = root(lam2, rec[L - 1]), D, N;
-    if (L == 1) {
-        D = {wair + h.x, h.y};
-        N = {wair - h.x, -h.y};
-    } else {
-        C w = root(lam2, rec[L - 2]), e;
-        D = {w.x + h.x, w.y + h.y};
-        N = {w.x - h.x, w.y - h.y};
+    Root b = root(lam2, rec[L - 1]);
+    if (L == 1) return rcoef_air(lam2, wair, b).y;
+    Root a = root(lam2, rec[L - 2]);
+    C N = rcoef(a, b), D = {1.0, 0.0};
 #pragma unroll 1
-        for (int n = L - 2;; --n) {
-            double Ex, Ey;
-            exp_c(w.x, w.y, th[n], tab, Ex, Ey);
-            e = {fma(N.x, Ex, fma(-N.y, Ey, D.x)), fma(N.x, Ey, fma(N.y, Ex, D.y))};
-            const C b = {fma(2.0, D.x, -e.x), fma(2.0, D.y, -e.y)};
-            h = {fma(w.x, b.x, -(w.y * b.y)), fma(w.x, b.y, w.y * b.x)};
-            if (n == 0) break;
-            w = root(lam2, rec[n - 1]);
-            D = {fma(w.x, e.x, fma(-w.y, e.y, h.x)), fma(w.x, e.y, fma(w.y, e.x, h.y))};
-            N = {fma(-2.0, h.x, D.x), fma(-2.0, h.y, D.y)};
+    for (int n = L - 2;; --n) {
+        double Ex, Ey;
+        exp_c(a.x, a.y, th[n], tab, Ex, Ey);
+        C r;
+        if (n > 0) {
+            b = a;
+            a = root(lam2, rec[n - 1]);
+            r = rcoef(a, b);
+        } else {
+            r = rcoef_air(lam2, wair, a);
         }
-        D = {fma(wair, e.x, h.x), fma(wair, e.y, h.y)};
-        N = {fma(-2.0, h.x, D.x), fma(-2.0, h.y, D.y)};
+        const C P = {fma(N.x, Ex, -(N.y * Ey)), fma(N.x, Ey, N.y * Ex)};
+        N = {fma(r.x, D.x, fma(-r.y, D.y, P.x)), fma(r.x, D.y, fma(r.y, D.x, P.y))};
+        D = {fma(r.x, P.x, fma(-r.y, P.y, D.x)), fma(r.x, P.y, fma(r.y, P.x, D.y))};
+        if (n == 0) break;
     }
-    // |D| to about one by a power of two: the squares stay in range
-    const int top = max(__double2hiint(D.x) & 0x7ff00000, __double2hiint(D.y) & 0x7ff00000);
-    const double z = __hiloint2double(min(max(0x7fe00000 - top, 0x00100000), 0x7fd00000), 0);
-    D = {D.x * z, D.y * z};
-    N = {N.x * z, N.y * z};
-    const double v = fma(D.x, D.x, D.y * D.y);
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(v));
-    const double r = fma(-v, y, 1.0);  // 1 / v = y (1 + r + r^2 + ..)
-    return fma(N.y, D.x, -(N.x * D.y)) * fma(fma(r, r, r), y, y);
+    return fma(N.y, D.x, -(N.x * D.y)) * rcp(fma(D.x, D.x, D.y * D.y));
 }
 
 }  // namespace f64
