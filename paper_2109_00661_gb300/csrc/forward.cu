@@ -435,10 +435,10 @@ int launch_forward_f64(const aem_system *sys, const aem_models_f64 *models, doub
 //   E = exp(-2 u h) = exp2(e w.x) (cos(e ln2 w.y) + i sin(e ln2 w.y)),
 //   e = -sqrt(2) h log2(e).
 // The Moebius step (N, D) <- (r D + N E, D + r N E) keeps R_0 = N / D.
-// Lengths are counted in the power of two next to the system's 2 h + a
+// Lengths are counted in a power of two of the order of the system's 2 h + a
 // (aem_system::len: lambda, s and h scaled by it exactly), so that |lambda^2 + s|^2
 // and the product of two reciprocals' arguments stay inside the FP32 range
-// whatever the geometry.
+// whatever the geometry, for conductivities past any metal's.
 using namespace f32x2;  // paired FP32 helpers and the hardware approximations (f32x2.h)
 
 constexpr double kLn2Pi = 1.83787706640934548356;  // ln(2 pi)

@@ -332,7 +332,10 @@ extern "C" int aem_system_create(const aem_system_desc *desc, aem_system **out) 
         return cuda_fail(e, "cudaDeviceGetAttribute");
     }
     const SystemTables &h = s->host;
-    const double len = std::exp2(std::floor(std::log2(2.0 * h.h + h.a)));
+    // 2^-8 of 2 h + a: the abscissae reach down to 1e-5 / (2 h + a), whose fourth
+    // power in this unit is still 1e-31, and |s|^2 stays finite up to s of 1e18
+    // in it: 1e14 S/m at 10 MHz under a loop at 3 km
+    const double len = std::exp2(std::floor(std::log2(2.0 * h.h + h.a)) - 8.0);
     std::vector<double> lamu(h.lam);
     for (double &l : lamu) l *= len;
     s->len = (float)len;
