@@ -412,7 +412,7 @@ size_t reweight_smem_bytes(int N, int C) {
 
 struct RwArgs {
     const double *ll;
-    const int *perm, *off, *counts;
+    const int *perm, *off;
     int N, M;
     double alpha;
     int iters;
@@ -2532,9 +2532,9 @@ static int take_status(smc_state *st) {
 }
 
 static int launch_reweight(smc_state *st, cudaStream_t stream) {
-    const RwArgs a{st->cur.ll, st->perm,  st->off,  st->counts, st->N,   st->M,   st->d.alpha, st->d.bisect_iters,
-                   st->gamma,  0.0,       st->gamma, st->logz,  1,       st->Wg,  nullptr,     st->dgamma,
-                   st->done,   st->d_status};
+    const RwArgs a{st->cur.ll, st->perm, st->off,   st->N,   st->M, st->d.alpha, st->d.bisect_iters, st->gamma,
+                   0.0,        st->gamma, st->logz, 1,       st->Wg, nullptr,    st->dgamma,         st->done,
+                   st->d_status};
     return launch_reweight(a, st->S, st->sys->num_sms, stream);
 }
 
@@ -3263,39 +3263,33 @@ extern "C" int smc_restore(smc_state *st, const void *buf, size_t size) {
 }
 
 // ----------------------------------------------------- standalone entries
-extern "C" size_t aem_smc_workspace_bytes(int n, int n_models) {
-    if (n < 0 || n_models < 1) return 0;
-    size_t b = 0;
-    b += sizeof(int) * 2 * (size_t)n;                 // kappa, lam split of the model ids
-    b += sizeof(int) * (size_t)n;                     // perm
-    b += sizeof(int) * (size_t)(2 * n_models + 1);    // off, counts
-    b += sizeof(double) * (size_t)n;                  // grouped weights
-    b += sizeof(unsigned long long) * (size_t)n;      // integer CDF
-    b += sizeof(double) + sizeof(int) + 64 * 8;       // gamma, done, alignment slack
-    return b;
-}
-
 namespace {
 struct Workspace {
-    double *Wg;
     int *perm, *off, *counts;
 };
 
-Workspace carve(void *base, int n, int M) {
-    auto align = [](size_t v) { return (v + 63) & ~(size_t)63; };
-    char *p = (char *)base;
+// Lays a workspace out from base (64-byte aligned; null: the size alone) and
+// returns its size.
+size_t carve(void *base, int n, int M, Workspace *w) {
     size_t o = 0;
+    auto take = [&](int **q, size_t count) {
+        *q = base ? (int *)((char *)base + o) : nullptr;
+        o += (sizeof(int) * count + 63) & ~(size_t)63;
+    };
+    take(&w->perm, (size_t)n);
+    take(&w->off, (size_t)M + 1);
+    take(&w->counts, (size_t)M);
+    return o;
+}
+}  // namespace
+
+extern "C" size_t aem_smc_workspace_bytes(int n, int n_models) {
+    if (n < 0 || n_models < 1) return 0;
     Workspace w;
-    w.Wg = (double *)(p + o);
-    o = align(o + sizeof(double) * n);
-    w.perm = (int *)(p + o);
-    o = align(o + sizeof(int) * n);
-    w.off = (int *)(p + o);
-    o = align(o + sizeof(int) * (M + 1));
-    w.counts = (int *)(p + o);
-    return w;
+    return carve(nullptr, n, n_models, &w);
 }
 
+namespace {
 int check_standalone(int n, int n_models, const void *work, size_t bytes, const char *name) {
     if (n < 1 || n > AEM_SMC_MAX_PARTICLES || n_models < 1 || n_models > AEM_SMC_MAX_MODELS)
         return fail(AEM_ERR_INVALID_ARG, std::string(name) + ": n or n_models out of range");
@@ -3314,7 +3308,8 @@ extern "C" int aem_reweight(const double *ll, const int *model, int n, int n_mod
         !(gamma_prev >= 0 && gamma_prev < 1) || bisect_iters < 1 || bisect_iters > 200)
         return fail(AEM_ERR_INVALID_ARG, "aem_reweight: NULL pointer or value out of range");
     cudaStream_t s = (cudaStream_t)stream;
-    Workspace w = carve(work, n, n_models);
+    Workspace w;
+    carve(work, n, n_models, &w);
     if ((rc = stage_kernel_attributes())) return rc;
     int dev = 0, num_sms = 0;
     AEM_CUDA_TRY(cudaGetDevice(&dev));
@@ -3322,8 +3317,8 @@ extern "C" int aem_reweight(const double *ll, const int *model, int n, int n_mod
     group_kernel<<<1, kGroupThreads, group_smem_bytes(n), s>>>(nullptr, nullptr, model, n, 1, n_models, w.perm, w.off, w.counts, nullptr,
                                              W);
     AEM_CUDA_TRY(cudaGetLastError());
-    const RwArgs a{ll,      w.perm,  w.off,    w.counts, n, n_models, alpha, bisect_iters, nullptr,
-                   gamma_prev, nullptr, logz_inc, 0,     nullptr, W,  dgamma, reached_one, nullptr};
+    const RwArgs a{ll,      w.perm,  w.off,    n, n_models, alpha, bisect_iters, nullptr,
+                   gamma_prev, nullptr, logz_inc, 0, nullptr,  W,     dgamma,       reached_one, nullptr};
     return launch_reweight(a, 1, num_sms, s);
 }
 
@@ -3334,7 +3329,8 @@ extern "C" int aem_resample_systematic(const double *W, const int *model, int n,
     if (rc) return rc;
     if (!W || !model || !u40 || !ancestor) return fail(AEM_ERR_INVALID_ARG, "aem_resample_systematic: NULL pointer");
     cudaStream_t s = (cudaStream_t)stream;
-    Workspace w = carve(work, n, n_models);
+    Workspace w;
+    carve(work, n, n_models, &w);
     if ((rc = stage_kernel_attributes())) return rc;
     group_kernel<<<1, kGroupThreads, group_smem_bytes(n), s>>>(nullptr, nullptr, model, n, 1, n_models, w.perm, w.off, w.counts, ancestor,
                                              nullptr);
