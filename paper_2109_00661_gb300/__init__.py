@@ -47,7 +47,9 @@ def _stream_ptr(stream):
     if stream is not None:
         return ctypes.c_void_p(stream.cuda_stream)
     torch = _torch()
-    return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch.cuda.current_device()))
+    # the handle without a Stream object (1 us less per call) where the release has it
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    return ctypes.c_void_p(raw(torch.cuda.current_device()) if raw else torch.cuda.current_stream().cuda_stream)
 
 
 def _dptr(t):
