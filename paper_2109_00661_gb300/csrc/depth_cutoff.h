@@ -20,9 +20,8 @@ namespace aem {
 // exceeds att (-1: every lambda); non-increasing in j.  s(n) gives (Re s_n,
 // Im s_n), h[n] the thicknesses.  The hardware approximations suffice: the
 // thresholds only need to be right to well under the exp(-att0) margin.
-// Returns ms.
 template <class S>
-__device__ __forceinline__ float depth_thresholds(S s, const float *h, int L, float att0, float *th) {
+__device__ __forceinline__ void depth_thresholds(S s, const float *h, int L, float att0, float *th) {
     using namespace f32x2;
     float s2max = 0.f, ms = 0.f;
     for (int n = 0; n < L; ++n) {
@@ -43,7 +42,6 @@ __device__ __forceinline__ float depth_thresholds(S s, const float *h, int L, fl
         const float q = 0.5f * att * rcp_approx(H);
         th[j] = C > att ? -1.f : fmaf(q, q, ms);
     }
-    return ms;
 }
 
 // The layer count one abscissa needs: 1 + the number of thresholds lambda^2

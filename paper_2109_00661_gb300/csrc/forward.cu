@@ -76,7 +76,7 @@ constexpr int kExN = kTab64Octave, kScN = kTab64Turn;
 constexpr double kShift = 6755399441055744.0;  // 1.5 * 2^52: the low word of x + kShift is round(x)
 
 // Tables of the complex exponential (Tang 1989's scheme): 2^(j / kExN), sine
-// and cosine of 2 pi j / kScN (kTabDoubles in this order, forward_f64_tables).
+// and cosine of 2 pi j / kScN (kTab64Doubles in this order, f64_tables in system.cpp).
 struct Tables {
     double2 sc[kScN];
     double ex[kExN];
@@ -507,6 +507,9 @@ __device__ __forceinline__ void mobius2_d1(C2x2 &N, C2x2 &D, C2x2 r, const Root 
     D.im = fma2(r.re, Py, mul2(r.im, Px));
 }
 
+// A load of the records or exponents by shared-memory address.  It is volatile
+// but clobbers no memory: what orders it after the stores is the barrier between
+// them and the empty clobber that opens every item (item_of).
 __device__ __forceinline__ ulonglong2 lds16(unsigned a) {
     ulonglong2 v;
     asm volatile("ld.shared.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "r"(a));
@@ -870,6 +873,7 @@ __global__ void __launch_bounds__(NT, MINB) forward_f32_kernel(ModelsView<float>
                     }
                     const ulonglong2 lw = KR[k];
                     float v0, v1;
+                    asm volatile("" ::: "memory");  // lds16
                     body(lw, rec_a + (unsigned)(f * LS) * 16u, v0, v1);
                     float h0, h1;
                     up2(HW[k], h0, h1);
