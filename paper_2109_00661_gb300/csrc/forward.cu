@@ -994,7 +994,7 @@ __global__ void __launch_bounds__(NT, MINB) forward_f32_kernel(ModelsView<float>
                 gate_part[warp][g] = make_float2(acc - base, err);
             }
         }
-        __syncthreads();
+        if (gates_out || ll_out) __syncthreads();
         double term = 0.0;
         if (tid < G && (gates_out || ll_out)) {
             float acc = 0.f, err = 0.f;
