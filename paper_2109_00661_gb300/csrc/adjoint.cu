@@ -35,7 +35,7 @@
 // units: about 100 paired operations and 20 special-function ones per pair and
 // layer for both passes.  Differentiating the Moebius chain interface by
 // interface took 163 and 28: 16384 models of 60 x 200 items with 1 to 10
-// layers, forward kernel included, 7.05 -> 4.89 ms.  E_n is formed again on the
+// layers, forward kernel included, 7.05 -> 4.86 ms.  E_n is formed again on the
 // way down: kept from the way up it costs 16 bytes of local memory per layer
 // each way, 5.58 against 5.23 ms.
 #include <cuda_runtime.h>

@@ -677,7 +677,7 @@ __host__ __device__ inline int vals_words(int F, int K2) {
 // earth (40 frequencies, 120 abscissae, up to 8 layers) it is 5.4e-7 of the
 // norm against 64 bits, 1.1e-6 without (1.3e-6 with the differenced s before
 // that); on the 60 x 200 system 4.4e-7 against 1.3e-6, and the gradient's
-// error falls with it by 2 to 4.  32,768 models of the former: 0.94 ms, 0.92
+// error falls with it by 2 to 4.  32,768 models of the former: 0.93 ms, 0.91
 // without (0.95 with TwoProd and TwoSum).
 // The order of every sum is fixed by the item indices alone.  (The throughput
 // system's 60 x 100 items take one round.)
@@ -1063,9 +1063,9 @@ size_t smem_bytes_f32(int F, int G, int K, int LS) {
 // (about 55 steps) overflows the instruction cache when many small CTAs are
 // each at another layer count, while the small CTAs lose less at the barriers
 // between a model's phases.  2^17 random models of the 60-frequency,
-// 200-abscissa system: 9.13 ms unrolled at 256 x 3, 10.8 ms looped at 128 x 8;
-// 32,768 models of the 40-frequency, 120-abscissa one (up to 8 layers): 0.96
-// and 0.89 ms.  (10.34 and 1.07 ms before the interface coefficient of the
+// 200-abscissa system, dynamic: 9.36 ms unrolled at 256 x 3, 10.8 ms looped at 128 x 8;
+// 32,768 models of the 40-frequency, 120-abscissa one (up to 8 layers): 1.03
+// and 0.92 ms.  (10.34 and 1.07 ms before the interface coefficient of the
 // roots alone, all unrolled.)
 struct F32Shape {
     int nt, minb;
@@ -1139,9 +1139,9 @@ int shape_of_launch(const aem_system *sys, int LS, int n_models, bool counter, i
     // are resident (the value buffer of many frequencies and abscissae leaves
     // room for fewer CTAs), the smaller one on a tie, with dynamic scheduling
     // once there are more models than resident CTAs.  3,001 and 20,000 models of
-    // up to 10 layers of the 60 x 200 system: 340 and 1889 us at 128 x 8 in
-    // fixed order, 254 and 1472 us; up to 8 layers of the 40 x 120 system, where
-    // 128 x 8 stays: 117 and 671 us, 109 and 555 us.
+    // up to 10 layers of the 60 x 200 system: 341 and 1950 us at 128 x 8 in
+    // fixed order, 260 and 1486 us; up to 8 layers of the 40 x 120 system, where
+    // 128 x 8 stays: 120 and 654 us, 108 and 555 us.
     int shape = sys->f32_shape[LS];
     if (shape < 0) {
         if (n_models <= 2 * sys->num_sms) {
