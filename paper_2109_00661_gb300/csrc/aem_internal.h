@@ -73,7 +73,7 @@ struct aem_system {
     // abscissae in it
     float len = 1.f, *d_lamu_f = nullptr;
     // float pairs (value, what its rounding left): omega mu0 in that unit [F];
-    // T [G*F], then a bound on each gate's sum of |T| over |Im H| <= 1 [G]
+    // T [F*G] (by frequency), then a bound on each gate's sum of |T| over |Im H| <= 1 [G]
     float2 *d_wmu_f = nullptr, *d_T_pair = nullptr;
     // the FP64 forward kernel's tables: sine and cosine of 2 pi j / kTab64Turn in
     // pairs, then 2^(j / kTab64Octave)

@@ -662,9 +662,9 @@ __host__ __device__ inline int vals_words(int F, int K2) {
 // Shared memory (dynamic), in order: REC[F*LS] (ulonglong2: per frequency and
 // layer the (Re s, Re s) and (Im s, Im s) pairs), KR[K2] (ulonglong2: per
 // abscissa pair the (lambda^2, -sqrt(2) lambda) pairs), HW[K2] (the pairs'
-// Hankel weights), vals[vals_words], imh[F] (float pairs), Ts[(F+1)*G] (float
-// pairs: T by frequency, then the bounds of d_T_pair), TH[F*LS] (float: the
-// depth cutoff's thresholds).  The items (frequency major, F*K2 of
+// Hankel weights), vals[vals_words], imh[F] (float pairs), Ts[F*G] (T by
+// frequency), bound[G] (d_T_pair's), TH[F*LS] (float: the depth cutoff's
+// thresholds).  The items (frequency major, F*K2 of
 // them) are taken in rounds of kValsWords: every item stores its weighted pair
 // value at its own index in the buffer; after the round each frequency the
 // round touched is summed by four consecutive lanes (lane s adds the values at
@@ -677,7 +677,7 @@ __host__ __device__ inline int vals_words(int F, int K2) {
 // earth (40 frequencies, 120 abscissae, up to 8 layers) it is 5.4e-7 of the
 // norm against 64 bits, 1.1e-6 without (1.3e-6 with the differenced s before
 // that); on the 60 x 200 system 4.4e-7 against 1.3e-6, and the gradient's
-// error falls with it by 2 to 4.  32,768 models of the former: 0.93 ms, 0.91
+// error falls with it by 2 to 4.  32,768 models of the former: 0.94 ms, 0.91
 // without (0.95 with TwoProd and TwoSum).
 // The order of every sum is fixed by the item indices alone.  (The throughput
 // system's 60 x 100 items take one round.)
@@ -710,8 +710,8 @@ __global__ void __launch_bounds__(NT, MINB) forward_f32_kernel(ModelsView<float>
     u64 *HW = reinterpret_cast<u64 *>(KR + K2);
     float *vals = reinterpret_cast<float *>(HW + K2);
     float2 *imh = reinterpret_cast<float2 *>(vals + vals_words(F, K2));
-    float2 *Ts = imh + F;
-    float *TH = reinterpret_cast<float *>(Ts + (size_t)G * (F + 1));  // depth-cutoff thresholds, [F][LS]
+    float *Ts = reinterpret_cast<float *>(imh + F), *bound = Ts + (size_t)G * F;
+    float *TH = bound + G;  // depth-cutoff thresholds, [F][LS]
     __shared__ ulonglong2 HE[AEM_MAX_LAYERS];
     __shared__ float lh[AEM_MAX_LAYERS];
     __shared__ float lsig[AEM_MAX_LAYERS], lm[AEM_MAX_LAYERS], ltau[AEM_MAX_LAYERS], lc[AEM_MAX_LAYERS];
@@ -721,10 +721,7 @@ __global__ void __launch_bounds__(NT, MINB) forward_f32_kernel(ModelsView<float>
     __shared__ unsigned imh_max;  // the largest |Im H| of the model, as its bits
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    for (int i = tid; i < G * (F + 1); i += blockDim.x) {
-        const int g = i / F;
-        Ts[g < G ? (i - g * F) * G + g : i] = g_T[i];
-    }
+    for (int i = tid; i < G * (F + 1); i += blockDim.x) Ts[i] = g_T[i].x;
     // abscissa pairs (k, k + K2); an odd K pads the last pair with a zero weight
     for (int k = tid; k < K2; k += blockDim.x) {
         const int kb = k + K2 < K ? k + K2 : K - 1;
@@ -976,19 +973,23 @@ __global__ void __launch_bounds__(NT, MINB) forward_f32_kernel(ModelsView<float>
         // warp, lane = gate.  The sum begins at a power of two above all its
         // partial sums, so that what it rounds off of a product is exact (Dekker's
         // Fast2Sum): t x - (sum after - sum before), six operations a term
-        // where TwoProd and TwoSum take thirteen.
+        // where TwoProd and TwoSum take thirteen.  T's low parts are read from
+        // global memory: beside the high ones they would cost systems of many
+        // gates and frequencies a resident CTA (64 x 128 x 200, 8,000 models:
+        // 2.32 ms against 1.62).
         if (warp < kDotParts && (gates_out || ll_out)) {
             const int j0 = F * warp / kDotParts, j1 = F * (warp + 1) / kDotParts;
             const float xmax = __uint_as_float(imh_max);
             for (int g = lane; g < G; g += 32) {
-                const float top = Ts[G * F + g].x * xmax;  // >= sum_j |t_j x_j|
+                const float top = bound[g] * xmax;  // >= sum_j |t_j x_j|
                 const float base = __uint_as_float(min((__float_as_uint(top) >> 23) + 2u, 254u) << 23);
                 float acc = base, err = 0.f;
 #pragma unroll 4
                 for (int j = j0; j < j1; ++j) {
-                    const float2 t = Ts[j * G + g], x = imh[j];
-                    const float sum = fmaf(t.x, x.x, acc);
-                    err = fmaf(t.x, x.y, fmaf(t.y, x.x, err)) + fmaf(t.x, x.x, acc - sum);
+                    const float t = Ts[j * G + g], lo = __ldg(&g_T[j * G + g].y);
+                    const float2 x = imh[j];
+                    const float sum = fmaf(t, x.x, acc);
+                    err = fmaf(t, x.y, fmaf(lo, x.x, err)) + fmaf(t, x.x, acc - sum);
                     acc = sum;
                 }
                 gate_part[warp][g] = make_float2(acc - base, err);
@@ -1052,7 +1053,7 @@ __global__ void __launch_bounds__(NT, MINB) forward_f32_kernel(ModelsView<float>
 size_t smem_bytes_f32(int F, int G, int K, int LS) {
     const int K2 = (K + 1) / 2;
     return sizeof(ulonglong2) * ((size_t)F * LS + K2) + sizeof(u64) * (size_t)K2 +
-           sizeof(float) * (vals_words(F, K2) + 2 * (size_t)F + 2 * (size_t)G * (F + 1) + (size_t)F * LS);
+           sizeof(float) * (vals_words(F, K2) + 2 * (size_t)F + (size_t)G * (F + 1) + (size_t)F * LS);
 }
 
 // Launch shapes of forward_f32_kernel: threads per CTA, resident CTAs per SM

@@ -341,11 +341,16 @@ extern "C" int aem_system_create(const aem_system_desc *desc, aem_system **out) 
     s->len = (float)len;
     std::vector<double> wmu(h.omega);
     for (double &w : wmu) w *= kMu0 * len * len;
-    std::vector<double> Tb(h.T);  // T, then for every gate F max_f |T| (a bound on its sums, with a margin)
+    // T by frequency, then for every gate F max_f |T| (a bound on its sums, with a margin)
+    std::vector<double> Tb((size_t)h.G * (h.F + 1));
     for (int g = 0; g < h.G; ++g) {
         double top = 0;
-        for (int f = 0; f < h.F; ++f) top = std::max(top, std::fabs(h.T[(size_t)g * h.F + f]));
-        Tb.push_back(1.001 * h.F * top);
+        for (int f = 0; f < h.F; ++f) {
+            const double t = h.T[(size_t)g * h.F + f];
+            Tb[(size_t)f * h.G + g] = t;
+            top = std::max(top, std::fabs(t));
+        }
+        Tb[(size_t)h.F * h.G + g] = 1.001 * h.F * top;
     }
     const std::vector<double> &tab64 = f64_tables();
     if ((rc = upload(&s->d_omega_f, h.omega)) || (rc = upload(&s->d_lam_f, h.lam)) || (rc = upload(&s->d_hw_f, h.hw)) ||
