@@ -124,8 +124,9 @@ typedef struct {
 /* Forward model (Section 2): gates [device, P*G] row-major by model, and
  * optionally Im Hz_s at the frequency nodes (imh [device, P*F], may be NULL;
  * gates may be NULL if only imh is wanted).  The f32 entry computes the
- * layer recursion, Hankel sum and gate transform in FP32; the f64 entry is
- * the plain double-precision form of the same arithmetic.  Asynchronous.  The
+ * layer recursion and Hankel sum in FP32 and the gate transform in float
+ * pairs, rounded at the end; the f64 entry is the plain double-precision form
+ * of the same arithmetic.  Asynchronous.  The
  * f32 entry, and every call that evaluates the FP32 forward model, records
  * AEM_ERR_TIMEOUT in the system's status word (aem_system_status) should a
  * CTA's bounded wait for its next model give up; it then waits once more and
